@@ -948,6 +948,10 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_vol_min_blocks<real, n, SW, SP
 #undef FLEXI_LIFT_VOL_PARAMS
 #undef FLEXI_LIFT_VOL_ARGS
 
+}  // namespace flexi
+#include "k_lift_fx.cuh"
+namespace flexi {
+
 // a2-a4, a6, a7 for small FP64 meshes (fewer elements than SMs, n <= 4; standard form,
 // BR1): one element per CTA, spread over three thread groups of n^3 threads.  The lifting
 // computes one gradient component per group, the physical fluxes one direction per group,
@@ -2020,6 +2024,23 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
   return cudaGetLastError();
 }
 
+// fixed-point lifting + volume kernel (FP64, standard form, BR1)
+template <int n, bool LGL>
+static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double>& ops, const Phys<double>& ph,
+                             int store_grad, cudaStream_t st) {
+  using C = Cfg<n>;
+  constexpr size_t smem = lift_fx_smem<n>() > lift_vol_smem<double, n, 0>() ? lift_fx_smem<n>() : lift_vol_smem<double, n, 0>();
+  auto* kernel = &k_lift_vol_fx<n, LGL>;
+  static std::atomic<unsigned long long> attr{0};
+  cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
+  if (err != cudaSuccess) return err;
+  kernel<<<(m.K + C::NE - 1) / C::NE, C::T, smem, st>>>(
+      U, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf, (const double*)m.fgeo, m.elemSide,
+      (double*)m.Gf, (double*)m.Utv, store_grad ? (double*)m.Gvol : nullptr, m.K, m.S, m.Sface, (const double*)m.QB, ops,
+      m.fx, ph);
+  return cudaGetLastError();
+}
+
 template <typename real>
 cudaError_t launch_lift_vol(const DevMesh& m, const real* U, const Ops<real>& ops, const Phys<real>& ph,
                             int store_grad, cudaStream_t st) {
@@ -2058,6 +2079,14 @@ cudaError_t launch_lift_vol(const DevMesh& m, const real* U, const Ops<real>& op
       }
 #undef FLEXI_G3
       return cudaGetLastError();
+    }
+  }
+  if constexpr (sizeof(real) == 8) {
+    if (!m.br2 && m.split == 0 && m.fx.ok) {
+      if (m.lgl) {
+        FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, true>(m, U, ops, ph, store_grad, st));
+      }
+      FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, false>(m, U, ops, ph, store_grad, st));
     }
   }
   if (m.br2) {

@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "dg_common.cuh"
+#include "fx.cuh"
 
 namespace flexi {
 
@@ -52,6 +53,7 @@ struct DevMesh {
   const int* mvirt = nullptr;  // [nV] int4 (big side, type | a<<2 | b<<3, o, oinv)
   const int* mbig = nullptr;   // [nBig][8] (type, virtual side of position 0..3 or -1)
   void* QB = nullptr;          // [nBig][15][n^2] BR1 lifting flux of the big element
+  FxOps fx{};                  // fixed-point line operators (FP64 form)
   unsigned* status = nullptr;  // device status word (bit 0: non-physical face state)
 };
 

@@ -1,0 +1,85 @@
+"""Fixed-point line contractions of the FP64 form against the FP64 body of the same kernel.
+
+Scaling the units by powers of two (velocity by 2^b, pressure by 2^2b, viscosity by 2^b)
+scales every FP64 operation of the right-hand side exactly, so U_t of the scaled state is
+the scaled U_t.  At b = 120 the pressure leaves the fixed-point range and the element goes
+through the FP64 body; unscaled it goes through the fixed-point contractions.
+
+Tolerance, derived: both evaluations round each term of the sums of Eq. semiDiscrete.  A
+line's n + 2 terms in each of 3 directions, through the lifting and the volume sweep, give
+at most 2 * 3 (n + 2) roundings of 2^-53 relative to |terms|, bounded by
+T_v = max|F_v| * rowsum(|Dhat| + |lhat|) * max|Ja| / min J per variable, with the same again
+for the products and the pointwise fluxes.
+"""
+import numpy as np
+import pytest
+
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _rhs(mesh, N, nodes, U, b, poke=None):
+    import torch
+
+    from paper_1910_02858_gb300 import Solver, SolverConfig
+    from paper_1910_02858_gb300 import flexi as F
+
+    f = 2.0 ** b
+    s = Solver(SolverConfig(N=N, Ngeo=mesh.Ngeo, node_type=nodes, riemann=F.RIEMANN_RUSANOV, mu=0.01 * f), mesh.coords, mesh.conn)
+    scale = np.array([1.0, f, f, f, f * f]).reshape(1, 5, 1, 1, 1)
+    V = U * scale
+    if poke is not None:
+        V[poke[:-1]] = poke[-1]
+    Ut = s.rhs(torch.tensor(V, device="cuda:0"), 0.0).cpu().numpy()
+    s.close()
+    return Ut / (scale * f)
+
+
+def _case(N, nodes, mapping):
+    from oracle.basis import Basis
+
+    mesh = wl.box_mesh((3, 2, 4), lo=(0.0,) * 3, hi=(2 * np.pi,) * 3, Ngeo=N if mapping == "sine" else 1, mapping=mapping,
+                       reorient_seed=N)
+    U = wl.perturbed(mesh.node_coords(N, nodes), seed=N)
+    b = Basis(N, nodes)
+    D = b.Dhat.abs().sum(1) + b.lhat_minus.abs() + b.lhat_plus.abs()
+    h = 2 * np.pi / np.array([3, 2, 4]) / 2
+    ja = 1.4 * max(h[0] * h[1], h[1] * h[2], h[0] * h[2])
+    J = 0.3 * h.prod()
+    p = np.abs(U[:, 4]).max()
+    F = np.array([1.0, 2.0 * p, 2.0 * p, 2.0 * p, 2.0 * p])  # largest flux of each variable, generously
+    T = F * float(D.max()) * ja / J
+    return mesh, U, 4 * 2 * 3 * (N + 3) * 2.0 ** -53 * T
+
+
+@pytest.mark.parametrize("mapping", ["cartesian", "sine"])
+@pytest.mark.parametrize("nodes", [0, 1])
+@pytest.mark.parametrize("N", [1, 2, 3, 4, 5, 6, 7])
+def test_matches_fp64_body(N, nodes, mapping):
+    if mapping == "sine" and N == 1:
+        pytest.skip("the map is the identity at degree 1")
+    mesh, U, tol = _case(N, nodes, mapping)
+    a, c = _rhs(mesh, N, nodes, U, 0), _rhs(mesh, N, nodes, U, 120)
+    for v in range(5):
+        assert np.abs(a[:, v] - c[:, v]).max() <= tol[v], v
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("N", [2, 5, 7])
+def test_non_finite_values_spread_alike(N, bad):
+    mesh, U, _ = _case(N, 0, "cartesian")
+    poke = (5, 2, N, 1, 0, bad)
+    a, c = _rhs(mesh, N, 0, U, 0, poke), _rhs(mesh, N, 0, U, 120, poke)
+    assert not np.isfinite(a).all()
+    assert np.array_equal(np.isfinite(a), np.isfinite(c))
+
+
+def test_wide_ranges_within_an_element():
+    """A field that falls by 2^40 across each element: the error stays that of FP64 relative to the largest terms."""
+    mesh, U, tol = _case(7, 0, "cartesian")
+    ramp = 2.0 ** (-40.0 * np.linspace(0.0, 1.0, 8)).reshape(1, 1, 1, 8)
+    U[:, 1:4] *= ramp[:, None]
+    a, c = _rhs(mesh, 7, 0, U, 0), _rhs(mesh, 7, 0, U, 120)
+    for v in range(5):
+        assert np.abs(a[:, v] - c[:, v]).max() <= tol[v], v
