@@ -27,20 +27,14 @@ constexpr int FXH = MAXN / 2;
 // q_d = q(+1) - q(-1),
 //   y_i = E_i + O_i, y_{N-i} = O_i - E_i,
 //   E_i = sum_a DE_ia e_a + t_i q_d,  O_i = sum_a DO_ia o_a + s_i q_s,
-// which halves the multiply-adds.  An entry c is stored as round(c 2^(60 - cE)) =
-// h 2^30 + l with |l| <= 2^29; m* hold the rounding constant of the middle sum and the
-// mean of the omitted low-by-low products.
+// which halves the multiply-adds.  An entry c is stored as round(c 2^kc) = h 2^32 + l,
+// |l| <= 2^31, with kc the largest for which every row's sum of magnitudes stays below 2^62.
 struct FxOps {
   int eh[FXH][FXH], el[FXH][FXH];  // DE[i][a], i < n/2, a < (n+1)/2
   int oh[FXH][FXH], ol[FXH][FXH];  // DO[i][a], i < (n+1)/2, a < n/2
   int sh[FXH], sl[FXH], th[FXH], tl[FXH];
-  int peh[FXH], pel[FXH], poh[FXH], pol[FXH];  // prolongation: l(+-1), 58 bits under 2^pE
-  long long meq[FXH], moq[FXH];  // middle sums of E and O with face terms
-  long long me[FXH], mo[FXH];    // and without
-  long long mpe, mpo;
-  int cE, pE;
-  int rsh;  // the lifting's three-direction sums shifted right by rsh stay below 2^60
-  int ok;   // 0: the operators do not fit the format (not reached for n <= 8)
+  int peh[FXH], pel[FXH], poh[FXH], pol[FXH];  // prolongation to the line's ends, scale 2^kp
+  int kc, kp;
 };
 
 // host construction from the FP64 operators (integer rounding of scaled doubles: the
@@ -49,69 +43,51 @@ inline FxOps make_fx_ops(const Ops<double>& o, int n) {
   FxOps f;
   std::memset(&f, 0, sizeof(f));
   const int N = n - 1, h = n / 2, c = (n + 1) / 2;
-  double big = 0, row = 0, pbig = 0;
+  double row = 0, prow = 0, pe = 0, po = 0;
   for (int i = 0; i < n; ++i) {
-    double s = std::fabs(o.lhm[i]) + std::fabs(o.lhp[i]);
-    big = std::fmax(big, std::fmax(std::fabs(o.lhm[i]), std::fabs(o.lhp[i])));
-    pbig = std::fmax(pbig, std::fabs(o.lp[i]));
-    for (int a = 0; a < n; ++a) {
-      s += std::fabs(o.DhatT[a * n + i]);
-      big = std::fmax(big, std::fabs(o.DhatT[a * n + i]));
+    double e = 0.5 * std::fabs(o.lhp[i] - o.lhm[i]), d = 0.5 * std::fabs(o.lhp[i] + o.lhm[i]);
+    for (int a = 0; a < c; ++a) {
+      const double x = o.DhatT[a * n + i], y = 2 * a == N ? x : o.DhatT[(N - a) * n + i];
+      e += 0.5 * std::fabs(x + y);
+      d += 0.5 * std::fabs(x - y);
     }
-    row = std::fmax(row, s);
+    row = std::fmax(row, std::fmax(e, d));
   }
-  std::frexp(big, &f.cE);
-  std::frexp(pbig, &f.pE);
-  int re;
-  std::frexp(3.0 * row, &re);
-  const int bits = 57 + re - f.cE;  // |sum over three directions| < 2^bits
-  f.rsh = bits > 60 ? bits - 60 : 0;
-  f.ok = bits <= 62 ? 1 : 0;
+  for (int a = 0; a < c; ++a) {
+    pe += 2 * a == N ? std::fabs(o.lp[a]) : 0.5 * std::fabs(o.lp[a] + o.lm[a]);
+    po += 0.5 * std::fabs(o.lp[a] - o.lm[a]);
+  }
+  prow = std::fmax(pe, po);
+  int x;
+  std::frexp(row * (1 + 1e-12), &x);
+  f.kc = 62 - x;
+  std::frexp(prow * (1 + 1e-12), &x);
+  f.kp = 62 - x;
   auto split = [](long long v, int& hi, int& lo) {
-    const long long q = (v + (1ll << 29)) >> 30;
-    hi = (int)q;
-    lo = (int)(v - q * (1ll << 30));
+    lo = (int)(unsigned)(v & 0xffffffffll);
+    hi = (int)((v - lo) / (1ll << 32));
   };
-  // the operators' symmetric means: A = 2^(59 - cE) times the entry
+  // the operators' symmetric means: A = 2^(kc - 1) times twice the entry, halved below
   auto A = [&](int i, int a) {
-    return std::llrint(std::ldexp(o.DhatT[a * n + i], 58 - f.cE)) -
-           std::llrint(std::ldexp(o.DhatT[(N - a) * n + N - i], 58 - f.cE));
+    return std::llrint(std::ldexp(o.DhatT[a * n + i], f.kc - 2)) -
+           std::llrint(std::ldexp(o.DhatT[(N - a) * n + N - i], f.kc - 2));
   };
   auto Q = [&](int i) {
-    return std::llrint(std::ldexp(o.lhp[i], 58 - f.cE)) + std::llrint(std::ldexp(o.lhm[N - i], 58 - f.cE));
+    return std::llrint(std::ldexp(o.lhp[i], f.kc - 2)) + std::llrint(std::ldexp(o.lhm[N - i], f.kc - 2));
+  };
+  auto L = [&](int a) {
+    return std::llrint(std::ldexp(o.lp[a], f.kp - 2)) + std::llrint(std::ldexp(o.lm[N - a], f.kp - 2));
   };
   for (int i = 0; i < h; ++i) {
-    long long m = 0;
-    for (int a = 0; a < c; ++a) {
-      split(2 * a == N ? 2 * A(i, a) : A(i, a) + A(i, N - a), f.eh[i][a], f.el[i][a]);
-      m += f.el[i][a];
-    }
+    for (int a = 0; a < c; ++a) split(2 * a == N ? 2 * A(i, a) : A(i, a) + A(i, N - a), f.eh[i][a], f.el[i][a]);
     split(Q(i) - Q(N - i), f.th[i], f.tl[i]);
-    f.me[i] = (1ll << 29) + m / 2;
-    f.meq[i] = f.me[i] + f.tl[i] / 2;
   }
   for (int i = 0; i < c; ++i) {
-    long long m = 0;
-    for (int a = 0; a < h; ++a) {
-      split(A(i, a) - A(i, N - a), f.oh[i][a], f.ol[i][a]);
-      m += f.ol[i][a];
-    }
+    for (int a = 0; a < h; ++a) split(A(i, a) - A(i, N - a), f.oh[i][a], f.ol[i][a]);
     split(Q(i) + Q(N - i), f.sh[i], f.sl[i]);
-    f.mo[i] = (1ll << 29) + m / 2;
-    f.moq[i] = f.mo[i] + f.sl[i] / 2;
   }
-  f.mpe = f.mpo = 1ll << 29;
-  auto L = [&](int a) {  // 2^(57 - pE) l_a(+1), mean with its mirror image
-    return std::llrint(std::ldexp(o.lp[a], 56 - f.pE)) + std::llrint(std::ldexp(o.lm[N - a], 56 - f.pE));
-  };
-  for (int a = 0; a < c; ++a) {
-    split(2 * a == N ? 2 * L(a) : L(a) + L(N - a), f.peh[a], f.pel[a]);
-    f.mpe += f.pel[a] / 2;
-  }
-  for (int a = 0; a < h; ++a) {
-    split(L(a) - L(N - a), f.poh[a], f.pol[a]);
-    f.mpo += f.pol[a] / 2;
-  }
+  for (int a = 0; a < c; ++a) split(2 * a == N ? 2 * L(a) : L(a) + L(N - a), f.peh[a], f.pel[a]);
+  for (int a = 0; a < h; ++a) split(L(a) - L(N - a), f.poh[a], f.pol[a]);
   return f;
 }
 
@@ -120,15 +96,24 @@ inline FxOps make_fx_ops(const Ops<double>& o, int n) {
 // ---------------------------------------------------------------------------
 using fx64 = long long;
 
+// c + a b with 32-bit signed a, b (IMAD.WIDE; written out because the compiler otherwise
+// sign-extends operands from the constant bank and multiplies 64 x 64 bits)
+__device__ __forceinline__ fx64 fx_mad(int a, int b, fx64 c) {
+  fx64 r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
+
 // magnitude word: ordered like |x|, its exponent field is x's (NaN and infinities 2047)
 __device__ __forceinline__ int fx_mag(double x) { return __double2hiint(x) & 0x7fffffff; }
 
-// x 2^(60 - (E - 1022)) for |x| < 2^(E - 1022), E a biased exponent field; truncated
+// x 2^(B - (E - 1022)) for |x| < 2^(E - 1022), E a biased exponent field, B >= 53; truncated
+template <int B>
 __device__ __forceinline__ fx64 fx_from(double x, int E) {
   const int hi = __double2hiint(x);
   const int ex = (hi >> 20) & 0x7ff;
   const unsigned mh = (unsigned)(hi & 0xfffff) | 0x100000u;
-  unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(x)) << 7;
+  unsigned long long m = (((unsigned long long)mh << 32) | (unsigned)__double2loint(x)) << (B - 53);
   m = ex == 0 ? 0 : m >> min(E - ex, 63);  // subnormal values count as zero
   const long long s = (long long)(hi >> 31);
   return ((fx64)m ^ s) - s;
@@ -139,40 +124,59 @@ __device__ __forceinline__ double fx_to(fx64 r, int t) {
   const long long s = r >> 63;
   const unsigned long long a = (unsigned long long)((r ^ s) - s);
   const unsigned ahi = (unsigned)(a >> 32), alo = (unsigned)a;
-  const int lz = __clz(ahi ? ahi : alo) + (ahi ? 0 : 32);  // >= 1 for a != 0
+  const int lz = __clz(ahi ? ahi : alo) + (ahi ? 0 : 32);  // >= 1; 64 for zero
   const unsigned long long m = ((a << (lz - 1)) + 0x200) >> 10;
   const int e = 1086 + t - lz;
   const unsigned long long b = ((unsigned long long)(unsigned)(e - 1) << 52) + m;
-  return __longlong_as_double((a == 0 || e < 1) ? 0ll : (long long)(b | (unsigned long long)(s & (1ll << 63))));
+  return __longlong_as_double((lz == 64 || e < 1) ? 0ll : (long long)(b | ((unsigned long long)s << 63)));
 }
 
-// a value split into 30-bit halves, v = h 2^30 + l, 0 <= l < 2^30 (|v| < 2^61)
+// a value as v = h 2^32 + l with the low half signed, |l| <= 2^31 (|v| < 2^62)
 struct FxSplit {
   int h, l;
 };
-__device__ __forceinline__ FxSplit fx_split(fx64 v) { return {(int)(v >> 30), (int)v & 0x3fffffff}; }
+__device__ __forceinline__ FxSplit fx_split(fx64 v) {
+  return {(int)(v >> 32) + (int)((unsigned)v >> 31), (int)(unsigned)v};
+}
 
-// a b / 2^60 (the mean of the omitted low-by-low product is in the rounding constant)
+// Sum of products / 2^64: the high products and the two kinds of cross products are
+// accumulated apart (the low products lie below the result's last bit, and signed low
+// halves have mean zero).  The cross sum carries an offset of 2^63, so that its high word
+// joins the high sum without a sign extension, and half a unit of the result.
+struct FxAcc {
+  fx64 hh = -(1ll << 31), mid = (fx64)0x8000000080000000ull;
+  __device__ __forceinline__ void add(FxSplit a, FxSplit b) { add(a, b.h, b.l); }
+  __device__ __forceinline__ void add(FxSplit a, int h, int l) {
+    hh = fx_mad(a.h, h, hh);
+    mid = fx_mad(a.h, l, mid);
+    mid = fx_mad(a.l, h, mid);
+  }
+  __device__ __forceinline__ fx64 get() const { return hh + (fx64)((unsigned long long)mid >> 32); }
+};
+
 __device__ __forceinline__ fx64 fx_mul(FxSplit a, FxSplit b) {
-  const fx64 mid = (fx64)a.h * b.l + ((fx64)a.l * b.h + ((1ll << 29) + (1ll << 28)));
-  return (fx64)a.h * b.h + (mid >> 30);
+  FxAcc s;
+  s.add(a, b);
+  return s.get();
 }
 
 // rounded right shift, sh >= 1
 __device__ __forceinline__ fx64 fx_shr(fx64 v, int sh) { return (v + (1ll << (sh - 1))) >> sh; }
 
-// One line of a D_hat contraction: x[0..n) -> y(i, value) for every output node i; FACE: plus
-// the face terms l_hat_i(-1) qm + l_hat_i(+1) qp (Gauss-Lobatto: only at the line's ends)
-template <int n, bool LGL, bool FACE, typename Put>
-__device__ __forceinline__ void fx_line(const fx64 (&x)[n], fx64 qm, fx64 qp, const FxOps& o, Put put) {
+// One line of a D_hat contraction in place: x[0], x[stride], ... (|x| < 2^59.6) become the
+// contraction (< 2^58.6); FACE: plus the face terms l_hat_i(-1) qm + l_hat_i(+1) qp
+// (Gauss-Lobatto: only at the line's ends)
+template <int n, bool LGL, bool FACE>
+__device__ __forceinline__ void fx_line(fx64* __restrict__ p, int stride, fx64 qm, fx64 qp, const FxOps& o) {
   constexpr int h = n / 2, c = (n + 1) / 2, N = n - 1;
   FxSplit e[c], d[h];
 #pragma unroll
   for (int a = 0; a < h; ++a) {
-    e[a] = fx_split(x[a] + x[N - a]);
-    d[a] = fx_split(x[a] - x[N - a]);
+    const fx64 x = p[a * stride], y = p[(N - a) * stride];
+    e[a] = fx_split(x + y);
+    d[a] = fx_split(x - y);
   }
-  if constexpr (n & 1) e[c - 1] = fx_split(x[c - 1]);
+  if constexpr (n & 1) e[c - 1] = fx_split(p[(c - 1) * stride]);
   FxSplit qs{0, 0}, qd{0, 0};
   if constexpr (FACE) {
     qs = fx_split(qp + qm);
@@ -181,75 +185,64 @@ __device__ __forceinline__ void fx_line(const fx64 (&x)[n], fx64 qm, fx64 qp, co
 #pragma unroll
   for (int i = 0; i < c; ++i) {
     const bool face = FACE && (!LGL || i == 0);
-    fx64 hh = 0, mid = face ? o.moq[i] : o.mo[i];
+    FxAcc so;
 #pragma unroll
-    for (int a = 0; a < h; ++a) {
-      hh += (fx64)d[a].h * o.oh[i][a];
-      mid += (fx64)d[a].h * o.ol[i][a];
-      mid += (fx64)d[a].l * o.oh[i][a];
-    }
-    if (face) {
-      hh += (fx64)qs.h * o.sh[i];
-      mid += (fx64)qs.h * o.sl[i];
-      mid += (fx64)qs.l * o.sh[i];
-    }
-    const fx64 O = hh + (mid >> 30);
+    for (int a = 0; a < h; ++a) so.add(d[a], o.oh[i][a], o.ol[i][a]);
+    if (face) so.add(qs, o.sh[i], o.sl[i]);
+    const fx64 O = so.get();
     if (i < h) {
-      hh = 0;
-      mid = face ? o.meq[i] : o.me[i];
+      FxAcc se;
 #pragma unroll
-      for (int a = 0; a < c; ++a) {
-        hh += (fx64)e[a].h * o.eh[i][a];
-        mid += (fx64)e[a].h * o.el[i][a];
-        mid += (fx64)e[a].l * o.eh[i][a];
-      }
-      if (face) {
-        hh += (fx64)qd.h * o.th[i];
-        mid += (fx64)qd.h * o.tl[i];
-        mid += (fx64)qd.l * o.th[i];
-      }
-      const fx64 E = hh + (mid >> 30);
-      put(i, O + E);
-      put(N - i, O - E);
+      for (int a = 0; a < c; ++a) se.add(e[a], o.eh[i][a], o.el[i][a]);
+      if (face) se.add(qd, o.th[i], o.tl[i]);
+      const fx64 E = se.get();
+      p[i * stride] = O + E;
+      p[(N - i) * stride] = O - E;
     } else {
-      put(i, O);
+      p[i * stride] = O;
     }
   }
 }
 
 // both end values of a line, sum_a l_a(-1) x_a and sum_a l_a(+1) x_a
 template <int n>
-__device__ __forceinline__ void fx_ends(const fx64 (&x)[n], const FxOps& o, fx64& ym, fx64& yp) {
+__device__ __forceinline__ void fx_ends(const fx64* __restrict__ p, int stride, const FxOps& o, fx64& ym, fx64& yp) {
   constexpr int h = n / 2, c = (n + 1) / 2, N = n - 1;
-  fx64 he = 0, me = o.mpe, ho = 0, mo = o.mpo;
+  FxAcc e, d;
 #pragma unroll
   for (int a = 0; a < c; ++a) {
-    const FxSplit e = fx_split(2 * a == N ? x[a] : x[a] + x[N - a]);
-    he += (fx64)e.h * o.peh[a];
-    me += (fx64)e.h * o.pel[a];
-    me += (fx64)e.l * o.peh[a];
-    if (a < h) {
-      const FxSplit d = fx_split(x[a] - x[N - a]);
-      ho += (fx64)d.h * o.poh[a];
-      mo += (fx64)d.h * o.pol[a];
-      mo += (fx64)d.l * o.poh[a];
+    const fx64 x = p[a * stride];
+    if (2 * a == N) {
+      e.add(fx_split(x), o.peh[a], o.pel[a]);
+    } else {
+      const fx64 y = p[(N - a) * stride];
+      e.add(fx_split(x + y), o.peh[a], o.pel[a]);
+      if (a < h) d.add(fx_split(x - y), o.poh[a], o.pol[a]);
     }
   }
-  const fx64 e = he + (me >> 30), d = ho + (mo >> 30);
-  yp = e + d;
-  ym = e - d;
+  const fx64 E = e.get(), D = d.get();
+  yp = E + D;
+  ym = E - D;
 }
 
-// largest magnitude word over the threads of an element into a shared slot: one
-// reduction and one shared atomic per warp where a CTA holds one element (WARP; every
-// thread of mask calls it), else one atomic per thread
-template <bool WARP>
-__device__ __forceinline__ void fx_max(int* slot, int mag, unsigned mask) {
+// Largest magnitude words of n fields over the threads of an element: get(s) is the
+// thread's word for slot s.  One warp reduction per slot, lane s keeps the s-th, one shared
+// atomic per warp where a CTA holds one element (every thread of mask calls it, and every
+// warp has at least COUNT of them); else one atomic per thread and slot.
+template <bool WARP, int COUNT, typename Get>
+__device__ __forceinline__ void fx_max(int* slots, unsigned mask, Get get) {
   if constexpr (WARP) {
-    mag = __reduce_max_sync(mask, mag);
-    if ((threadIdx.x & 31) == 0) atomicMax(slot, mag);
+    const int lane = threadIdx.x & 31;
+    int mine = 0;
+#pragma unroll
+    for (int s = 0; s < COUNT; ++s) {
+      const int r = __reduce_max_sync(mask, get(s));
+      mine = lane == s ? r : mine;
+    }
+    if (lane < COUNT) atomicMax(slots + lane, mine);
   } else {
-    atomicMax(slot, mag);
+#pragma unroll
+    for (int s = 0; s < COUNT; ++s) atomicMax(slots + s, get(s));
   }
 }
 

@@ -2029,7 +2029,7 @@ template <int n, bool LGL>
 static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double>& ops, const Phys<double>& ph,
                              int store_grad, cudaStream_t st) {
   using C = Cfg<n>;
-  constexpr size_t smem = lift_fx_smem<n>() > lift_vol_smem<double, n, 0>() ? lift_fx_smem<n>() : lift_vol_smem<double, n, 0>();
+  constexpr size_t smem = lift_fx_smem<n>();
   auto* kernel = &k_lift_vol_fx<n, LGL>;
   static std::atomic<unsigned long long> attr{0};
   cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
@@ -2082,7 +2082,7 @@ cudaError_t launch_lift_vol(const DevMesh& m, const real* U, const Ops<real>& op
     }
   }
   if constexpr (sizeof(real) == 8) {
-    if (!m.br2 && m.split == 0 && m.fx.ok) {
+    if (!m.br2 && m.split == 0) {
       if (m.lgl) {
         FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, true>(m, U, ops, ph, store_grad, st));
       }
