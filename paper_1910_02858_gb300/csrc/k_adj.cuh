@@ -4,9 +4,9 @@
 // periodic meshes, meshes with boundary sides and (BR1) mortar meshes: the
 // interpolation of the big side's state and gradients and the projections of the
 // lifting and numerical fluxes are linear and are transposed in place
-// (k_adj_mortar_interp, k_adj_mortar_project).  Numerical flux: the Roe fluxes have a hand-written
-// reverse; HLLC, Rusanov and the entropy-conservative flux are differentiated in
-// forward mode (dual numbers, ten tangents per face node).
+// (k_adj_mortar_interp, k_adj_mortar_project).  Numerical flux: Roe, HLLC and Rusanov have
+// hand-written reverses; the entropy-conservative flux is differentiated in forward mode
+// (dual numbers, ten tangents per face node).
 // Boundary sides: the outer state is a function of the inner one (outflow: the
 // same state; slip wall: normal velocity reversed, a reflection; exact state:
 // independent of U) and the outer gradient is the inner one, so their adjoints
@@ -282,8 +282,228 @@ __device__ __forceinline__ void roe_vjp(const real WL[NV], const real WR[NV], co
   side(WR, ER, unR, HR, irR, isR, lHR, lsR, lWR);
 }
 
+// Euler normal flux reverse with u = v . n and the energy E as variables of their own:
+// lamf -> adjoints of W (velocity and pressure parts of f), of E and of u
+template <typename real>
+__device__ __forceinline__ void euler_normal_vjp(const real W[NV], real E, real u, const real n[3], const real lf[NV],
+                                                 real lW[NV], real& lE, real& lu) {
+  const real lv = lf[1] * W[1] + lf[2] * W[2] + lf[3] * W[3];
+  const real a = lf[0] + lv;
+  lW[0] = u * a;
+  lu = dg_fma(W[0], a, lf[4] * (E + W[4]));
+  const real m = W[0] * u;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) lW[1 + c] = lf[1 + c] * m;
+  lW[4] = dg_fma(lf[4], u, lf[1] * n[0] + lf[2] * n[1] + lf[3] * n[2]);
+  lE = lf[4] * u;
+}
+
+// adjoints of E = p / (gamma - 1) + rho |v|^2 / 2 and u = v . n carried to W
+template <typename real>
+__device__ __forceinline__ void energy_normal_vjp(const real W[NV], real q2, const real n[3], const Phys<real>& ph, real lE,
+                                                  real lu, real lW[NV]) {
+  lW[0] = dg_fma(real(0.5) * lE, q2, lW[0]);
+  const real a = lE * W[0];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) lW[1 + c] = dg_fma(a, W[1 + c], dg_fma(lu, n[c], lW[1 + c]));
+  lW[4] = dg_fma(lE, ph.inv_gm1, lW[4]);
+}
+
+// HLLC flux reverse (riemann_hllc): given lamf, accumulate lamWL, lamWR.  The wave speeds' min and
+// max and the star region follow the branch of the forward evaluation.  One forward and one
+// reverse pass (about 300 operations) in place of ten dual-number evaluations.
+template <typename real>
+__device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], const real n[3], const Phys<real>& ph,
+                                         const real lf[NV], real lWL[NV], real lWR[NV]) {
+  // ---- forward
+  const real irL = real(1) / WL[0], irR = real(1) / WR[0];
+  const real q2L = WL[1] * WL[1] + WL[2] * WL[2] + WL[3] * WL[3];
+  const real q2R = WR[1] * WR[1] + WR[2] * WR[2] + WR[3] * WR[3];
+  const real EL = WL[4] * ph.inv_gm1 + real(0.5) * WL[0] * q2L;
+  const real ER = WR[4] * ph.inv_gm1 + real(0.5) * WR[0] * q2R;
+  const real uL = WL[1] * n[0] + WL[2] * n[1] + WL[3] * n[2];
+  const real uR = WR[1] * n[0] + WR[2] * n[1] + WR[3] * n[2];
+  const real cL = dg_sqrt(ph.gamma * WL[4] * irL);
+  const real cR = dg_sqrt(ph.gamma * WR[4] * irR);
+  const real r = dg_sqrt(WR[0] * irL);
+  const real iw = real(1) / (real(1) + r);
+  const real HL = (EL + WL[4]) * irL, HR = (ER + WR[4]) * irR;
+  real vel[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) vel[c] = (WL[1 + c] + r * WR[1 + c]) * iw;
+  const real H = (HL + r * HR) * iw;
+  const real c = dg_sqrt(ph.gm1 * (H - real(0.5) * (vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2])));
+  const real un = vel[0] * n[0] + vel[1] * n[1] + vel[2] * n[2];
+  const bool ownL = uL - cL < un - c, ownR = uR + cR > un + c;
+  const real SL = ownL ? uL - cL : un - c;
+  const real SR = ownR ? uR + cR : un + c;
+  real lK[NV], lEK, luK;  // adjoints of the upwind state, its energy and normal velocity
+  if (SL >= real(0) || SR <= real(0)) {  // supersonic: the flux of one side
+    const bool left = SL >= real(0);
+    real W[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) W[v] = left ? WL[v] : WR[v];
+    euler_normal_vjp(W, left ? EL : ER, left ? uL : uR, n, lf, lK, lEK, luK);
+    energy_normal_vjp(W, left ? q2L : q2R, n, ph, lEK, luK, lK);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      lWL[v] += left ? lK[v] : real(0);
+      lWR[v] += left ? real(0) : lK[v];
+    }
+    return;
+  }
+  const real mL = WL[0] * (SL - uL), mR = WR[0] * (SR - uR);
+  const real iD = real(1) / (mL - mR);
+  const real Ss = (WR[4] - WL[4] + mL * uL - mR * uR) * iD;
+  const bool left = Ss >= real(0);
+  real W[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) W[v] = left ? WL[v] : WR[v];
+  const real E = left ? EL : ER, u = left ? uL : uR, S = left ? SL : SR, m = left ? mL : mR;
+  const real irK = left ? irL : irR, q2 = left ? q2L : q2R;
+  // ---- reverse of f = F(W) + S (U* - U): U* = fac (1, v + (Ss - u) n, B),
+  // fac = m / (S - Ss), B = E / rho + (Ss - u)(Ss + p / m)
+  const real dS = S - Ss, du = Ss - u;
+  const real q = real(1) / (m * dS);
+  const real fac = m * m * q, pm = W[4] * dS * q;  // p / m
+  const real B = dg_fma(E, irK, du * (Ss + pm));
+  euler_normal_vjp(W, E, u, n, lf, lK, lEK, luK);
+  const real ln = lf[1] * n[0] + lf[2] * n[1] + lf[3] * n[2];
+  const real lv = lf[1] * W[1] + lf[2] * W[2] + lf[3] * W[3];
+  const real Sf = S * fac, Sf4 = Sf * lf[4];
+  const real star = lf[0] + lv + du * ln + lf[4] * B;  // lamf . U* / fac
+  const real a = lf[0] + lv;
+  lK[0] = dg_fma(-S, a, lK[0]);
+  lK[0] = dg_fma(-Sf4 * irK, E * irK, lK[0]);
+  const real b = Sf - S * W[0];
+#pragma unroll
+  for (int c2 = 0; c2 < 3; ++c2) lK[1 + c2] = dg_fma(lf[1 + c2], b, lK[1 + c2]);
+  const real im = dS * q;  // 1 / m
+  lK[4] = dg_fma(Sf4 * du, im, lK[4]);
+  lEK += dg_fma(Sf4, irK, -S * lf[4]);
+  luK -= dg_fma(Sf4, Ss + pm, Sf * ln);
+  real lS = dg_fma(fac, star, -(W[0] * a + lf[4] * E));
+  real lSs = dg_fma(Sf, ln, Sf4 * (Ss + pm + du));
+  real lm = -Sf4 * du * pm * im;
+  const real lfac = S * star, idS = m * q;  // 1 / (S - Ss)
+  lm = dg_fma(lfac, idS, lm);
+  lS = dg_fma(-lfac * fac, idS, lS);
+  lSs = dg_fma(lfac * fac, idS, lSs);
+  // ---- reverse of Ss and of m_K = rho_K (S_K - u_K)
+  const real lN = lSs * iD, lD = -lN * Ss;
+  const real lmL = (left ? lm : real(0)) + dg_fma(lN, uL, lD);
+  const real lmR = (left ? real(0) : lm) - dg_fma(lN, uR, lD);
+  real lSL = dg_fma(lmL, WL[0], left ? lS : real(0)), lSR = dg_fma(lmR, WR[0], left ? real(0) : lS);
+  real luL = dg_fma(lN, mL, (left ? luK : real(0)) - lmL * WL[0]);
+  real luR = dg_fma(-lN, mR, (left ? real(0) : luK) - lmR * WR[0]);
+  real aL[NV], aR[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    aL[v] = left ? lK[v] : real(0);
+    aR[v] = left ? real(0) : lK[v];
+  }
+  aL[0] = dg_fma(lmL, SL - uL, aL[0]);
+  aR[0] = dg_fma(lmR, SR - uR, aR[0]);
+  aL[4] -= lN;
+  aR[4] += lN;
+  real lEL = left ? lEK : real(0), lER = left ? real(0) : lEK;
+  // ---- reverse of the wave speeds
+  luL += ownL ? lSL : real(0);
+  luR += ownR ? lSR : real(0);
+  const real lcL = ownL ? -lSL : real(0), lcR = ownR ? lSR : real(0);
+  const real lun = (ownL ? real(0) : lSL) + (ownR ? real(0) : lSR);
+  const real lc = (ownR ? real(0) : lSR) - (ownL ? real(0) : lSL);
+  if (!ownL || !ownR) {  // Roe averages
+    const real lH = lc * real(0.5) * ph.gm1 / c;
+    real lvel[3], dot = lH * (HR - H);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      lvel[k] = dg_fma(-lH, vel[k], lun * n[k]);
+      dot = dg_fma(lvel[k], WR[1 + k] - vel[k], dot);
+    }
+    const real wR = r * iw, lr = dot * iw;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      aL[1 + k] = dg_fma(lvel[k], iw, aL[1 + k]);
+      aR[1 + k] = dg_fma(lvel[k], wR, aR[1 + k]);
+    }
+    const real hr = real(0.5) * lr * r;
+    const real hL = lH * iw * irL, hR = lH * wR * irR;
+    aL[0] -= dg_fma(hL, HL, hr * irL);
+    aR[0] += dg_fma(-hR, HR, hr * irR);
+    aL[4] += hL;
+    aR[4] += hR;
+    lEL += hL;
+    lER += hR;
+  }
+  if (ownL) {  // c_L = sqrt(gamma p / rho)
+    const real x = real(0.5) * lcL * cL;
+    aL[0] = dg_fma(-x, irL, aL[0]);
+    aL[4] += x / WL[4];
+  }
+  if (ownR) {
+    const real x = real(0.5) * lcR * cR;
+    aR[0] = dg_fma(-x, irR, aR[0]);
+    aR[4] += x / WR[4];
+  }
+  energy_normal_vjp(WL, q2L, n, ph, lEL, luL, aL);
+  energy_normal_vjp(WR, q2R, n, ph, lER, luR, aR);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    lWL[v] += aL[v];
+    lWR[v] += aR[v];
+  }
+}
+
+// Rusanov flux reverse: given lamf, accumulate lamWL, lamWR
+template <typename real>
+__device__ __forceinline__ void rusanov_vjp(const real WL[NV], const real WR[NV], const real n[3], const Phys<real>& ph,
+                                            const real lf[NV], real lWL[NV], real lWR[NV]) {
+  const real uL = WL[1] * n[0] + WL[2] * n[1] + WL[3] * n[2];
+  const real uR = WR[1] * n[0] + WR[2] * n[1] + WR[3] * n[2];
+  const real cL = dg_sqrt(ph.gamma * WL[4] / WL[0]), cR = dg_sqrt(ph.gamma * WR[4] / WR[0]);
+  const real sL = dg_abs(uL) + cL, sR = dg_abs(uR) + cR;
+  const bool selL = sL > sR;  // as the forward maximum selects
+  const real lam = selL ? sL : sR;
+  real jump = real(0);  // lamf . (U_R - U_L)
+  const real half = real(0.5);
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const real* W = side ? WR : WL;
+    const real u = side ? uR : uL, sg = side ? -half * lam : half * lam;  // dU weight: +-lambda / 2
+    const real q2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
+    const real E = W[4] * ph.inv_gm1 + half * W[0] * q2;
+    real hf[NV], a[NV], lE, lu;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) hf[v] = half * lf[v];
+    euler_normal_vjp(W, E, u, n, hf, a, lE, lu);
+    const real lv = lf[1] * W[1] + lf[2] * W[2] + lf[3] * W[3];
+    const real s = dg_fma(W[0], lf[0] + lv, lf[4] * E);
+    jump = side ? jump + s : jump - s;
+    a[0] = dg_fma(sg, lf[0] + lv, a[0]);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[1 + c] = dg_fma(sg * W[0], lf[1 + c], a[1 + c]);
+    lE = dg_fma(sg, lf[4], lE);
+    energy_normal_vjp(W, q2, n, ph, lE, lu, a);
+    real* l = side ? lWR : lWL;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) l[v] += a[v];
+  }
+  const real ll = -half * jump;  // adjoint of lambda
+  const real u = selL ? uL : uR, c = selL ? cL : cR;
+  const real g = u < real(0) ? -ll : ll;
+  const real rho = selL ? WL[0] : WR[0], p = selL ? WL[4] : WR[4];
+  const real x = half * ll * c;
+  real a[NV] = {-x / rho, g * n[0], g * n[1], g * n[2], x / p};
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    lWL[v] += selL ? a[v] : real(0);
+    lWR[v] += selL ? real(0) : a[v];
+  }
+}
+
 // ---------------------------------------------------------------------------
-// reverse of the other numerical fluxes by forward-mode differentiation
+// reverse of the entropy-conservative flux by forward-mode differentiation
 // ---------------------------------------------------------------------------
 // Dual number x + dx eps (eps^2 = 0): the templated flux functions of
 // dg_common.cuh evaluated on Dual<real> give their directional derivative.
@@ -533,9 +753,10 @@ __global__ void __launch_bounds__(Cfg<n>::T) k_adj_lamface(const real* __restric
   }
 }
 
-// DUAL: the flux reverse by dual numbers (HLLC, Rusanov, entropy-conservative);
-// otherwise the hand-written Roe reverse.
-template <typename real, int n, bool DUAL>
+// RS: the flux (FLEXI_RIEMANN_*; 0 both Roe fluxes); the entropy-conservative one by dual
+// numbers, the others by hand-written reverse.  HLLC by hand instead of dual numbers:
+// 504 curved elements, N = 6: 667 -> 90 us.
+template <typename real, int n, int RS>
 __global__ void __launch_bounds__(128) k_adj_face(const real* __restrict__ Wf, const real* __restrict__ Gf,
                                                   const real* __restrict__ fgeo, const real* __restrict__ LF,
                                                   real* __restrict__ LWf, real* __restrict__ LGf, int S, int nBC,
@@ -575,7 +796,11 @@ __global__ void __launch_bounds__(128) k_adj_face(const real* __restrict__ Wf, c
   real lGL[15], lGR[15];
 #pragma unroll
   for (int c = 0; c < 15; ++c) lGL[c] = lGR[c] = real(0);
-  if constexpr (DUAL)
+  if constexpr (RS == 1)
+    hllc_vjp(WL, WR, nv, ph, lf, lWL, lWR);
+  else if constexpr (RS == 3)
+    rusanov_vjp(WL, WR, nv, ph, lf, lWL, lWR);
+  else if constexpr (RS == 4)
     riemann_vjp_dual(WL, WR, nv, ph, lf, lWL, lWR);
   else
     roe_vjp(WL, WR, nv, ph, ph.riemann == 2, lf, lWL, lWR);
@@ -1263,6 +1488,11 @@ static cudaError_t rhs_adjoint_n(const DevMesh& m, const real* U, const real* la
   if ((err = launch_mortar_state<real>(m, mo, ph, st)) != cudaSuccess) return err;
   if (m.br2) {
     if ((err = lift_vol_n<real, n, 0, false, 0, true>(m, U, ops, ph, 1, st)) != cudaSuccess) return err;
+  } else if constexpr (sizeof(real) == 8) {
+    // the lifting without the volume integral
+    if ((err = m.lgl ? lift_fx_n<n, true>(m, U, ops, ph, 1, st, 0) : lift_fx_n<n, false>(m, U, ops, ph, 1, st, 0)) !=
+        cudaSuccess)
+      return err;
   } else {
     if ((err = lift_vol_n<real, n, 0>(m, U, ops, ph, 1, st)) != cudaSuccess) return err;
   }
@@ -1271,14 +1501,17 @@ static cudaError_t rhs_adjoint_n(const DevMesh& m, const real* U, const real* la
   if (m.nBig > 0)  // the big element's flux adjoint to slot 1 of its virtual sides
     k_adj_mortar_project<real, n, 1><<<m.nBig, kMortarThreads, 0, st>>>((const real*)a.LF, (real*)a.LF, nullptr,
                                                                        m.mbig, mv, m.S, m.Sface, m.vbase, mo);
-  if (ph.riemann == 0 || ph.riemann == 2)
-    k_adj_face<real, n, false><<<sgrid, 128, 0, st>>>((const real*)m.Wf, (const real*)m.Gf, (const real*)m.fgeo,
-                                                      (const real*)a.LF, (real*)a.LWf, (real*)a.LGf, m.S, m.nBC,
-                                                      m.Sface, ph);
-  else
-    k_adj_face<real, n, true><<<sgrid, 128, 0, st>>>((const real*)m.Wf, (const real*)m.Gf, (const real*)m.fgeo,
-                                                     (const real*)a.LF, (real*)a.LWf, (real*)a.LGf, m.S, m.nBC,
-                                                     m.Sface, ph);
+#define FLEXI_ADJ_FACE(RSV)                                                                                     \
+  k_adj_face<real, n, RSV><<<sgrid, 128, 0, st>>>((const real*)m.Wf, (const real*)m.Gf, (const real*)m.fgeo,     \
+                                                  (const real*)a.LF, (real*)a.LWf, (real*)a.LGf, m.S, m.nBC,    \
+                                                  m.Sface, ph)
+  switch (ph.riemann) {
+    case 1: FLEXI_ADJ_FACE(1); break;
+    case 3: FLEXI_ADJ_FACE(3); break;
+    case 4: FLEXI_ADJ_FACE(4); break;
+    default: FLEXI_ADJ_FACE(0); break;
+  }
+#undef FLEXI_ADJ_FACE
   if (m.nBig > 0)  // virtual sides' gradient adjoints (slot 1) to the big element's face gradient
     k_adj_mortar_interp<real, n, 15, false><<<m.nBig, kMortarThreads, 0, st>>>((real*)a.LGf, m.mbig, mv, m.S,
                                                                               m.Sface, m.vbase, mo);

@@ -2024,10 +2024,10 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
   return cudaGetLastError();
 }
 
-// fixed-point lifting + volume kernel (FP64, standard form, BR1)
+// fixed-point lifting + volume kernel (FP64, standard form, BR1); volume = 0: the lifting alone
 template <int n, bool LGL>
 static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double>& ops, const Phys<double>& ph,
-                             int store_grad, cudaStream_t st) {
+                             int store_grad, cudaStream_t st, int volume = 1) {
   using C = Cfg<n>;
   constexpr size_t smem = lift_fx_smem<n>();
   auto* kernel = &k_lift_vol_fx<n, LGL>;
@@ -2036,8 +2036,8 @@ static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double
   if (err != cudaSuccess) return err;
   kernel<<<(m.K + C::NE - 1) / C::NE, C::T, smem, st>>>(
       U, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf, (const double*)m.fgeo, m.elemSide,
-      (double*)m.Gf, (double*)m.Utv, store_grad ? (double*)m.Gvol : nullptr, m.K, m.S, m.Sface, (const double*)m.QB, ops,
-      m.fx, ph);
+      (double*)m.Gf, volume ? (double*)m.Utv : nullptr, store_grad ? (double*)m.Gvol : nullptr, m.K, m.S, m.Sface,
+      (const double*)m.QB, ops, m.fx, ph);
   return cudaGetLastError();
 }
 

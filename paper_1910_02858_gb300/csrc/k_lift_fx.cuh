@@ -121,6 +121,7 @@ __device__ __noinline__ void lift_vol_fp64(const double* U, const double* Ja, co
     }
     __syncthreads();
   }
+  if (Utv == nullptr) return;
   double F[3][NV];
   for (int d = 0; d < 3; ++d) flux_total(Uo, W, G, d, ph, F[d]);
   for (int l = 0; l < 3; ++l)
@@ -351,6 +352,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
     }
     __syncthreads();
   }
+  if (Utv == nullptr) return;  // the adjoint's recompute needs the gradients only
   // a6: physical fluxes in FP64, contravariant fluxes in fixed point
   fx64* own = sA + el * 15 * n3p + pn;  // the thread's entries
   {
