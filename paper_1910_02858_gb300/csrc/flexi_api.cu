@@ -39,7 +39,7 @@ struct flexi_ctx {
   size_t rs = 8;
   DevMesh m;
   // FP64 geometry (always) and FP32 copies (FP32 forms)
-  double *Ja64 = nullptr, *sJ64 = nullptr, *wJ = nullptr, *xsol = nullptr, *fgeo64 = nullptr, *xbc = nullptr;
+  double *Ja64 = nullptr, *sJ64 = nullptr, *wJ = nullptr, *fgeo64 = nullptr, *xbc = nullptr;
   float *Ja32 = nullptr, *sJ32 = nullptr, *fgeo32 = nullptr;
   int* elemSide = nullptr;
   int* bcKind = nullptr;       // device [nBC]
@@ -161,6 +161,15 @@ const Phys<double>& ph_of<double>(const flexi_ctx* c) { return c->ph64; }
 template <>
 const Phys<float>& ph_of<float>(const flexi_ctx* c) { return c->ph32; }
 
+// the source parameters at time t
+SourceParams source_at(const flexi_ctx* c, double t) {
+  SourceParams q = c->src;
+  const double a = M_PI * std::fmod(2.0 * t, 2.0);
+  q.st = std::sin(a);
+  q.ct = std::cos(a);
+  return q;
+}
+
 // one evaluation of the operator up to (and excluding) the surface kernel
 // face = false: without the face fluxes (k_surf_face computes them)
 template <typename real>
@@ -205,7 +214,7 @@ flexi_status do_rhs(flexi_ctx* c, const real* U, real* Ut, double t, cudaStream_
   if (s != FLEXI_OK) return s;
   RkStage<real> rk{real(0), real(0), real(0), 0};
   Prof pr(c, KC_SURF, st);
-  CK(launch_surf<real>(c->m, 0, nullptr, nullptr, Ut, rk, t, c->src, ops_of<real>(c), ph_of<real>(c), st));
+  CK(launch_surf<real>(c->m, 0, nullptr, nullptr, Ut, rk, source_at(c, t), ops_of<real>(c), ph_of<real>(c), st));
   return FLEXI_OK;
 }
 
@@ -236,7 +245,7 @@ flexi_status do_rk_step_fused(flexi_ctx* c, real* U, real* dU, double t, double 
       if (res != FLEXI_OK) break;
       RkStage<real> rk{(real)RK_A[k], (real)RK_B[k], (real)dt, (k < 4 || prolong_last) ? 1 : 0};
       Prof pr(c, KC_SURF, st);
-      if (launch_surf_face(c->m, win, wout, U, dU, rk, tk, c->src, ops_of<real>(c), ph_of<real>(c), st) !=
+      if (launch_surf_face(c->m, win, wout, U, dU, rk, source_at(c, tk), ops_of<real>(c), ph_of<real>(c), st) !=
           cudaSuccess)
         res = FLEXI_ECUDA;
     }
@@ -259,7 +268,7 @@ flexi_status do_rk_step(flexi_ctx* c, real* U, real* dU, double t, double dt, re
     if (s != FLEXI_OK) return s;
     RkStage<real> rk{(real)RK_A[k], (real)RK_B[k], (real)dt, (k < 4 || prolong_last) ? 1 : 0};
     Prof pr(c, KC_SURF, st);
-    CK(launch_surf<real>(c->m, 1, U, dU, nullptr, rk, tk, c->src, ops_of<real>(c), ph_of<real>(c), st));
+    CK(launch_surf<real>(c->m, 1, U, dU, nullptr, rk, source_at(c, tk), ops_of<real>(c), ph_of<real>(c), st));
   }
   return FLEXI_OK;
 }
@@ -485,7 +494,6 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   AL(c->bcKind, (size_t)std::max(c->nBC, 1));  // zero: every boundary takes the exact state
   AL(c->elemSide, (size_t)K * 6);
   AL(c->status, 1);
-  if (p->source) AL(c->xsol, (size_t)K * 3 * n3);
 
   // ---- temporary geometry buffers
   std::vector<void*> tmp;
@@ -586,7 +594,12 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   for (int l = 0; l < 3; ++l) CK(geom_apply1d(Xr, dX[l], dDs, 3 * K, n, n, n, l, n, st));
   CK(geom_jacobian(dX, c->sJ64, c->wJ, wdev, K, n, c->status, st));
   CK(geom_faces(c->Ja64, X, sideM, dlm, dlp, c->fgeo64, c->xbc, S, c->nBC, n, st));
-  if (p->source) CK(cudaMemcpyAsync(c->xsol, X, (size_t)K * 3 * n3 * 8, cudaMemcpyDeviceToDevice, st));
+  if (p->source) {
+    unsigned char* phase;
+    AL(phase, (size_t)K * 2 * n3 * c->rs);
+    CK(geom_phase(X, phase, c->fp64, K, n3, st));
+    c->m.phase = phase;
+  }
   unsigned bad = 0;
   CK(cudaMemcpyAsync(&bad, c->status, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -615,7 +628,6 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   c->m.elemSide = c->elemSide;
   c->m.xbc = c->xbc;
   c->m.bcKind = c->bcKind;
-  c->m.xsol = c->xsol;
   c->m.status = c->status;
   c->m.sweep_mode = p->precision == FLEXI_FP32_TF32 ? 1 : (p->precision == FLEXI_FP32_BF16 ? 2 : 0);
   c->m.lgl = p->node_type == FLEXI_NODES_LOBATTO ? 1 : 0;

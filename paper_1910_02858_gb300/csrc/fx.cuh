@@ -34,7 +34,8 @@ struct FxOps {
   int oh[FXH][FXH], ol[FXH][FXH];  // DO[i][a], i < (n+1)/2, a < n/2
   int sh[FXH], sl[FXH], th[FXH], tl[FXH];
   int peh[FXH], pel[FXH], poh[FXH], pol[FXH];  // prolongation to the line's ends, scale 2^kp
-  int kc, kp;
+  int lh[MAXN], ll[MAXN];  // l_hat_i(+1), scale 2^kl (l_hat_i(-1) is the entry of N - i)
+  int kc, kp, kl;
 };
 
 // host construction from the FP64 operators (integer rounding of scaled doubles: the
@@ -86,6 +87,12 @@ inline FxOps make_fx_ops(const Ops<double>& o, int n) {
     for (int a = 0; a < h; ++a) split(A(i, a) - A(i, N - a), f.oh[i][a], f.ol[i][a]);
     split(Q(i) + Q(N - i), f.sh[i], f.sl[i]);
   }
+  double lmax = 0;
+  for (int i = 0; i < n; ++i) lmax = std::fmax(lmax, std::fmax(std::fabs(o.lhp[i]), std::fabs(o.lhm[i])));
+  std::frexp(lmax * (1 + 1e-12), &x);
+  f.kl = 62 - x;
+  for (int i = 0; i < n; ++i)
+    split(std::llrint(std::ldexp(o.lhp[i], f.kl - 1)) + std::llrint(std::ldexp(o.lhm[N - i], f.kl - 1)), f.lh[i], f.ll[i]);
   for (int a = 0; a < c; ++a) split(2 * a == N ? 2 * L(a) : L(a) + L(N - a), f.peh[a], f.pel[a]);
   for (int a = 0; a < h; ++a) split(L(a) - L(N - a), f.poh[a], f.pol[a]);
   return f;

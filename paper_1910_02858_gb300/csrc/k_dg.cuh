@@ -950,6 +950,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_vol_min_blocks<real, n, SW, SP
 
 }  // namespace flexi
 #include "k_lift_fx.cuh"
+#include "k_surf_fx.cuh"
 namespace flexi {
 
 // a2-a4, a6, a7 for small FP64 meshes (fewer elements than SMs, n <= 4; standard form,
@@ -1532,7 +1533,7 @@ template <typename real, int n, int MODE, bool LGL, int TM = 1>
 __global__ void __launch_bounds__(Cfg<n>::T * TM, TM > 1 ? 1 : ((sizeof(real) == 4 && Cfg<n>::T == 512) ? 4 : ((sizeof(real) == 4 && Cfg<n>::T == 216) ? 8 : 2))) k_surf(
     const real* __restrict__ Ff, const int* __restrict__ elemSide, const real* __restrict__ sJ,
     const real* __restrict__ Utv, real* __restrict__ U, real* __restrict__ dU, real* __restrict__ Ut,
-    real* __restrict__ Wf, const double* __restrict__ xsol, RkStage<real> rk, double t, SourceParams src, int K,
+    real* __restrict__ Wf, const real* __restrict__ phase, RkStage<real> rk, SourceParams src, int K,
     int S, Ops<real> ops, Phys<real> ph, unsigned* __restrict__ status) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T * TM;
@@ -1609,21 +1610,12 @@ __global__ void __launch_bounds__(Cfg<n>::T * TM, TM > 1 ? 1 : ((sizeof(real) ==
       ut[v] = s * scale;
     }
     if (src.on) {
-      double x[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) x[c] = xsol[((size_t)e * 3 + c) * n3 + node];
+      const real* p = phase + (size_t)e * 2 * n3 + node;
       const real sdt = MODE == 1 ? rk.dt : real(1);
-      if constexpr (sizeof(real) == 4) {
-        float Sv[NV];
-        manufactured_source_f32(x, t, (float)src.gamma, (float)src.mu, (float)src.Pr, Sv);
+      real Sv[NV];
+      manufactured_source(p[0], p[n3], src, Sv);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) ut[v] = dg_fma(sdt, Sv[v], ut[v]);
-      } else {
-        double Sv[NV];
-        manufactured_source(x, t, src.gamma, src.mu, src.Pr, Sv);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) ut[v] = dg_fma(sdt, (real)Sv[v], ut[v]);
-      }
+      for (int v = 0; v < NV; ++v) ut[v] = dg_fma(sdt, Sv[v], ut[v]);
     }
   }
   if (MODE == 0) {
@@ -1668,8 +1660,8 @@ template <int RS, bool LGL>
 __global__ void __launch_bounds__(384) k_surf_face(
     const double* __restrict__ WfIn, const double* __restrict__ Gf, const double* __restrict__ fgeo,
     const int* __restrict__ elemSide, const double* __restrict__ sJ, const double* __restrict__ Utv,
-    double* __restrict__ U, double* __restrict__ dU, double* __restrict__ WfOut, const double* __restrict__ xsol,
-    RkStage<double> rk, double t, SourceParams src, int K, int S, int nBC, Ops<double> ops, Phys<double> ph,
+    double* __restrict__ U, double* __restrict__ dU, double* __restrict__ WfOut, const double* __restrict__ phase,
+    RkStage<double> rk, SourceParams src, int K, int S, int nBC, Ops<double> ops, Phys<double> ph,
     unsigned* __restrict__ status) {
   using real = double;
   constexpr int n = 4, n2 = n * n, n3 = n2 * n, n3p = Cfg<n>::n3p, T = 384, FN = 6 * n2;
@@ -1775,11 +1767,9 @@ __global__ void __launch_bounds__(384) k_surf_face(
     }
     real ut = a * -(rk.dt * sj);
     if (src.on) {
-      double x[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) x[c] = xsol[((size_t)e * 3 + c) * n3 + node];
+      const double* p = phase + (size_t)e * 2 * n3 + node;
       double Sv[NV];
-      manufactured_source(x, t, src.gamma, src.mu, src.Pr, Sv);
+      manufactured_source(p[0], p[n3], src, Sv);
       const double Su = uv == 0 ? Sv[0] : (uv == 1 ? Sv[1] : (uv == 2 ? Sv[2] : (uv == 3 ? Sv[3] : Sv[4])));
       ut = dg_fma(rk.dt, (real)Su, ut);
     }
@@ -1809,8 +1799,8 @@ template <int RS>
 __global__ void __launch_bounds__(384) k_surf_face2(
     const double* __restrict__ WfIn, const double* __restrict__ Gf, const double* __restrict__ fgeo,
     const int* __restrict__ elemSide, const double* __restrict__ sJ, const double* __restrict__ Utv,
-    double* __restrict__ U, double* __restrict__ dU, double* __restrict__ WfOut, const double* __restrict__ xsol,
-    RkStage<double> rk, double t, SourceParams src, int K, int S, int nBC, Ops<double> ops, Phys<double> ph,
+    double* __restrict__ U, double* __restrict__ dU, double* __restrict__ WfOut, const double* __restrict__ phase,
+    RkStage<double> rk, SourceParams src, int K, int S, int nBC, Ops<double> ops, Phys<double> ph,
     unsigned* __restrict__ status) {
   using real = double;
   constexpr int n = 4, n2 = n * n, n3 = n2 * n, n3p = Cfg<n>::n3p, hk = n / 2, h3 = n3 / 2;
@@ -1927,11 +1917,9 @@ __global__ void __launch_bounds__(384) k_surf_face2(
     if (k == n - 1) a = dg_fma(lhp[k], sF[(5 * NV + uv) * n2 + pq2], a);
     real ut = a * -(rk.dt * sj);
     if (src.on) {
-      double x[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) x[c] = xsol[((size_t)e * 3 + c) * n3 + node];
+      const double* p = phase + (size_t)e * 2 * n3 + node;
       double Sv[NV];
-      manufactured_source(x, t, src.gamma, src.mu, src.Pr, Sv);
+      manufactured_source(p[0], p[n3], src, Sv);
       const double Su = uv == 0 ? Sv[0] : (uv == 1 ? Sv[1] : (uv == 2 ? Sv[2] : (uv == 3 ? Sv[3] : Sv[4])));
       ut = dg_fma(rk.dt, (real)Su, ut);
     }
@@ -1982,7 +1970,13 @@ static cudaError_t prolong_n(const DevMesh& m, const real* U, const Ops<real>& o
                              cudaStream_t st) {
   using C = Cfg<n>;
   const int grid = (m.K + C::NE - 1) / C::NE;
-  k_prolong<real, n, LGL><<<grid, C::T, 0, st>>>(U, m.elemSide, (real*)m.Wf, m.K, m.S, ops, ph, m.status);
+  // FP64: in fixed point wherever the surface kernel writes the face states so (surf_n), which
+  // keeps a run's bits independent of how its steps are called
+  if (sizeof(real) == 8 && !(n <= 4 && grid < m.nsm)) {
+    if constexpr (sizeof(real) == 8) k_prolong_fx<n, LGL><<<grid, C::T, 0, st>>>(U, m.elemSide, (double*)m.Wf, m.K, m.S, ops, m.fx, ph, m.status);
+  } else {
+    k_prolong<real, n, LGL><<<grid, C::T, 0, st>>>(U, m.elemSide, (real*)m.Wf, m.K, m.S, ops, ph, m.status);
+  }
   return cudaGetLastError();
 }
 
@@ -2151,14 +2145,14 @@ cudaError_t launch_face(const DevMesh& m, const Phys<real>& ph, cudaStream_t st)
 }
 
 template <typename real, int n, bool LGL>
-static cudaError_t surf_n(const DevMesh& m, int mode, real* U, real* dU, real* Ut, const RkStage<real>& rk, double t,
+static cudaError_t surf_n(const DevMesh& m, int mode, real* U, real* dU, real* Ut, const RkStage<real>& rk,
                           const SourceParams& src, const Ops<real>& ops, const Phys<real>& ph, cudaStream_t st) {
   using C = Cfg<n>;
   const int grid = (m.K + C::NE - 1) / C::NE;
 #define FLEXI_SURF(MODEV, TMV)                                                                                    \
   k_surf<real, n, MODEV, LGL, TMV><<<grid, C::T * TMV, 0, st>>>((const real*)m.Ff, m.elemSide, (const real*)m.sJ, \
-                                                                 (const real*)m.Utv, U, dU, Ut, (real*)m.Wf, m.xsol, \
-                                                                 rk, t, src, m.K, m.S, ops, ph, m.status)
+                                                                 (const real*)m.Utv, U, dU, Ut, (real*)m.Wf, (const real*)m.phase, \
+                                                                 rk, src, m.K, m.S, ops, ph, m.status)
   if constexpr (n <= 4) {
     if (grid < m.nsm) {  // fewer CTAs than SMs: six times the threads for the face loops
       if (mode == 0)
@@ -2168,21 +2162,32 @@ static cudaError_t surf_n(const DevMesh& m, int mode, real* U, real* dU, real* U
       return cudaGetLastError();
     }
   }
-  if (mode == 0)
-    FLEXI_SURF(0, 1);
-  else
-    FLEXI_SURF(1, 1);
+  if constexpr (sizeof(real) == 8) {
+    if (mode == 0)
+      k_surf_fx<n, 0, LGL><<<grid, C::T, 0, st>>>((const double*)m.Ff, m.elemSide, (const double*)m.sJ, (const double*)m.Utv, U,
+                                                  dU, Ut, (double*)m.Wf, (const double*)m.phase, rk, src, m.K, m.S, ops, m.fx,
+                                                  ph, m.status);
+    else
+      k_surf_fx<n, 1, LGL><<<grid, C::T, 0, st>>>((const double*)m.Ff, m.elemSide, (const double*)m.sJ, (const double*)m.Utv, U,
+                                                  dU, Ut, (double*)m.Wf, (const double*)m.phase, rk, src, m.K, m.S, ops, m.fx,
+                                                  ph, m.status);
+  } else {
+    if (mode == 0)
+      FLEXI_SURF(0, 1);
+    else
+      FLEXI_SURF(1, 1);
+  }
 #undef FLEXI_SURF
   return cudaGetLastError();
 }
 
 template <typename real>
-cudaError_t launch_surf(const DevMesh& m, int mode, real* U, real* dU, real* Ut, const RkStage<real>& rk, double t,
+cudaError_t launch_surf(const DevMesh& m, int mode, real* U, real* dU, real* Ut, const RkStage<real>& rk,
                         const SourceParams& src, const Ops<real>& ops, const Phys<real>& ph, cudaStream_t st) {
   if (m.lgl) {
-    FLEXI_DISPATCH_N(m.n, return surf_n<real, NN, true>(m, mode, U, dU, Ut, rk, t, src, ops, ph, st));
+    FLEXI_DISPATCH_N(m.n, return surf_n<real, NN, true>(m, mode, U, dU, Ut, rk, src, ops, ph, st));
   }
-  FLEXI_DISPATCH_N(m.n, return surf_n<real, NN, false>(m, mode, U, dU, Ut, rk, t, src, ops, ph, st));
+  FLEXI_DISPATCH_N(m.n, return surf_n<real, NN, false>(m, mode, U, dU, Ut, rk, src, ops, ph, st));
   return cudaSuccess;
 }
 

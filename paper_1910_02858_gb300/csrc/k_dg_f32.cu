@@ -13,7 +13,7 @@ template cudaError_t launch_face<float>(const DevMesh&, const Phys<float>&, cuda
 template cudaError_t launch_mortar_state<float>(const DevMesh&, const MortarOps<float>&, const Phys<float>&, cudaStream_t);
 template cudaError_t launch_mortar_grad<float>(const DevMesh&, const MortarOps<float>&, const Phys<float>&, cudaStream_t);
 template cudaError_t launch_mortar_flux<float>(const DevMesh&, const MortarOps<float>&, cudaStream_t);
-template cudaError_t launch_surf<float>(const DevMesh&, int, float*, float*, float*, const RkStage<float>&, double,
+template cudaError_t launch_surf<float>(const DevMesh&, int, float*, float*, float*, const RkStage<float>&,
                                        const SourceParams&, const Ops<float>&, const Phys<float>&, cudaStream_t);
 template cudaError_t launch_reduce<float>(const float*, const float*, const double*, const double*, const double*,
                                          long long, int, const Phys<float>&, double, double*, int, cudaStream_t);

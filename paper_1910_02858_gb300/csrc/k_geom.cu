@@ -152,4 +152,28 @@ cudaError_t convert_f64_to_f32(const double* in, float* out, size_t count, cudaS
   return cudaGetLastError();
 }
 
+namespace {
+template <typename real>
+__global__ void k_phase(const double* __restrict__ X, real* __restrict__ phase, int K, int n3) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (long long)K * n3) return;
+  const long long e = t / n3;
+  const int node = (int)(t - e * n3);
+  const double* x = X + e * 3 * n3 + node;
+  double s, c;
+  sincospi(x[0] + x[n3] + x[2 * n3], &s, &c);
+  phase[e * 2 * n3 + node] = (real)s;
+  phase[(e * 2 + 1) * n3 + node] = (real)c;
+}
+}  // namespace
+
+cudaError_t geom_phase(const double* X, void* phase, bool fp64, int K, int n3, cudaStream_t st) {
+  const unsigned grid = (unsigned)(((size_t)K * n3 + 255) / 256);
+  if (fp64)
+    k_phase<double><<<grid, 256, 0, st>>>(X, (double*)phase, K, n3);
+  else
+    k_phase<float><<<grid, 256, 0, st>>>(X, (float*)phase, K, n3);
+  return cudaGetLastError();
+}
+
 }  // namespace flexi

@@ -40,7 +40,7 @@ struct DevMesh {
   const int* elemSide = nullptr;  // [K][6] packed (side<<4 | slave<<3 | orient)
   const double* xbc = nullptr;    // [nBC][3][n^2] face node coordinates of boundary sides
   const int* bcKind = nullptr;    // [nBC] 0 exact state, 1 outflow, 2 slip wall
-  const double* xsol = nullptr;   // [K][3][n^3] (only with a source term)
+  const void* phase = nullptr;    // [K][2][n^3] sin, cos of pi (x + y + z) at the nodes (only with a source term)
   void* Wf = nullptr;          // [2][S][5][n^2] primitive face states (slot 0 master, 1 slave/boundary)
   void* Gf = nullptr;          // [2][S][15][n^2] lifted gradients on the faces (index d*5+v)
   void* Ff = nullptr;          // [S][5][n^2] numerical flux f* s_hat in the master normal
@@ -55,11 +55,6 @@ struct DevMesh {
   void* QB = nullptr;          // [nBig][15][n^2] BR1 lifting flux of the big element
   FxOps fx{};                  // fixed-point line operators (FP64 form)
   unsigned* status = nullptr;  // device status word (bit 0: non-physical face state)
-};
-
-struct SourceParams {
-  int on = 0;
-  double gamma = 1.4, mu = 0, Pr = 0.72;
 };
 
 template <typename real>
@@ -88,14 +83,14 @@ cudaError_t launch_mortar_flux(const DevMesh& m, const MortarOps<real>& mo, cuda
 // mode 0: Ut = L(U); mode 1: RK stage update of U, dU in place
 template <typename real>
 cudaError_t launch_surf(const DevMesh& m, int mode, real* U, real* dU, real* Ut, const RkStage<real>& rk,
-                        double t, const SourceParams& src, const Ops<real>& ops, const Phys<real>& ph,
+                        const SourceParams& src, const Ops<real>& ops, const Phys<real>& ph,
                         cudaStream_t st);
 
 // a5 and a8-a10 of an RK stage in one kernel (FP64, n = 4, no mortars, BR1; meant for
 // meshes with fewer elements than SMs): face states read from WfIn, those of the new U
 // written to WfOut when rk.prolong (WfOut != WfIn: other elements still read WfIn)
 cudaError_t launch_surf_face(const DevMesh& m, const void* WfIn, void* WfOut, double* U, double* dU,
-                             const RkStage<double>& rk, double t, const SourceParams& src, const Ops<double>& ops,
+                             const RkStage<double>& rk, const SourceParams& src, const Ops<double>& ops,
                              const Phys<double>& ph, cudaStream_t st);
 // adjoint of the right-hand side: out = (dL/dU)^T lam  (uses Gvol written by
 // launch_lift_vol with store_grad = 1); mode 1 accumulates out += scale * result
@@ -141,6 +136,8 @@ cudaError_t geom_jacobian(const double* const dX[3], double* sJ, double* wJ, con
                           unsigned* bad, cudaStream_t st);
 cudaError_t geom_faces(const double* Ja, const double* X, const int* sideMaster, const double* lm,
                        const double* lp, double* fgeo, double* xbc, int S, int nBC, int n, cudaStream_t st);
+// sine and cosine of pi (x + y + z) at the solution nodes, [K][2][n^3]
+cudaError_t geom_phase(const double* X, void* phase, bool fp64, int K, int n3, cudaStream_t st);
 cudaError_t convert_f64_to_f32(const double* in, float* out, size_t count, cudaStream_t st);
 
 }  // namespace flexi
