@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fp64_math.cuh"
+
 namespace flexi {
 
 constexpr int NV = 5;     // conserved / lifted variables
@@ -87,15 +89,36 @@ __device__ __forceinline__ int vol_index(int l, int a, int p, int q, int n) {
 // ---------------------------------------------------------------------------
 // pointwise physics
 // ---------------------------------------------------------------------------
+// division and roots: on the integer pipes in the FP64 form (fp64_math.cuh)
 template <typename real>
-__device__ __forceinline__ void cons_to_prim(const real U[NV], real W[NV], const Phys<real>& ph) {
-  real ir = real(1) / U[0];
+__device__ __forceinline__ real dg_rcp(real x) { return real(1) / x; }
+__device__ __forceinline__ double dg_rcp(double x) { return fp64_rcp(x); }
+
+template <typename real>
+__device__ __forceinline__ real dg_div(real a, real b) { return a / b; }
+// the quotient's rounding error is taken out by one residual; operands or quotients near the
+// ends of the range take the division
+__device__ __forceinline__ double dg_div(double a, double b) {
+  const double r = fp64_rcp(b);
+  const double q = a * r;
+  const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu, eq = ((unsigned)__double2hiint(q) >> 20) & 0x7ffu;
+  if (eb - 64u > 1900u || eq - 64u > 1900u) return a / b;
+  return fma(fma(-q, b, a), r, q);
+}
+
+template <typename real>
+__device__ __forceinline__ void cons_to_prim(const real U[NV], const real ir, real W[NV], const Phys<real>& ph) {
   real u = U[1] * ir, v = U[2] * ir, w = U[3] * ir;
   W[0] = U[0];
   W[1] = u;
   W[2] = v;
   W[3] = w;
   W[4] = ph.gm1 * (U[4] - real(0.5) * (U[1] * u + U[2] * v + U[3] * w));
+}
+
+template <typename real>
+__device__ __forceinline__ void cons_to_prim(const real U[NV], real W[NV], const Phys<real>& ph) {
+  cons_to_prim(U, dg_rcp(U[0]), W, ph);
 }
 
 template <typename real>
@@ -107,9 +130,9 @@ __device__ __forceinline__ void prim_to_cons(const real W[NV], real U[NV], const
   U[4] = W[4] * ph.inv_gm1 + real(0.5) * (U[1] * W[1] + U[2] * W[2] + U[3] * W[3]);
 }
 
-// Navier-Stokes flux F^c_d - F^v_d in physical direction d; G[d*5 + v] = dW_v/dx_d
+// Navier-Stokes flux F^c_d - F^v_d in physical direction d; G[d*5 + v] = dW_v/dx_d, ir = 1 / rho
 template <typename real>
-__device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], const real G[15], int d,
+__device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], const real ir, const real G[15], int d,
                                            const Phys<real>& ph, real F[NV]) {
   const real ud = W[1 + d];
   const real p = W[4];
@@ -119,7 +142,6 @@ __device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], c
 #pragma unroll
   for (int c = 0; c < 3; ++c) tau[c] = ph.mu * (G[d * 5 + 1 + c] + G[c * 5 + 1 + d]);
   tau[d] -= real(2.0 / 3.0) * ph.mu * div;
-  const real ir = real(1) / W[0];
   const real dT = (G[d * 5 + 4] - p * ir * G[d * 5 + 0]) * ir;  // d(p/rho)/dx_d
   const real fv4 = tau[0] * W[1] + tau[1] * W[2] + tau[2] * W[3] + ph.lam_th * dT;
   F[0] = U[1 + d];
@@ -128,6 +150,12 @@ __device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], c
   F[3] = U[3] * ud - tau[2];
   F[1 + d] += p;
   F[4] = ud * (U[4] + p) - fv4;
+}
+
+template <typename real>
+__device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], const real G[15], int d,
+                                           const Phys<real>& ph, real F[NV]) {
+  flux_total(U, W, dg_rcp(W[0]), G, d, ph, F);
 }
 
 // normal viscous flux F^v . n, with ir = 1 / rho of the state
@@ -157,20 +185,20 @@ __device__ __forceinline__ void visc_normal(const real W[NV], const real ir, con
 template <typename real>
 __device__ __forceinline__ void visc_normal(const real W[NV], const real G[15], const real n[3],
                                             const Phys<real>& ph, real f[NV]) {
-  visc_normal(W, real(1) / W[0], G, n, ph, f);
+  visc_normal(W, dg_rcp(W[0]), G, n, ph, f);
 }
 
 template <typename real>
 __device__ __forceinline__ real dg_sqrt(real x);
 template <>
-__device__ __forceinline__ double dg_sqrt<double>(double x) { return sqrt(x); }
+__device__ __forceinline__ double dg_sqrt<double>(double x) { return fp64_sqrt(x); }
 template <>
 __device__ __forceinline__ float dg_sqrt<float>(float x) { return sqrtf(x); }
 
 template <typename real>
 __device__ __forceinline__ real dg_rsqrt(real x);
 template <>
-__device__ __forceinline__ double dg_rsqrt<double>(double x) { return rsqrt(x); }
+__device__ __forceinline__ double dg_rsqrt<double>(double x) { return fp64_rsqrt(x); }
 template <>
 __device__ __forceinline__ float dg_rsqrt<float>(float x) { return rsqrtf(x); }
 
@@ -218,7 +246,7 @@ __device__ __forceinline__ void riemann_hllc(const real WL[NV], const real WR[NV
   const real cL = dg_sqrt(ph.gamma * WL[4] * irL);
   const real cR = dg_sqrt(ph.gamma * WR[4] * irR);
   const real r = dg_sqrt(WR[0] * irL);
-  const real iw = real(1) / (real(1) + r);
+  const real iw = dg_rcp(real(1) + r);
   const real HL = (EL + WL[4]) * irL, HR = (ER + WR[4]) * irR;
   real vel[3];
 #pragma unroll
@@ -237,7 +265,7 @@ __device__ __forceinline__ void riemann_hllc(const real WL[NV], const real WR[NV
     return;
   }
   const real mL = WL[0] * (SL - uL), mR = WR[0] * (SR - uR);
-  const real Ss = (WR[4] - WL[4] + mL * uL - mR * uR) / (mL - mR);
+  const real Ss = dg_div(WR[4] - WL[4] + mL * uL - mR * uR, mL - mR);
   const bool left = Ss >= real(0);
   real W[NV];  // the upwind state, selected by value (a pointer select would force the arrays to memory)
 #pragma unroll
@@ -250,7 +278,7 @@ __device__ __forceinline__ void riemann_hllc(const real WL[NV], const real WR[NV
   euler_normal(W, E, uK, n, f);
   // star state: fac (1, S* n + v_t, E/rho + (S*-u)(S* + p/(rho(S-u)))), fac = mK / (S - S*)
   const real dS = S - Ss;
-  const real q = real(1) / (mK * dS);
+  const real q = dg_rcp(mK * dS);
   const real fac = mK * mK * q;
   const real U0 = W[0];
   f[0] += S * (fac - U0);
@@ -266,7 +294,7 @@ __device__ __forceinline__ void riemann_hllc(const real WL[NV], const real WR[NV
 template <typename real>
 __device__ __forceinline__ void riemann_hllc(const real WL[NV], const real WR[NV], const real n[3],
                                              const Phys<real>& ph, real f[NV]) {
-  riemann_hllc(WL, WR, real(1) / WL[0], real(1) / WR[0], n, ph, f);
+  riemann_hllc(WL, WR, dg_rcp(WL[0]), dg_rcp(WR[0]), n, ph, f);
 }
 
 // Roe flux (5-wave, frame-free); smooth != 0: Harten-type smoothing of |lambda| (below
@@ -302,7 +330,7 @@ __device__ __forceinline__ void roe_dissipation(const real WL[NV], const real WR
   // sqrt(rho) H = (E + p) / sqrt(rho)
   const real isL = dg_rsqrt(WL[0]), isR = dg_rsqrt(WR[0]);
   const real sL = WL[0] * isL, sR = WR[0] * isR;
-  const real iw = real(1) / (sL + sR);
+  const real iw = dg_rcp(sL + sR);
   real vel[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) vel[c] = dg_fma(sL, WL[1 + c], sR * WR[1 + c]) * iw;
@@ -367,7 +395,7 @@ __device__ __forceinline__ void riemann_rusanov(const real WL[NV], const real WR
   euler_normal(WR, ER, uR, n, FR);
   prim_to_cons(WL, UL, ph);
   prim_to_cons(WR, UR, ph);
-  const real cL = dg_sqrt(ph.gamma * WL[4] / WL[0]), cR = dg_sqrt(ph.gamma * WR[4] / WR[0]);
+  const real cL = dg_sqrt(dg_div(ph.gamma * WL[4], WL[0])), cR = dg_sqrt(dg_div(ph.gamma * WR[4], WR[0]));
   const real lam = fmax(dg_abs(uL) + cL, dg_abs(uR) + cR);
 #pragma unroll
   for (int v = 0; v < NV; ++v) f[v] = real(0.5) * (FL[v] + FR[v]) - real(0.5) * lam * (UR[v] - UL[v]);
@@ -381,12 +409,11 @@ template <>
 __device__ __forceinline__ float dg_log<float>(float x) { return logf(x); }
 
 // logarithmic mean (a - b)/(ln a - ln b) of positive a, b (Ismail & Roe form):
-// zeta = a/b, f = (zeta - 1)/(zeta + 1), u = f^2; mean = (a + b)/(2 F) with
-// F = atanh(f)/f = ln(zeta)/(2 f), or its series sum_k u^k/(2k + 1) to u^7 for u < 1e-2
+// f = (a - b)/(a + b), u = f^2; mean = (a + b)/(2 F) with
+// F = atanh(f)/f = ln(a/b)/(2 f), or its series sum_k u^k/(2k + 1) to u^7 for u < 1e-2
 template <typename real>
 __device__ __forceinline__ real log_mean(real a, real b) {
-  const real zeta = a / b;
-  const real f = (zeta - real(1)) / (zeta + real(1));
+  const real f = dg_div(a - b, a + b);
   const real u = f * f;
   real F;
   if (u < real(1e-2)) {
@@ -399,9 +426,9 @@ __device__ __forceinline__ real log_mean(real a, real b) {
     F = F * u + real(1.0 / 3.0);
     F = F * u + real(1);
   } else {
-    F = dg_log(zeta) / (real(2) * f);
+    F = dg_div(dg_log(dg_div(a, b)), real(2) * f);
   }
-  return (a + b) / (real(2) * F);
+  return dg_div(a + b, real(2) * F);
 }
 
 // Chandrashekar's entropy-conservative two-point flux in the direction Jm (the
@@ -413,12 +440,12 @@ __device__ __forceinline__ void ec_flux(real ra, const real ua[3], real ba, real
                                         real bb, real qb, const real Jm[3], const Phys<real>& ph, real f[NV]) {
   const real um[3] = {real(0.5) * (ua[0] + ub[0]), real(0.5) * (ua[1] + ub[1]), real(0.5) * (ua[2] + ub[2])};
   const real frho = log_mean(ra, rb) * (um[0] * Jm[0] + um[1] * Jm[1] + um[2] * Jm[2]);
-  const real ptil = real(0.5) * (ra + rb) / (ba + bb);
+  const real ptil = dg_div(real(0.5) * (ra + rb), ba + bb);
   f[0] = frho;
   f[1] = frho * um[0] + ptil * Jm[0];
   f[2] = frho * um[1] + ptil * Jm[1];
   f[3] = frho * um[2] + ptil * Jm[2];
-  f[4] = frho * (real(0.5) * ph.inv_gm1 / log_mean(ba, bb) - real(0.25) * (qa + qb)) + um[0] * f[1] + um[1] * f[2] +
+  f[4] = frho * (dg_div(real(0.5) * ph.inv_gm1, log_mean(ba, bb)) - real(0.25) * (qa + qb)) + um[0] * f[1] + um[1] * f[2] +
          um[2] * f[3];
 }
 
@@ -427,8 +454,8 @@ template <typename real>
 __device__ __forceinline__ void riemann_ec(const real WL[NV], const real WR[NV], const real n[3], const Phys<real>& ph,
                                            real f[NV]) {
   const real uL[3] = {WL[1], WL[2], WL[3]}, uR[3] = {WR[1], WR[2], WR[3]};
-  ec_flux(WL[0], uL, real(0.5) * WL[0] / WL[4], uL[0] * uL[0] + uL[1] * uL[1] + uL[2] * uL[2], WR[0], uR,
-          real(0.5) * WR[0] / WR[4], uR[0] * uR[0] + uR[1] * uR[1] + uR[2] * uR[2], n, ph, f);
+  ec_flux(WL[0], uL, dg_div(real(0.5) * WL[0], WL[4]), uL[0] * uL[0] + uL[1] * uL[1] + uL[2] * uL[2], WR[0], uR,
+          dg_div(real(0.5) * WR[0], WR[4]), uR[0] * uR[0] + uR[1] * uR[1] + uR[2] * uR[2], n, ph, f);
 }
 
 // numerical flux of a compile-time kind RS (FLEXI_RIEMANN_*: 0 Roe and 2 smoothed Roe
@@ -456,7 +483,7 @@ __device__ __forceinline__ void riemann(const real WL[NV], const real WR[NV], co
   else if (ph.riemann == 4)
     riemann_ec(WL, WR, n, ph, f);
   else
-    riemann_roe(WL, WR, real(1) / WL[0], real(1) / WR[0], n, ph, ph.riemann == 2, f);
+    riemann_roe(WL, WR, dg_rcp(WL[0]), dg_rcp(WR[0]), n, ph, ph.riemann == 2, f);
 }
 
 // exact states (Dirichlet data) -- conservative variables at x, time t

@@ -43,7 +43,7 @@ namespace flexi {
 template <typename real>
 __device__ __forceinline__ void prim_vjp(const real W[NV], const real lamW[NV], const Phys<real>& ph,
                                          real lamU[NV]) {
-  const real ir = real(1) / W[0];
+  const real ir = dg_rcp(W[0]);
   const real q2 = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];
   real l0 = lamW[0] + lamW[4] * ph.gm1 * real(0.5) * q2;
 #pragma unroll
@@ -61,7 +61,7 @@ __device__ __forceinline__ void visc_vjp(const real W[NV], const real G[15], con
                                          const Phys<real>& ph, real lamW[NV], real lamG[15]) {
   const real mu = ph.mu;
   const real div = G[0 * 5 + 1] + G[1 * 5 + 2] + G[2 * 5 + 3];
-  const real ir = real(1) / W[0];
+  const real ir = dg_rcp(W[0]);
   real ldiv = real(0);
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -137,7 +137,7 @@ __device__ __forceinline__ void roe_vjp(const real WL[NV], const real WR[NV], co
   const real isL = dg_rsqrt(WL[0]), isR = dg_rsqrt(WR[0]);
   const real sL = WL[0] * isL, sR = WR[0] * isR;
   const real irL = isL * isL, irR = isR * isR;
-  const real iws = real(1) / (sL + sR);
+  const real iws = dg_rcp(sL + sR);
   const real HL = (EL + WL[4]) * irL, HR = (ER + WR[4]) * irR;
   real vel[3];
 #pragma unroll
@@ -316,7 +316,7 @@ template <typename real>
 __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], const real n[3], const Phys<real>& ph,
                                          const real lf[NV], real lWL[NV], real lWR[NV]) {
   // ---- forward
-  const real irL = real(1) / WL[0], irR = real(1) / WR[0];
+  const real irL = dg_rcp(WL[0]), irR = dg_rcp(WR[0]);
   const real q2L = WL[1] * WL[1] + WL[2] * WL[2] + WL[3] * WL[3];
   const real q2R = WR[1] * WR[1] + WR[2] * WR[2] + WR[3] * WR[3];
   const real EL = WL[4] * ph.inv_gm1 + real(0.5) * WL[0] * q2L;
@@ -326,7 +326,7 @@ __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], c
   const real cL = dg_sqrt(ph.gamma * WL[4] * irL);
   const real cR = dg_sqrt(ph.gamma * WR[4] * irR);
   const real r = dg_sqrt(WR[0] * irL);
-  const real iw = real(1) / (real(1) + r);
+  const real iw = dg_rcp(real(1) + r);
   const real HL = (EL + WL[4]) * irL, HR = (ER + WR[4]) * irR;
   real vel[3];
 #pragma unroll
@@ -353,7 +353,7 @@ __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], c
     return;
   }
   const real mL = WL[0] * (SL - uL), mR = WR[0] * (SR - uR);
-  const real iD = real(1) / (mL - mR);
+  const real iD = dg_rcp(mL - mR);
   const real Ss = (WR[4] - WL[4] + mL * uL - mR * uR) * iD;
   const bool left = Ss >= real(0);
   real W[NV];
@@ -364,7 +364,7 @@ __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], c
   // ---- reverse of f = F(W) + S (U* - U): U* = fac (1, v + (Ss - u) n, B),
   // fac = m / (S - Ss), B = E / rho + (Ss - u)(Ss + p / m)
   const real dS = S - Ss, du = Ss - u;
-  const real q = real(1) / (m * dS);
+  const real q = dg_rcp(m * dS);
   const real fac = m * m * q, pm = W[4] * dS * q;  // p / m
   const real B = dg_fma(E, irK, du * (Ss + pm));
   euler_normal_vjp(W, E, u, n, lf, lK, lEK, luK);
@@ -414,7 +414,7 @@ __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], c
   const real lun = (ownL ? real(0) : lSL) + (ownR ? real(0) : lSR);
   const real lc = (ownR ? real(0) : lSR) - (ownL ? real(0) : lSL);
   if (!ownL || !ownR) {  // Roe averages
-    const real lH = lc * real(0.5) * ph.gm1 / c;
+    const real lH = dg_div(lc * real(0.5) * ph.gm1, c);
     real lvel[3], dot = lH * (HR - H);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -439,12 +439,12 @@ __device__ __forceinline__ void hllc_vjp(const real WL[NV], const real WR[NV], c
   if (ownL) {  // c_L = sqrt(gamma p / rho)
     const real x = real(0.5) * lcL * cL;
     aL[0] = dg_fma(-x, irL, aL[0]);
-    aL[4] += x / WL[4];
+    aL[4] += dg_div(x, WL[4]);
   }
   if (ownR) {
     const real x = real(0.5) * lcR * cR;
     aR[0] = dg_fma(-x, irR, aR[0]);
-    aR[4] += x / WR[4];
+    aR[4] += dg_div(x, WR[4]);
   }
   energy_normal_vjp(WL, q2L, n, ph, lEL, luL, aL);
   energy_normal_vjp(WR, q2R, n, ph, lER, luR, aR);
@@ -461,7 +461,7 @@ __device__ __forceinline__ void rusanov_vjp(const real WL[NV], const real WR[NV]
                                             const real lf[NV], real lWL[NV], real lWR[NV]) {
   const real uL = WL[1] * n[0] + WL[2] * n[1] + WL[3] * n[2];
   const real uR = WR[1] * n[0] + WR[2] * n[1] + WR[3] * n[2];
-  const real cL = dg_sqrt(ph.gamma * WL[4] / WL[0]), cR = dg_sqrt(ph.gamma * WR[4] / WR[0]);
+  const real cL = dg_sqrt(dg_div(ph.gamma * WL[4], WL[0])), cR = dg_sqrt(dg_div(ph.gamma * WR[4], WR[0]));
   const real sL = dg_abs(uL) + cL, sR = dg_abs(uR) + cR;
   const bool selL = sL > sR;  // as the forward maximum selects
   const real lam = selL ? sL : sR;
@@ -494,7 +494,7 @@ __device__ __forceinline__ void rusanov_vjp(const real WL[NV], const real WR[NV]
   const real g = u < real(0) ? -ll : ll;
   const real rho = selL ? WL[0] : WR[0], p = selL ? WL[4] : WR[4];
   const real x = half * ll * c;
-  real a[NV] = {-x / rho, g * n[0], g * n[1], g * n[2], x / p};
+  real a[NV] = {-dg_div(x, rho), g * n[0], g * n[1], g * n[2], dg_div(x, p)};
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     lWL[v] += selL ? a[v] : real(0);
@@ -518,8 +518,8 @@ struct Dual {
   friend __device__ Dual operator-(Dual a) { return Dual(-a.v, -a.d); }
   friend __device__ Dual operator*(Dual a, Dual b) { return Dual(a.v * b.v, a.d * b.v + a.v * b.d); }
   friend __device__ Dual operator/(Dual a, Dual b) {
-    const r q = a.v / b.v;
-    return Dual(q, (a.d - q * b.d) / b.v);
+    const r q = dg_div(a.v, b.v);
+    return Dual(q, dg_div(a.d - q * b.d, b.v));
   }
   __device__ Dual& operator+=(Dual b) { return *this = *this + b; }
   __device__ Dual& operator-=(Dual b) { return *this = *this - b; }
@@ -613,7 +613,7 @@ __device__ void riemann_vjp_dual(const real WL[NV], const real WR[NV], const rea
 template <typename real>
 __device__ __forceinline__ void log_mean_d(real a, real b, real& L, real& dLda, real& iL) {
   const real s = a + b;
-  const real is = real(1) / s;
+  const real is = dg_rcp(s);
   const real f = (a - b) * is;
   const real u = f * f;
   real F, Fp;
@@ -634,10 +634,10 @@ __device__ __forceinline__ void log_mean_d(real a, real b, real& L, real& dLda, 
     Fp = Fp * u + real(2.0 / 5.0);
     Fp = Fp * u + real(1.0 / 3.0);
   } else {
-    F = dg_log(a / b) / (real(2) * f);
-    Fp = (real(1) / (real(1) - u) - F) / (real(2) * u);
+    F = dg_div(dg_log(dg_div(a, b)), real(2) * f);
+    Fp = dg_div(dg_rcp(real(1) - u) - F, real(2) * u);
   }
-  const real iF = real(1) / F;
+  const real iF = dg_rcp(F);
   L = real(0.5) * s * iF;
   iL = real(2) * F * is;
   dLda = real(0.5) * iF * (real(1) - real(4) * f * b * Fp * iF * is);
@@ -662,7 +662,7 @@ __device__ __forceinline__ void ec_pair_vjp(const real Wx[NV], real bx, real ipx
   log_mean_d(bx, ba, Lb, dLb, iLb);
   const real qa = Wa[1] * Wa[1] + Wa[2] * Wa[2] + Wa[3] * Wa[3];
   const real frho = Lr * Un;
-  const real ibs = real(1) / (bx + ba);
+  const real ibs = dg_rcp(bx + ba);
   const real pt = real(0.5) * (Wx[0] + Wa[0]) * ibs;
   const real Ep = real(0.5) * inv_gm1 * iLb - real(0.25) * (qx + qa);
   const real B = w[0] + w[1] * um[0] + w[2] * um[1] + w[3] * um[2] +
@@ -922,8 +922,8 @@ __global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
     for (int c = 0; c < 9; ++c) wj[(NV + c) * n3] = jac[c];
     // kinetic-energy-preserving pairs: total enthalpy H = gamma/(gamma-1) p/rho + |u|^2/2;
     // entropy-conservative pairs: beta = rho / (2 p)
-    wj[14 * n3] = SPLIT == 1 ? (ph.inv_gm1 + real(1)) * W[4] / W[0] + real(0.5) * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3])
-                             : real(0.5) * W[0] / W[4];
+    wj[14 * n3] = SPLIT == 1 ? dg_div((ph.inv_gm1 + real(1)) * W[4], W[0]) + real(0.5) * (W[1] * W[1] + W[2] * W[2] + W[3] * W[3])
+                             : dg_div(real(0.5) * W[0], W[4]);
   }
   // face-gradient adjoints of the element's six faces (own slot)
   __syncthreads();
@@ -972,7 +972,7 @@ __global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
     const real* wj = sWJ + el * 15 * n3;
     // per node: the enthalpy and its partials with respect to rho and p (KEP pairs), or
     // beta, 1/p and |u|^2 (EC pairs)
-    const real gg = ph.inv_gm1 + real(1), irx = real(1) / W[0], ipx = real(1) / W[4];
+    const real gg = ph.inv_gm1 + real(1), irx = dg_rcp(W[0]), ipx = dg_rcp(W[4]);
     const real x14 = wj[14 * n3 + node];  // this node's staged H (KEP) or beta (EC)
     const real dHdr = -gg * W[4] * irx * irx, dHdp = gg * irx;
     const real qx = W[1] * W[1] + W[2] * W[2] + W[3] * W[3];

@@ -719,8 +719,8 @@ __device__ __forceinline__ void lift_vol_body(
     // beta = rho/(2p), |u|^2 (entropy conservative, Chandrashekar), and Ja (9).
 #pragma unroll
     for (int c = 0; c < 4; ++c) myb[c * n3p + pn] = W[c];
-    const real H = SPLIT == 2 ? W[1] * W[1] + W[2] * W[2] + W[3] * W[3] : (Uo[4] + W[4]) / W[0];
-    myb[4 * n3p + pn] = SPLIT == 2 ? real(0.5) * W[0] / W[4] : W[4];
+    const real H = SPLIT == 2 ? W[1] * W[1] + W[2] * W[2] + W[3] * W[3] : dg_div(Uo[4] + W[4], W[0]);
+    myb[4 * n3p + pn] = SPLIT == 2 ? dg_div(real(0.5) * W[0], W[4]) : W[4];
     myb[5 * n3p + pn] = H;
 #pragma unroll
     for (int c = 0; c < 9; ++c) myb[(6 + c) * n3p + pn] = jac[c];
@@ -746,7 +746,7 @@ __device__ __forceinline__ void lift_vol_body(
             const real Jm[3] = {real(0.5) * (J0 + f[(6 + 3 * l) * n3p]), real(0.5) * (J1 + f[(7 + 3 * l) * n3p]),
                                 real(0.5) * (J2 + f[(8 + 3 * l) * n3p])};
             real F[NV];
-            ec_flux(W[0], ua, real(0.5) * W[0] / W[4], H, f[0], ub, f[4 * n3p], f[5 * n3p], Jm, ph, F);
+            ec_flux(W[0], ua, dg_div(real(0.5) * W[0], W[4]), H, f[0], ub, f[4 * n3p], f[5 * n3p], Jm, ph, F);
 #pragma unroll
             for (int v = 0; v < NV; ++v) sm[v] += real(2) * d * F[v];
           } else {
@@ -1189,7 +1189,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(15 * n * n * n / 2) 
   }
   const real sj = sJ[(size_t)e * n3 + node];
   if ((wp & 3) == 3) {  // the primitive variables as cons_to_prim forms them: warps 3, 7, 11
-    const real ir = real(1) / Uo[0];
+    const real ir = dg_rcp(Uo[0]);
     const real u = Uo[1] * ir, vv = Uo[2] * ir, w = Uo[3] * ir;
     if (wp == 3) {
       sW[1 * n3p + pn] = u;
@@ -1360,7 +1360,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(15 * n * n * n / 2) 
           tau[c] = ph.mu * (Gn[(d * 5 + 1 + c) * n3p] + Gn[(c * 5 + 1 + d) * n3p]);
           if (c == d) tau[c] -= real(2.0 / 3.0) * ph.mu * div;
         }
-        const real ir = real(1) / Wn[0];
+        const real ir = dg_rcp(Wn[0]);
         const real dT = (Gn[(d * 5 + 4) * n3p] - p * ir * Gn[(d * 5 + 0) * n3p]) * ir;
         const real fv4 = tau[0] * Wn[1] + tau[1] * Wn[2] + tau[2] * Wn[3] + ph.lam_th * dT;
         F = ud * (Uo[4] + p) - fv4;
@@ -1452,7 +1452,7 @@ __global__ void __launch_bounds__(128, sizeof(real) == 4 ? 8 : 1) k_face(const r
   for (int d = 0; d < 3; ++d) nv[d] = fgeo[((size_t)side * 4 + d) * n2 + pq];
   const real sa = fgeo[((size_t)side * 4 + 3) * n2 + pq];
   real f[NV], fl[NV], fr[NV];
-  const real irL = real(1) / WL[0], irR = real(1) / WR[0];  // shared by the Riemann and viscous fluxes
+  const real irL = dg_rcp(WL[0]), irR = dg_rcp(WR[0]);  // shared by the Riemann and viscous fluxes
   riemann_kind<RS>(WL, WR, irL, irR, nv, ph, f);
   visc_normal(WL, irL, GL, nv, ph, fl);
   visc_normal(WR, irR, GR, nv, ph, fr);
@@ -1495,7 +1495,7 @@ __global__ void __launch_bounds__(128) k_face3(const real* __restrict__ Wf, cons
       else
         roe_central(WL, WR, nv, ph, out);
     } else {
-      riemann_kind<RS>(WL, WR, real(1) / WL[0], real(1) / WR[0], nv, ph, out);
+      riemann_kind<RS>(WL, WR, dg_rcp(WL[0]), dg_rcp(WR[0]), nv, ph, out);
     }
   } else {
     // role 1: the master (slot 0) side, role 2: the slave or boundary (slot 1) side,
@@ -1507,7 +1507,7 @@ __global__ void __launch_bounds__(128) k_face3(const real* __restrict__ Wf, cons
     const int gslot = bnd ? 0 : slot;
 #pragma unroll
     for (int c = 0; c < 15; ++c) Gx[c] = Gf[((size_t)(gslot * S + side) * 15 + c) * n2 + pq];
-    visc_normal(Wx, real(1) / Wx[0], Gx, nv, ph, out);
+    visc_normal(Wx, dg_rcp(Wx[0]), Gx, nv, ph, out);
   }
 #pragma unroll
   for (int v = 0; v < NV; ++v) sf[role][v][lane] = out[v];
@@ -1717,7 +1717,7 @@ __global__ void __launch_bounds__(384) k_surf_face(
         else
           roe_central(WL, WR, nv, ph, out);
       } else {
-        riemann_kind<RS>(WL, WR, real(1) / WL[0], real(1) / WR[0], nv, ph, out);
+        riemann_kind<RS>(WL, WR, dg_rcp(WL[0]), dg_rcp(WR[0]), nv, ph, out);
       }
     } else {
       const int slot = role - 1;  // master, slave or boundary side (inner gradients on a boundary)
@@ -1727,7 +1727,7 @@ __global__ void __launch_bounds__(384) k_surf_face(
       const int gslot = bnd ? 0 : slot;
 #pragma unroll
       for (int c = 0; c < 15; ++c) Gx[c] = Gf[((size_t)(gslot * S + side) * 15 + c) * n2 + mpq];
-      visc_normal(Wx, real(1) / Wx[0], Gx, nv, ph, out);
+      visc_normal(Wx, dg_rcp(Wx[0]), Gx, nv, ph, out);
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) sf[role][v][fn] = out[v];
@@ -1876,7 +1876,7 @@ __global__ void __launch_bounds__(384) k_surf_face2(
         else
           roe_central(WL, WR, nv, ph, out);
       } else {
-        riemann_kind<RS>(WL, WR, real(1) / WL[0], real(1) / WR[0], nv, ph, out);
+        riemann_kind<RS>(WL, WR, dg_rcp(WL[0]), dg_rcp(WR[0]), nv, ph, out);
       }
     } else {
       const int slot = role - 1;
@@ -1886,7 +1886,7 @@ __global__ void __launch_bounds__(384) k_surf_face2(
       const int gslot = bnd ? 0 : slot;
 #pragma unroll
       for (int c = 0; c < 15; ++c) Gx[c] = Gf[((size_t)(gslot * S + side) * 15 + c) * n2 + mpq];
-      visc_normal(Wx, real(1) / Wx[0], Gx, nv, ph, out);
+      visc_normal(Wx, dg_rcp(Wx[0]), Gx, nv, ph, out);
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) sf[role][v][fh] = out[v];

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
       for (int c = 0; c < 9; ++c) mJ[c % 3] = max(mJ[c % 3], fx_mag(Ja[((size_t)e * 9 + c) * n3 + node]));
       sj = sJ[(size_t)e * n3 + node];
     }
-    cons_to_prim(Uo, W, ph);
+    cons_to_prim(Uo, 1.0 / Uo[0], W, ph);  // the FP64 pipe has room here: divisions stay on it
   }
   __syncthreads();
   int* mag = sMag + el * FX_SLOTS;
@@ -362,10 +362,11 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
       for (int v = 0; v < NV; ++v) Uo[v] = U[((size_t)e * NV + v) * n3 + node];
     }
     int mx[NV] = {0, 0, 0, 0, 0};
+    const double ir = 1.0 / Uo[0];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       double F[NV];
-      flux_total(Uo, W, G, d, ph, F);
+      flux_total(Uo, W, ir, G, d, ph, F);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         own[(d * NV + v) * n3p] = __double_as_longlong(F[v]);
