@@ -49,6 +49,7 @@ struct flexi_ctx {
   double* partial = nullptr;
   double* partial_host = nullptr;
   int red_blocks = 0;
+  unsigned* red_arrived = nullptr;  // blocks of the reduction that are done
   void *Ustate = nullptr, *dUstate = nullptr;
   void* adj_scratch = nullptr;
   Ops<double> ops64{};
@@ -669,8 +670,9 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   }
   c->Ustate = Us; c->dUstate = dUs;
   c->red_blocks = std::max(1, std::min(4 * 152, (int)(((size_t)K * n3 + 255) / 256)));
-  AL(c->partial, (size_t)c->red_blocks * kReduceQuantities);
-  if (cudaMallocHost(&c->partial_host, sizeof(double) * c->red_blocks * kReduceQuantities) != cudaSuccess)
+  AL(c->partial, (size_t)(c->red_blocks + 1) * kReduceQuantities + 1);  // results and status word, then the blocks' sums
+  AL(c->red_arrived, 1);
+  if (cudaMallocHost(&c->partial_host, sizeof(double) * (kReduceQuantities + 1)) != cudaSuccess)
     return FLEXI_ENOMEM;
   CK(cudaStreamSynchronize(st));
 #undef AL
@@ -712,17 +714,11 @@ flexi_status do_reduce(flexi_ctx* c, const void* U, const void* Ut, double cfl, 
   {
     Prof pr(c, KC_RED, st);
     CK(launch_reduce<real>((const real*)U, (const real*)Ut, c->wJ, c->Ja64, c->sJ64, (long long)c->K * c->n3, c->n3,
-                           ph_of<real>(c), kv, c->partial, c->red_blocks, st));
+                           ph_of<real>(c), kv, c->partial, c->red_blocks, c->status, c->red_arrived, st));
   }
-  CK(cudaMemcpyAsync(c->partial_host, c->partial, sizeof(double) * c->red_blocks * kReduceQuantities,
-                     cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(c->partial_host, c->partial, sizeof(double) * (kReduceQuantities + 1), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  double acc[kReduceQuantities] = {0};
-  for (int b = 0; b < c->red_blocks; ++b)
-    for (int q = 0; q < kReduceQuantities; ++q) {
-      const double val = c->partial_host[b * kReduceQuantities + q];
-      if (q < 7) acc[q] += val; else acc[q] = std::max(acc[q], val);
-    }
+  const double* acc = c->partial_host;
   for (int q = 0; q < 7; ++q) out[q] = acc[q];
   const int N = c->N;
   const double dtc = cfl * 2.0 / ((2.0 * N + 1.0) * acc[7]);
@@ -997,9 +993,7 @@ flexi_status flexi_reduce(flexi_ctx* c, const void* U, const void* Ut, double cf
   cudaStream_t st = (cudaStream_t)stream;
   const flexi_status s = c->fp64 ? do_reduce<double>(c, U, Ut, cfl, out, st) : do_reduce<float>(c, U, Ut, cfl, out, st);
   if (s != FLEXI_OK) return s;
-  unsigned flag = 0;
-  CK(cudaMemcpy(&flag, c->status, sizeof(unsigned), cudaMemcpyDeviceToHost));
-  if (flag) {
+  if (c->partial_host[kReduceQuantities] != 0.0) {  // the status word, read by the reduction
     CK(cudaMemset(c->status, 0, sizeof(unsigned)));
     return FLEXI_ENONPHYSICAL;
   }

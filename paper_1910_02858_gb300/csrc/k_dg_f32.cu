@@ -16,5 +16,6 @@ template cudaError_t launch_mortar_flux<float>(const DevMesh&, const MortarOps<f
 template cudaError_t launch_surf<float>(const DevMesh&, int, float*, float*, float*, const RkStage<float>&,
                                        const SourceParams&, const Ops<float>&, const Phys<float>&, cudaStream_t);
 template cudaError_t launch_reduce<float>(const float*, const float*, const double*, const double*, const double*,
-                                         long long, int, const Phys<float>&, double, double*, int, cudaStream_t);
+                                         long long, int, const Phys<float>&, double, double*, int, const unsigned*, unsigned*,
+                                         cudaStream_t);
 }  // namespace flexi

@@ -16,7 +16,8 @@ template cudaError_t launch_mortar_flux<double>(const DevMesh&, const MortarOps<
 template cudaError_t launch_surf<double>(const DevMesh&, int, double*, double*, double*, const RkStage<double>&,
                                        const SourceParams&, const Ops<double>&, const Phys<double>&, cudaStream_t);
 template cudaError_t launch_reduce<double>(const double*, const double*, const double*, const double*, const double*,
-                                         long long, int, const Phys<double>&, double, double*, int, cudaStream_t);
+                                         long long, int, const Phys<double>&, double, double*, int, const unsigned*, unsigned*,
+                                         cudaStream_t);
 
 cudaError_t launch_surf_face(const DevMesh& m, const void* WfIn, void* WfOut, double* U, double* dU,
                                     const RkStage<double>& rk, const SourceParams& src,

@@ -106,7 +106,7 @@ cudaError_t launch_axpby(real* y, const real* x, real a, real b, size_t count, c
 template <typename real>
 cudaError_t launch_reduce(const real* U, const real* Ut, const double* wJ, const double* Ja64, const double* sJ64,
                           long long nodes, int n3, const Phys<real>& ph, double kv_coef, double* partial,
-                          int nblocks, cudaStream_t st);
+                          int nblocks, const unsigned* status, unsigned* arrived, cudaStream_t st);
 constexpr int kReduceQuantities = 9;
 }  // namespace flexi
 struct flexi_ctx;
