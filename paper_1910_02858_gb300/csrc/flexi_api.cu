@@ -339,6 +339,44 @@ void fill_mortar_ops(MortarOps<real>& o, const std::vector<double>& x, const std
   }
 }
 
+// Metric terms Ja^l_d (l*3+d) and 1/J of an element whose mapping is affine to within the
+// rounding of its coordinates: x [ng^3][3] at the tensor product of the points xg
+bool affine_metrics(const double* x, const std::vector<double>& xg, int ng, double* out) {
+  const int last = ng - 1;
+  auto at = [&](int i, int j, int k, int d) { return x[((k * ng + j) * ng + i) * 3 + d]; };
+  double a[3][3], size = 0.0;  // a[l] = dx / dxi_l: mean of the four parallel edges over 2
+  for (int d = 0; d < 3; ++d) {
+    for (int l = 0; l < 3; ++l) a[l][d] = 0.0;
+    for (int p = 0; p < 2; ++p)
+      for (int q = 0; q < 2; ++q) {
+        a[0][d] += (at(last, p * last, q * last, d) - at(0, p * last, q * last, d)) * 0.125;
+        a[1][d] += (at(p * last, last, q * last, d) - at(p * last, 0, q * last, d)) * 0.125;
+        a[2][d] += (at(p * last, q * last, last, d) - at(p * last, q * last, 0, d)) * 0.125;
+      }
+  }
+  for (int d = 0; d < 3; ++d) {
+    double s = std::fabs(at(0, 0, 0, d));
+    for (int l = 0; l < 3; ++l) s += 2.0 * std::fabs(a[l][d]);
+    size = std::max(size, s);
+  }
+  const double tol = 16.0 * 2.220446049250313e-16 * size;  // a few units of the coordinates' rounding
+  for (int k = 0; k < ng; ++k)
+    for (int j = 0; j < ng; ++j)
+      for (int i = 0; i < ng; ++i)
+        for (int d = 0; d < 3; ++d) {
+          const double y = at(0, 0, 0, d) + (xg[i] + 1.0) * a[0][d] + (xg[j] + 1.0) * a[1][d] + (xg[k] + 1.0) * a[2][d];
+          if (!(std::fabs(at(i, j, k, d) - y) <= tol)) return false;
+        }
+  for (int l = 0; l < 3; ++l) {
+    const double *u = a[(l + 1) % 3], *v = a[(l + 2) % 3];
+    for (int d = 0; d < 3; ++d) out[l * 3 + d] = u[(d + 1) % 3] * v[(d + 2) % 3] - u[(d + 2) % 3] * v[(d + 1) % 3];
+  }
+  const double J = a[0][0] * out[0] + a[0][1] * out[1] + a[0][2] * out[2];
+  if (!(J > 0.0)) return false;
+  out[9] = 1.0 / J;
+  return true;
+}
+
 flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const double* coords, const int32_t* conn,
                             int M, const int32_t* mortars, cudaStream_t st) {
   if (cudaGetDevice(&c->device) != cudaSuccess) return FLEXI_ECUDA;
@@ -594,6 +632,42 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   CK(interp3(X0r, Xr, dVg2s, 3 * K, ng));
   for (int l = 0; l < 3; ++l) CK(geom_apply1d(Xr, dX[l], dDs, 3 * K, n, n, n, l, n, st));
   CK(geom_jacobian(dX, c->sJ64, c->wJ, wdev, K, n, c->status, st));
+  // affine elements: constant metric terms from the edge vectors (their differences from the
+  // derivatives above are the coordinates' rounding), where the lifting kernel has a variant
+  // for such elements (launch_lift_vol: not the small-mesh kernels, BR2 or split forms)
+  int nsm = 1;
+  CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+  if (c->fp64 && p->lifting == FLEXI_LIFTING_BR1 && p->split_form == FLEXI_SPLIT_STANDARD && !(n <= 4 && K < nsm)) {
+    std::vector<double> aff((size_t)K * 10, 0.0);
+    std::vector<int> flag(K, 0);
+    for (int e = 0; e < K; ++e) flag[e] = affine_metrics(coords + (size_t)e * ng3 * 3, xg, ng, &aff[(size_t)e * 10]) ? 1 : 0;
+    double* daff;
+    AL(daff, aff.size());
+    int* dflag;
+    AL(dflag, flag.size());
+    CK(cudaMemcpyAsync(daff, aff.data(), aff.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+    CK(cudaMemcpyAsync(dflag, flag.data(), flag.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+    CK(geom_affine(daff, dflag, c->Ja64, c->sJ64, c->wJ, wdev, K, n, st));
+    CK(cudaStreamSynchronize(st));
+    c->m.affine = daff;
+    // groups of elements per CTA, affine ones first (a big side's lifting flux is not a face mean)
+    for (int m2 = 0; m2 < M; ++m2) flag[mortars[15 * m2]] = 0;
+    const int ne = n3 >= 64 ? 1 : (64 + n3 - 1) / n3, groups = (K + ne - 1) / ne;  // Cfg<n>::NE
+    std::vector<int> order;
+    order.reserve(groups);
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int g = 0; g < groups; ++g) {
+        bool all = true;
+        for (int e = g * ne; e < std::min(K, (g + 1) * ne); ++e) all = all && flag[e];
+        if (all == (pass == 0)) order.push_back(g);
+      }
+      if (pass == 0) c->m.nAffine = (int)order.size();
+    }
+    int* dorder;
+    AL(dorder, order.size());
+    CK(cudaMemcpy(dorder, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
+    c->m.order = dorder;
+  }
   CK(geom_faces(c->Ja64, X, sideM, dlm, dlp, c->fgeo64, c->xbc, S, c->nBC, n, st));
   if (p->source) {
     unsigned char* phase;

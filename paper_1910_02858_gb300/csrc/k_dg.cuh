@@ -2023,15 +2023,31 @@ template <int n, bool LGL>
 static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double>& ops, const Phys<double>& ph,
                              int store_grad, cudaStream_t st, int volume = 1) {
   using C = Cfg<n>;
-  constexpr size_t smem = lift_fx_smem<n>();
-  auto* kernel = &k_lift_vol_fx<n, LGL>;
-  static std::atomic<unsigned long long> attr{0};
-  cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
-  if (err != cudaSuccess) return err;
-  kernel<<<(m.K + C::NE - 1) / C::NE, C::T, smem, st>>>(
-      U, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf, (const double*)m.fgeo, m.elemSide,
-      (double*)m.Gf, volume ? (double*)m.Utv : nullptr, store_grad ? (double*)m.Gvol : nullptr, m.K, m.S, m.Sface,
-      (const double*)m.QB, ops, m.fx, ph);
+  double* Utv = volume ? (double*)m.Utv : nullptr;
+  double* Gvol = store_grad ? (double*)m.Gvol : nullptr;
+  const int groups = (m.K + C::NE - 1) / C::NE;
+  if (m.nAffine > 0) {
+    constexpr size_t smem = lift_affine_smem_total<n>();
+    auto* kernel = &k_lift_vol_fx_affine<n, LGL>;
+    static std::atomic<unsigned long long> attr{0};
+    cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
+    if (err != cudaSuccess) return err;
+    kernel<<<m.nAffine, C::T, smem, st>>>(U, m.affine, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
+                                          (const double*)m.fgeo, m.elemSide, (double*)m.Gf, Utv, Gvol, m.K, m.S, m.Sface,
+                                          m.nAffine < groups ? m.order : nullptr, ops, m.fx, ph);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  if (m.nAffine < groups) {
+    constexpr size_t smem = lift_fx_smem<n>();
+    auto* kernel = &k_lift_vol_fx<n, LGL>;
+    static std::atomic<unsigned long long> attr{0};
+    cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
+    if (err != cudaSuccess) return err;
+    kernel<<<groups - m.nAffine, C::T, smem, st>>>(U, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
+                                                   (const double*)m.fgeo, m.elemSide, (double*)m.Gf, Utv, Gvol, m.K, m.S,
+                                                   m.Sface, (const double*)m.QB,
+                                                   m.nAffine > 0 ? m.order + m.nAffine : nullptr, ops, m.fx, ph);
+  }
   return cudaGetLastError();
 }
 

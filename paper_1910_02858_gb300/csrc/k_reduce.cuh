@@ -31,10 +31,10 @@ __device__ __forceinline__ void reduce_block(double (*red)[RED_T]) {
 // roots and 30 products), and only nodes whose upper bound reaches the block's largest lower
 // bound so far are evaluated in FP64 (100 operations): the maximum is the same value.  The
 // last block adds up the blocks' results in block order and puts the status word behind
-// them, so that one copy of 10 values reaches the host.  16^3, N = 7: 382 -> 231 us for the
-// kernel (HBM: 53 us), 429 -> 257 us for the call.
+// them, so that one copy of 10 values reaches the host.  16^3, N = 7: 382 -> 216 us for the
+// kernel (HBM: 53 us), 429 -> 240 us for the call.
 template <typename real>
-__global__ void __launch_bounds__(RED_T) k_reduce(const real* __restrict__ U, const real* __restrict__ Ut,
+__global__ void __launch_bounds__(RED_T, 4) k_reduce(const real* __restrict__ U, const real* __restrict__ Ut,
                                                  const double* __restrict__ wJ, const double* __restrict__ Ja64,
                                                  const double* __restrict__ sJ64, double* __restrict__ partial,
                                                  long long nodes, int n3, Phys<real> ph, double kv_coef,

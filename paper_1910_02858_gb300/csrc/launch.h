@@ -53,6 +53,12 @@ struct DevMesh {
   const int* mvirt = nullptr;  // [nV] int4 (big side, type | a<<2 | b<<3, o, oinv)
   const int* mbig = nullptr;   // [nBig][8] (type, virtual side of position 0..3 or -1)
   void* QB = nullptr;          // [nBig][15][n^2] BR1 lifting flux of the big element
+  // Affine elements (parallelepipeds without a mortar big side): their constant metric terms
+  // and 1/J, and the order in which the lifting kernels take the CTAs' element groups
+  // (Cfg<n>::NE consecutive elements): nAffine groups of affine elements, then the others
+  const double* affine = nullptr;  // [K][10] Ja^l_d at l*3+d, 1/J
+  const int* order = nullptr;      // [groups]
+  int nAffine = 0;
   FxOps fx{};                  // fixed-point line operators (FP64 form)
   unsigned* status = nullptr;  // device status word (bit 0: non-physical face state)
 };
@@ -136,6 +142,9 @@ cudaError_t geom_jacobian(const double* const dX[3], double* sJ, double* wJ, con
                           unsigned* bad, cudaStream_t st);
 cudaError_t geom_faces(const double* Ja, const double* X, const int* sideMaster, const double* lm,
                        const double* lp, double* fgeo, double* xbc, int S, int nBC, int n, cudaStream_t st);
+// constant metric terms of affine elements (flag[e] != 0): Ja, 1/J and the quadrature weights
+cudaError_t geom_affine(const double* aff, const int* flag, double* Ja, double* sJ, double* wJ, const double* w, int K, int n,
+                        cudaStream_t st);
 // sine and cosine of pi (x + y + z) at the solution nodes, [K][2][n^3]
 cudaError_t geom_phase(const double* X, void* phase, bool fp64, int K, int n3, cudaStream_t st);
 cudaError_t convert_f64_to_f32(const double* in, float* out, size_t count, cudaStream_t st);
