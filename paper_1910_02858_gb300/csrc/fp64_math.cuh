@@ -2,7 +2,8 @@
 // narrow (an FP64 warp instruction holds its sub-partition for 64 clocks, a division or a
 // square root 8-10 of them): one third-order Newton step on 62-bit integers from an FP32
 // seed, about 45-55 integer instructions.  Used where the FP64 pipe sets the time: HLLC
-// k_face at 16^3, N = 7: 238 -> 181 FP64 instructions per face node, 354 -> 275 us.  Results are within 0.52 units in the last place;
+// k_face at 16^3, N = 7: 238 -> 181 FP64 instructions per face node, 354 -> 275 us (then 226 with
+// fx_visc_normal).  Results are within 0.52 units in the last place;
 // zero, subnormal and very large arguments, infinities, NaN and negative radicands take the
 // language's operation.
 #pragma once

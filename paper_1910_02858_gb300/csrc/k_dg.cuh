@@ -1454,8 +1454,14 @@ __global__ void __launch_bounds__(128, sizeof(real) == 4 ? 8 : 1) k_face(const r
   real f[NV], fl[NV], fr[NV];
   const real irL = dg_rcp(WL[0]), irR = dg_rcp(WR[0]);  // shared by the Riemann and viscous fluxes
   riemann_kind<RS>(WL, WR, irL, irR, nv, ph, f);
-  visc_normal(WL, irL, GL, nv, ph, fl);
-  visc_normal(WR, irR, GR, nv, ph, fr);
+  if constexpr (sizeof(real) == 8) {
+    const FxNormal q = fx_normal(nv);
+    fx_visc_normal(WL, irL, GL, nv, q, ph, fl);
+    fx_visc_normal(WR, irR, GR, nv, q, ph, fr);
+  } else {
+    visc_normal(WL, irL, GL, nv, ph, fl);
+    visc_normal(WR, irR, GR, nv, ph, fr);
+  }
 #pragma unroll
   for (int v = 0; v < NV; ++v) Ff[((size_t)side * NV + v) * n2 + pq] = (f[v] - real(0.5) * (fl[v] + fr[v])) * sa;
 }
