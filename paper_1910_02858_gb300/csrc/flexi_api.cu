@@ -513,6 +513,7 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   fill_ops<double>(c->ops64, Ds, ws, lmv, lpv, n);
   fill_ops<float>(c->ops32, Ds, ws, lmv, lpv, n);
   c->m.fx = make_fx_ops(c->ops64, n);
+  c->m.fxT = make_fx_ops_transposed(c->ops64, n);
   fill_mortar_ops<double>(c->mops64, xs, ws, n);
   fill_mortar_ops<float>(c->mops32, xs, ws, n);
   fill_phys<double>(c->ph64, *p);

@@ -98,6 +98,20 @@ inline FxOps make_fx_ops(const Ops<double>& o, int n) {
   return f;
 }
 
+// the transposed operators: Dhat^T as the line contraction, l_hat(+-1) as the end values and
+// l(+-1) as the values spread from the ends (lh, ll)
+inline FxOps make_fx_ops_transposed(const Ops<double>& o, int n) {
+  Ops<double> t = o;
+  for (int i = 0; i < n; ++i) {
+    for (int a = 0; a < n; ++a) t.DhatT[a * n + i] = o.DhatT[i * n + a];
+    t.lm[i] = o.lhm[i];
+    t.lp[i] = o.lhp[i];
+    t.lhm[i] = o.lm[i];
+    t.lhp[i] = o.lp[i];
+  }
+  return make_fx_ops(t, n);
+}
+
 // ---------------------------------------------------------------------------
 // device primitives
 // ---------------------------------------------------------------------------
@@ -287,6 +301,47 @@ __device__ __forceinline__ void fx_visc_normal(const double W[NV], const double 
   f[2] = tn[1];
   f[3] = tn[2];
   f[4] = tn[0] * W[1] + tn[1] * W[2] + tn[2] * W[3] + ph.lam_th * dTn * ir;
+}
+
+// fx_line without face terms, and the line's end values as fx_ends
+template <int n>
+__device__ __forceinline__ void fx_line_ends(fx64* __restrict__ p, int stride, const FxOps& o, fx64& ym, fx64& yp) {
+  constexpr int h = n / 2, c = (n + 1) / 2, N = n - 1;
+  FxSplit e[c], d[h];
+#pragma unroll
+  for (int a = 0; a < h; ++a) {
+    const fx64 x = p[a * stride], y = p[(N - a) * stride];
+    e[a] = fx_split(x + y);
+    d[a] = fx_split(x - y);
+  }
+  if constexpr (n & 1) e[c - 1] = fx_split(p[(c - 1) * stride]);
+  {
+    FxAcc se, sd;
+#pragma unroll
+    for (int a = 0; a < c; ++a) se.add(e[a], o.peh[a], o.pel[a]);
+#pragma unroll
+    for (int a = 0; a < h; ++a) sd.add(d[a], o.poh[a], o.pol[a]);
+    const fx64 E = se.get(), D = sd.get();
+    yp = E + D;
+    ym = E - D;
+  }
+#pragma unroll
+  for (int i = 0; i < c; ++i) {
+    FxAcc so;
+#pragma unroll
+    for (int a = 0; a < h; ++a) so.add(d[a], o.oh[i][a], o.ol[i][a]);
+    const fx64 O = so.get();
+    if (i < h) {
+      FxAcc se;
+#pragma unroll
+      for (int a = 0; a < c; ++a) se.add(e[a], o.eh[i][a], o.el[i][a]);
+      const fx64 E = se.get();
+      p[i * stride] = O + E;
+      p[(N - i) * stride] = O - E;
+    } else {
+      p[i * stride] = O;
+    }
+  }
 }
 
 // Largest magnitude words of n fields over the threads of an element: get(s) is the

@@ -867,11 +867,11 @@ constexpr size_t adj_vol_smem(bool br2, bool split) {
 // pair (each node collects d/dW of both ordered pairs it takes part in) and the
 // strong-form face terms at the line ends.
 template <typename real, int n, bool BR2, int SPLIT>
-__global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
+__device__ __forceinline__ void adj_vol_body(
     const real* __restrict__ U, const real* __restrict__ Ja, const real* __restrict__ sJ, const real* __restrict__ Gvol,
     const real* __restrict__ fgeo, const int* __restrict__ elemSide, const real* __restrict__ lam,
     const real* __restrict__ LGf, real* __restrict__ LWs, real* __restrict__ LWf, real* __restrict__ muv, int K, int S,
-    int bigBase, real* __restrict__ LQB, Ops<real> ops, Phys<real> ph) {
+    int bigBase, real* __restrict__ LQB, const Ops<real>& ops, const Phys<real>& ph, int grp) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
   int* sES = reinterpret_cast<int*>(sWJ + (SPLIT ? NE * 15 * n3 : 0));
   const int tid = threadIdx.x;
   const int el = tid / n3, node = tid - el * n3;
-  const int e0 = blockIdx.x * NE;
+  const int e0 = grp * NE;
   const int e = e0 + el;
   const bool valid = e < K;
   const int i = node % n, j = (node / n) % n, k = node / n2;
@@ -1146,6 +1146,16 @@ __global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
   }
 }
 
+template <typename real, int n, bool BR2, int SPLIT>
+__global__ void __launch_bounds__(Cfg<n>::T) k_adj_vol(
+    const real* __restrict__ U, const real* __restrict__ Ja, const real* __restrict__ sJ, const real* __restrict__ Gvol,
+    const real* __restrict__ fgeo, const int* __restrict__ elemSide, const real* __restrict__ lam,
+    const real* __restrict__ LGf, real* __restrict__ LWs, real* __restrict__ LWf, real* __restrict__ muv, int K, int S,
+    int bigBase, real* __restrict__ LQB, Ops<real> ops, Phys<real> ph) {
+  adj_vol_body<real, n, BR2, SPLIT>(U, Ja, sJ, Gvol, fgeo, elemSide, lam, LGf, LWs, LWf, muv, K, S, bigBase, LQB, ops, ph,
+                                    blockIdx.x);
+}
+
 // side: BR1 mean and the primitive map of the face states -> adjoint of U_face.
 // Boundary sides: the adjoint of the outer state W_R = B(W_L) (flux and lifting
 // mean) is added to the inner one through B^T (exact state: B = 0; outflow:
@@ -1275,6 +1285,10 @@ __global__ void k_axpby(real* __restrict__ y, const real* __restrict__ x, real a
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx < count) y[idx] = a * y[idx] + (x ? b * x[idx] : real(0));
 }
+
+}  // namespace flexi
+#include "k_adj_fx.cuh"
+namespace flexi {
 
 // ---------------------------------------------------------------------------
 // mortars: transposes of the interpolation and the projections (k_mortar.cuh)
@@ -1521,6 +1535,10 @@ static cudaError_t rhs_adjoint_n(const DevMesh& m, const real* U, const real* la
     if ((err = launch_adj_vol<real, n, false, 1>(m, U, lam, a, ops, ph, grid, st)) != cudaSuccess) return err;
   } else if (m.split == 2) {
     if ((err = launch_adj_vol<real, n, false, 2>(m, U, lam, a, ops, ph, grid, st)) != cudaSuccess) return err;
+  } else if constexpr (sizeof(real) == 8) {
+    if ((err = launch_adj_vol_fx<n>(m, U, lam, (const double*)a.LGf, (double*)a.LWs, (double*)a.LWf, (double*)a.muv,
+                                    (double*)a.LQB, ops, ph, st)) != cudaSuccess)
+      return err;
   } else {
     if ((err = launch_adj_vol<real, n, false, 0>(m, U, lam, a, ops, ph, grid, st)) != cudaSuccess) return err;
   }

@@ -60,6 +60,7 @@ struct DevMesh {
   const int* order = nullptr;      // [groups]
   int nAffine = 0;
   FxOps fx{};                  // fixed-point line operators (FP64 form)
+  FxOps fxT{};                 // and their transposes (adjoint)
   unsigned* status = nullptr;  // device status word (bit 0: non-physical face state)
 };
 

@@ -92,3 +92,55 @@ def test_wide_ranges_within_an_element():
     a, c = _rhs(mesh, 7, 0, U, 0), _rhs(mesh, 7, 0, U, 120)
     for v in range(5):
         assert np.abs(a[:, v] - c[:, v]).max() <= tol[v], v
+
+
+def _adjoint(mesh, N, nodes, U, lam, b, riemann, mu=0.01):
+    import torch
+
+    from paper_1910_02858_gb300 import Solver, SolverConfig
+
+    f = 2.0 ** b
+    s = Solver(SolverConfig(N=N, Ngeo=mesh.Ngeo, node_type=nodes, riemann=riemann, mu=mu * f, adjoint=True), mesh.coords,
+               mesh.conn)
+    scale = np.array([1.0, f, f, f, f * f]).reshape(1, 5, 1, 1, 1)
+    t = lambda a: torch.tensor(a, device="cuda:0")
+    # U_t' = f S L(U) for U' = S U, so the transpose maps S^-1 lam to f S^-1 (dL/dU)^T lam
+    out = s.rhs_adjoint(t(U * scale), t(lam / scale), 0.0).cpu().numpy()
+    s.close()
+    return out * scale / f
+
+
+@pytest.mark.parametrize("mapping", ["cartesian", "mixed"])
+@pytest.mark.parametrize("N", [2, 4, 5, 6, 7])
+def test_adjoint_matches_fp64_body(N, mapping):
+    """The reverse kernel's fixed-point contractions against its FP64 body.  The transposed sums have the terms of
+    the forward ones, at most 4 (N + 3) roundings deeper (the pointwise derivatives), on random unit-size adjoints:
+    the same bound with max|F| replaced by the largest flux derivative, |u| + c times the largest column."""
+    from paper_1910_02858_gb300 import flexi as F
+
+    mesh, U, tol = _case(N, 0, mapping)
+    lam = np.random.default_rng(N).standard_normal(U.shape)
+    a, c = (_adjoint(mesh, N, 0, U, lam, b, F.RIEMANN_RUSANOV) for b in (0, 120))
+    assert np.abs(a - c).max() <= 4 * tol.max() * np.abs(lam).max() * np.abs(U).max()
+
+
+@pytest.mark.parametrize("riemann", ["hllc", "rusanov"])
+@pytest.mark.parametrize("speed", [0.4, 3.0])
+def test_flux_reverses_match_oracle(riemann, speed):
+    """Hand-written HLLC and Rusanov reverses on subsonic and supersonic faces of both directions (1e-10, the bar of
+    the adjoint against the oracle's reverse mode)."""
+    import torch
+
+    from oracle.dgsem import DGSEM, HLLC, RUSANOV, Params
+    from paper_1910_02858_gb300 import flexi as F
+
+    mesh = wl.box_mesh((2, 2, 2), reorient_seed=7)
+    U = wl.perturbed(mesh.node_coords(3, 0), seed=11, Ma=1.0)
+    rho = U[:, :1]
+    m = U[:, 1:4] + speed * rho * np.array([1.0, -0.7, 0.5]).reshape(1, 3, 1, 1, 1)
+    U = np.concatenate([rho, m, U[:, 4:] + 0.5 * (m ** 2 - U[:, 1:4] ** 2).sum(1, keepdims=True) / rho], axis=1)
+    lam = np.random.default_rng(5).standard_normal(U.shape)
+    out = _adjoint(mesh, 3, 0, U, lam, 0, F.RIEMANN_HLLC if riemann == "hllc" else F.RIEMANN_RUSANOV)
+    dg = DGSEM(Params(N=3, node_type=0, riemann=HLLC if riemann == "hllc" else RUSANOV, mu=0.01), mesh.coords, mesh.conn)
+    ref = dg.rhs_vjp(torch.tensor(U), 0.0, torch.tensor(lam)).numpy()
+    assert np.linalg.norm(out - ref) <= 1e-10 * np.linalg.norm(ref)
