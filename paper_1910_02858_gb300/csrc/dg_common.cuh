@@ -158,6 +158,19 @@ __device__ __forceinline__ void flux_total(const real U[NV], const real W[NV], c
   flux_total(U, W, dg_rcp(W[0]), G, d, ph, F);
 }
 
+// viscous flux F^v_d (its first component is zero)
+template <typename real>
+__device__ __forceinline__ void flux_viscous(const real W[NV], const real ir, const real G[15], int d, const Phys<real>& ph,
+                                             real F[NV]) {
+  const real div = G[0 * 5 + 1] + G[1 * 5 + 2] + G[2 * 5 + 3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) F[1 + c] = ph.mu * (G[d * 5 + 1 + c] + G[c * 5 + 1 + d]);
+  F[1 + d] -= real(2.0 / 3.0) * ph.mu * div;
+  const real dT = (G[d * 5 + 4] - W[4] * ir * G[d * 5 + 0]) * ir;
+  F[0] = real(0);
+  F[4] = F[1] * W[1] + F[2] * W[2] + F[3] * W[3] + ph.lam_th * dT;
+}
+
 // normal viscous flux F^v . n, with ir = 1 / rho of the state
 template <typename real>
 __device__ __forceinline__ void visc_normal(const real W[NV], const real ir, const real G[15], const real n[3],

@@ -49,7 +49,6 @@ struct flexi_ctx {
   double* partial = nullptr;
   double* partial_host = nullptr;
   int red_blocks = 0;
-  unsigned* red_arrived = nullptr;  // blocks of the reduction that are done
   void *Ustate = nullptr, *dUstate = nullptr;
   void* adj_scratch = nullptr;
   Ops<double> ops64{};
@@ -513,6 +512,7 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   fill_ops<double>(c->ops64, Ds, ws, lmv, lpv, n);
   fill_ops<float>(c->ops32, Ds, ws, lmv, lpv, n);
   c->m.fx = make_fx_ops(c->ops64, n);
+  c->m.fxD = make_fx_strong(c->ops64, n);
   c->m.fxT = make_fx_ops_transposed(c->ops64, n);
   fill_mortar_ops<double>(c->mops64, xs, ws, n);
   fill_mortar_ops<float>(c->mops32, xs, ws, n);
@@ -533,7 +533,7 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   AL(c->xbc, (size_t)std::max(c->nBC, 1) * 3 * n2);
   AL(c->bcKind, (size_t)std::max(c->nBC, 1));  // zero: every boundary takes the exact state
   AL(c->elemSide, (size_t)K * 6);
-  AL(c->status, 1);
+  AL(c->status, 2);  // the status word, and the count of finished blocks of the reduction
 
   // ---- temporary geometry buffers
   std::vector<void*> tmp;
@@ -635,39 +635,45 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   CK(geom_jacobian(dX, c->sJ64, c->wJ, wdev, K, n, c->status, st));
   // affine elements: constant metric terms from the edge vectors (their differences from the
   // derivatives above are the coordinates' rounding), where the lifting kernel has a variant
-  // for such elements (launch_lift_vol: not the small-mesh kernels, BR2 or split forms)
+  // for such elements (launch_lift_vol: not BR2 or the entropy-conservative form) and the mesh is not one of the
+  // smallest, whose kernels read the metric terms per node
   int nsm = 1;
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-  if (c->fp64 && p->lifting == FLEXI_LIFTING_BR1 && p->split_form == FLEXI_SPLIT_STANDARD && !(n <= 4 && K < nsm)) {
-    std::vector<double> aff((size_t)K * 10, 0.0);
-    std::vector<int> flag(K, 0);
-    for (int e = 0; e < K; ++e) flag[e] = affine_metrics(coords + (size_t)e * ng3 * 3, xg, ng, &aff[(size_t)e * 10]) ? 1 : 0;
-    double* daff;
-    AL(daff, aff.size());
-    int* dflag;
-    AL(dflag, flag.size());
-    CK(cudaMemcpyAsync(daff, aff.data(), aff.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CK(cudaMemcpyAsync(dflag, flag.data(), flag.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    CK(geom_affine(daff, dflag, c->Ja64, c->sJ64, c->wJ, wdev, K, n, st));
-    CK(cudaStreamSynchronize(st));
-    c->m.affine = daff;
-    // groups of elements per CTA, affine ones first (a big side's lifting flux is not a face mean)
-    for (int m2 = 0; m2 < M; ++m2) flag[mortars[15 * m2]] = 0;
-    const int ne = n3 >= 64 ? 1 : (64 + n3 - 1) / n3, groups = (K + ne - 1) / ne;  // Cfg<n>::NE
-    std::vector<int> order;
-    order.reserve(groups);
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int g = 0; g < groups; ++g) {
-        bool all = true;
-        for (int e = g * ne; e < std::min(K, (g + 1) * ne); ++e) all = all && flag[e];
-        if (all == (pass == 0)) order.push_back(g);
-      }
-      if (pass == 0) c->m.nAffine = (int)order.size();
+  if (c->fp64 && p->lifting == FLEXI_LIFTING_BR1 && p->split_form != FLEXI_SPLIT_EC && !(n <= 4 && K < nsm)) {
+    std::vector<double> aff((size_t)K * 10, 0.0);  // 1/J = 0: not affine
+    std::vector<char> flag(K);
+    bool any = false;
+    for (int e = 0; e < K; ++e) {
+      flag[e] = affine_metrics(coords + (size_t)e * ng3 * 3, xg, ng, &aff[(size_t)e * 10]);
+      any = any || flag[e];
     }
-    int* dorder;
-    AL(dorder, order.size());
-    CK(cudaMemcpy(dorder, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
-    c->m.order = dorder;
+    if (any) {
+      double* daff;
+      AL(daff, aff.size());
+      CK(cudaMemcpyAsync(daff, aff.data(), aff.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+      CK(geom_affine(daff, c->Ja64, c->sJ64, c->wJ, wdev, K, n, st));
+      CK(cudaStreamSynchronize(st));
+      c->m.affine = daff;
+      // groups of elements per CTA, affine ones first (a big side's lifting flux is not a face mean)
+      for (int m2 = 0; m2 < M; ++m2) flag[mortars[15 * m2]] = 0;
+      const int ne = n3 >= 64 ? 1 : (64 + n3 - 1) / n3, groups = (K + ne - 1) / ne;  // Cfg<n>::NE
+      std::vector<int> order;
+      order.reserve(groups);
+      for (int pass = 0; pass < 2; ++pass) {
+        for (int g = 0; g < groups; ++g) {
+          bool all = true;
+          for (int e = g * ne; e < std::min(K, (g + 1) * ne); ++e) all = all && flag[e];
+          if (all == (pass == 0)) order.push_back(g);
+        }
+        if (pass == 0) c->m.nAffine = (int)order.size();
+      }
+      if (c->m.nAffine > 0 && c->m.nAffine < groups) {
+        int* dorder;
+        AL(dorder, order.size());
+        CK(cudaMemcpy(dorder, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice));
+        c->m.order = dorder;
+      }
+    }
   }
   CK(geom_faces(c->Ja64, X, sideM, dlm, dlp, c->fgeo64, c->xbc, S, c->nBC, n, st));
   if (p->source) {
@@ -746,7 +752,6 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   c->Ustate = Us; c->dUstate = dUs;
   c->red_blocks = std::max(1, std::min(4 * 152, (int)(((size_t)K * n3 + 255) / 256)));
   AL(c->partial, (size_t)(c->red_blocks + 1) * kReduceQuantities + 1);  // results and status word, then the blocks' sums
-  AL(c->red_arrived, 1);
   if (cudaMallocHost(&c->partial_host, sizeof(double) * (kReduceQuantities + 1)) != cudaSuccess)
     return FLEXI_ENOMEM;
   CK(cudaStreamSynchronize(st));
@@ -789,7 +794,7 @@ flexi_status do_reduce(flexi_ctx* c, const void* U, const void* Ut, double cfl, 
   {
     Prof pr(c, KC_RED, st);
     CK(launch_reduce<real>((const real*)U, (const real*)Ut, c->wJ, c->Ja64, c->sJ64, (long long)c->K * c->n3, c->n3,
-                           ph_of<real>(c), kv, c->partial, c->red_blocks, c->status, c->red_arrived, st));
+                           ph_of<real>(c), kv, c->partial, c->red_blocks, c->status, c->status + 1, st));
   }
   CK(cudaMemcpyAsync(c->partial_host, c->partial, sizeof(double) * (kReduceQuantities + 1), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));

@@ -38,6 +38,31 @@ struct FxOps {
   int kc, kp, kl;
 };
 
+// strong-form derivative D[i][a] at a*n + i, scale 2^k (split forms)
+struct FxStrong {
+  int h[MAXN * MAXN], l[MAXN * MAXN];
+  int k;
+};
+inline FxStrong make_fx_strong(const Ops<double>& o, int n) {
+  FxStrong f;
+  std::memset(&f, 0, sizeof(f));
+  double row = 0;
+  for (int i = 0; i < n; ++i) {
+    double s = 0;
+    for (int a = 0; a < n; ++a) s += std::fabs(o.DT[a * n + i]);
+    row = std::fmax(row, s);
+  }
+  int x;
+  std::frexp(row * (1 + 1e-12), &x);
+  f.k = 62 - x;
+  for (int t = 0; t < n * n; ++t) {
+    const long long v = std::llrint(std::ldexp(o.DT[t], f.k));
+    f.l[t] = (int)(unsigned)(v & 0xffffffffll);
+    f.h[t] = (int)((v - f.l[t]) / (1ll << 32));
+  }
+  return f;
+}
+
 // host construction from the FP64 operators (integer rounding of scaled doubles: the
 // same on every machine)
 inline FxOps make_fx_ops(const Ops<double>& o, int n) {

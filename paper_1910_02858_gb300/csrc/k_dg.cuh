@@ -2024,8 +2024,9 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
   return cudaGetLastError();
 }
 
-// fixed-point lifting + volume kernel (FP64, standard form, BR1); volume = 0: the lifting alone
-template <int n, bool LGL>
+// fixed-point lifting + volume kernel (FP64, BR1; standard or kinetic-energy-preserving split
+// form); volume = 0: the lifting alone
+template <int n, bool LGL, bool KEP = false>
 static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double>& ops, const Phys<double>& ph,
                              int store_grad, cudaStream_t st, int volume = 1) {
   using C = Cfg<n>;
@@ -2034,25 +2035,25 @@ static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double
   const int groups = (m.K + C::NE - 1) / C::NE;
   if (m.nAffine > 0) {
     constexpr size_t smem = lift_affine_smem_total<n>();
-    auto* kernel = &k_lift_vol_fx_affine<n, LGL>;
+    auto* kernel = &k_lift_vol_fx_affine<n, LGL, KEP>;
     static std::atomic<unsigned long long> attr{0};
     cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
     if (err != cudaSuccess) return err;
     kernel<<<m.nAffine, C::T, smem, st>>>(U, m.affine, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
                                           (const double*)m.fgeo, m.elemSide, (double*)m.Gf, Utv, Gvol, m.K, m.S, m.Sface,
-                                          m.nAffine < groups ? m.order : nullptr, ops, m.fx, ph);
+                                          m.nAffine < groups ? m.order : nullptr, ops, m.fx, m.fxD, ph);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
   if (m.nAffine < groups) {
     constexpr size_t smem = lift_fx_smem<n>();
-    auto* kernel = &k_lift_vol_fx<n, LGL>;
+    auto* kernel = &k_lift_vol_fx<n, LGL, KEP>;
     static std::atomic<unsigned long long> attr{0};
     cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
     if (err != cudaSuccess) return err;
     kernel<<<groups - m.nAffine, C::T, smem, st>>>(U, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
                                                    (const double*)m.fgeo, m.elemSide, (double*)m.Gf, Utv, Gvol, m.K, m.S,
                                                    m.Sface, (const double*)m.QB,
-                                                   m.nAffine > 0 ? m.order + m.nAffine : nullptr, ops, m.fx, ph);
+                                                   m.nAffine > 0 ? m.order + m.nAffine : nullptr, ops, m.fx, m.fxD, ph);
   }
   return cudaGetLastError();
 }
@@ -2103,6 +2104,9 @@ cudaError_t launch_lift_vol(const DevMesh& m, const real* U, const Ops<real>& op
         FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, true>(m, U, ops, ph, store_grad, st));
       }
       FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, false>(m, U, ops, ph, store_grad, st));
+    }
+    if (!m.br2 && m.split == 1) {
+      FLEXI_DISPATCH_N(m.n, return lift_fx_n<NN, true, true>(m, U, ops, ph, store_grad, st));
     }
   }
   if (m.br2) {

@@ -107,25 +107,25 @@ cudaError_t geom_jacobian(const double* const dX[3], double* sJ, double* wJ, con
 }
 
 namespace {
-__global__ void k_affine(const double* __restrict__ aff, const int* __restrict__ flag, double* __restrict__ Ja,
+__global__ void k_affine(const double* __restrict__ aff, double* __restrict__ Ja,
                          double* __restrict__ sJ, double* __restrict__ wJ, const double* __restrict__ w, int K, int n) {
   const int n3 = n * n * n;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)K * n3) return;
   const long long e = idx / n3;
-  if (!flag[e]) return;
-  const int node = (int)(idx - e * n3);
   const double* a = aff + e * 10;
+  if (a[9] == 0.0) return;
+  const int node = (int)(idx - e * n3);
   for (int c = 0; c < 9; ++c) Ja[(e * 9 + c) * n3 + node] = a[c];
   sJ[idx] = a[9];
   wJ[idx] = w[node % n] * w[(node / n) % n] * w[node / (n * n)] / a[9];
 }
 }  // namespace
 
-cudaError_t geom_affine(const double* aff, const int* flag, double* Ja, double* sJ, double* wJ, const double* w, int K, int n,
+cudaError_t geom_affine(const double* aff, double* Ja, double* sJ, double* wJ, const double* w, int K, int n,
                         cudaStream_t st) {
   const long long tot = (long long)K * n * n * n;
-  k_affine<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(aff, flag, Ja, sJ, wJ, w, K, n);
+  k_affine<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(aff, Ja, sJ, wJ, w, K, n);
   return cudaGetLastError();
 }
 

@@ -40,7 +40,7 @@ __device__ __forceinline__ void fp64_line(double* __restrict__ p, int stride, do
 // The kernel below for elements outside the fixed-point range: the same schedule over the
 // same shared memory in FP64 (speed does not matter here, the footprint does: the general
 // FP64 body's would cost the resident second CTA).
-template <int n, bool LGL>
+template <int n, bool LGL, bool KEP>
 __device__ __noinline__ void lift_vol_fp64(const double* U, const double* Ja, const double* sJ, const double* Wf,
                                            const double* fgeo, double* Gf, double* Utv, double* Gvol, int K, int S,
                                            int bigBase, const double* QB, const Ops<double>& ops, const Phys<double>& ph,
@@ -123,22 +123,54 @@ __device__ __noinline__ void lift_vol_fp64(const double* U, const double* Ja, co
   }
   if (Utv == nullptr) return;
   double F[3][NV];
-  for (int d = 0; d < 3; ++d) flux_total(Uo, W, G, d, ph, F[d]);
+  for (int d = 0; d < 3; ++d) {
+    if constexpr (KEP) {
+      flux_viscous(W, dg_rcp(W[0]), G, d, ph, F[d]);
+      for (int v = 0; v < NV; ++v) F[d][v] = -F[d][v];
+    } else {
+      flux_total(Uo, W, G, d, ph, F[d]);
+    }
+  }
   for (int l = 0; l < 3; ++l)
     for (int v = 0; v < NV; ++v)
       own[(l * NV + v) * n3p] = jac[l * 3] * F[0][v] + jac[l * 3 + 1] * F[1][v] + jac[l * 3 + 2] * F[2][v];
   __syncthreads();
   lines(std::false_type{}, 0);
   __syncthreads();
+  double acc[NV];
+  for (int v = 0; v < NV; ++v) acc[v] = own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p];
+  if constexpr (KEP) {  // as split_volume_fx
+    const double H = dg_div(Uo[4] + W[4], W[0]);
+    for (int v = 0; v < NV; ++v) own[v * n3p] = W[v];
+    own[5 * n3p] = H;
+    for (int c = 0; c < 9; ++c) own[(6 + c) * n3p] = jac[c];
+    __syncthreads();
+    for (int l = 0; l < 3; ++l) {
+      const int il = l == 0 ? node % n : (l == 1 ? (node / n) % n : node / n2), stride = l == 0 ? 1 : (l == 1 ? P : P * n);
+      for (int a = 0; a < n; ++a) {
+        if (a == il) continue;
+        const double* f = own + (a - il) * stride;
+        const double j0 = jac[l * 3] + f[(6 + 3 * l) * n3p], j1 = jac[l * 3 + 1] + f[(7 + 3 * l) * n3p],
+                     j2 = jac[l * 3 + 2] + f[(8 + 3 * l) * n3p];
+        const double us = W[1] + f[n3p], vs = W[2] + f[2 * n3p], ws = W[3] + f[3 * n3p];
+        const double m = 0.125 * (W[0] + f[0]) * (us * j0 + vs * j1 + ws * j2), hp = 0.5 * (W[4] + f[4 * n3p]);
+        const double d = ops.DT[a * n + il];
+        acc[0] += d * (2.0 * m);
+        acc[1] += d * (m * us + hp * j0);
+        acc[2] += d * (m * vs + hp * j1);
+        acc[3] += d * (m * ws + hp * j2);
+        acc[4] += d * (m * (H + f[5 * n3p]));
+      }
+    }
+  }
   if (valid)
-    for (int v = 0; v < NV; ++v)
-      Utv[((size_t)e * NV + v) * n3 + node] = own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p];
+    for (int v = 0; v < NV; ++v) Utv[((size_t)e * NV + v) * n3 + node] = acc[v];
 }
 
 template <int n>
 constexpr size_t lift_fx_smem() {
   using C = Cfg<n>;
-  return 8 * C::NE * (15 * C::n3p + 48 * C::n2) + sizeof(int) * C::NE * (12 + 6 * C::n2 + FX_SLOTS + 32);
+  return 8 * C::NE * (15 * C::n3p + 48 * C::n2) + 8 * C::n2 + sizeof(int) * C::NE * (12 + 6 * C::n2 + FX_SLOTS + 32);
 }
 
 // CTAs per SM asked of the register allocator (n = 8: two of 512 threads at 64 registers)
@@ -232,13 +264,180 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
   return true;
 }
 
-template <int n, bool LGL>
+// Split form (kinetic-energy preserving, Gauss-Lobatto): the viscous flux as in volume_fx; the
+// advective part 2 sum_a D_ia F#(i, a) with one thread per node over its 3 (n - 1) pairs, in
+// fixed point: pair sums and their products replace 21 FP64 multiply-adds per pair.  The
+// diagonal terms 2 D_ii F(U_i) and the strong form's face terms -(+-1) l_hat(+-1) F(U_i) cancel
+// (2 w_i D_ii = +-1 at the ends, 0 inside), so neither is formed.  Scales: rho, (u, v, w),
+// H and Ja each under one power of two; p and the mass flux times velocity share one (sh).
+// 990 elements, N = 7: 1130 -> 232 us with the lifting.
+template <int n, bool AFF, typename Metric>
+__device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, double* __restrict__ Utv, const double (&W)[NV],
+                                                const double (&G)[15], int K, int grp, unsigned wmask, fx64* sA, int* sMag,
+                                                int2* sD, const FxOps& fx, const FxStrong& fd, const Phys<double>& ph,
+                                                Metric metric) {
+  using C = Cfg<n>;
+  constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p, P = C::P;
+  const int tid = threadIdx.x;
+  const int el = tid / n3, node = tid - el * n3;
+  const int e = grp * NE + el;
+  const bool valid = e < K;
+  int* mag = sMag + el * FX_SLOTS;
+  fx64* own = sA + el * 15 * n3p + pidx<n>(node % n, (node / n) % n, node / n2);
+  double H;
+  {
+    double E = 1.0;
+    if (valid) E = U[((size_t)e * NV + 4) * n3 + node];
+    const double ir = 1.0 / W[0];
+    H = (E + W[4]) * ir;
+    int mx[NV] = {0, 0, 0, 0, 0};  // slot 0: H, 1-4: viscous flux
+    mx[0] = fx_mag(H);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      double F[NV];
+      flux_viscous(W, ir, G, d, ph, F);
+#pragma unroll
+      for (int v = 1; v < NV; ++v) {
+        own[(d * NV + v) * n3p] = __double_as_longlong(-F[v]);
+        mx[v] = max(mx[v], fx_mag(F[v]));
+      }
+    }
+    fx_max<NE == 1, NV>(mag + FX_F, wmask, [&](int s) { return mx[s]; });
+  }
+  for (int t = tid; t < n2; t += T) sD[t] = make_int2(fd.h[t], fd.l[t]);
+  __syncthreads();
+  {
+    int bad = 0;
+    for (int t = tid; t < NE * NV; t += T)
+      bad |= (sMag[(t / NV) * FX_SLOTS + FX_F + t % NV] >> 20) > (t % NV == 0 ? FX_MAX_EXP + 200 : FX_MAX_FLUX);
+    if (__syncthreads_or(bad)) return false;
+  }
+  int EJm;
+  double vis[NV];
+  {
+    FxSplit ji[9];
+    metric(ji, EJm);
+#pragma unroll
+    for (int v = 1; v < NV; ++v) {
+      FxSplit F[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) F[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FX_F + v] >> 20));
+#pragma unroll
+      for (int l = 0; l < 3; ++l) {
+        FxAcc s;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) s.add(ji[l * 3 + d], F[d]);
+        own[(l * NV + v) * n3p] = s.get();
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int it = tid; it < NE * 12 * n2; it += T) {
+    const int q = it / n2, line = it - q * n2;
+    const int el2 = q / 12, c = q - el2 * 12, l = c >> 2, f = el2 * 15 + l * NV + 1 + (c & 3);
+    int stride;
+    const int at = fx_line_at<n>(l, line, stride);
+    fx_line<n, true, false>(sA + f * n3p + at, stride, 0, 0, fx);
+  }
+  __syncthreads();
+  vis[0] = 0.0;
+#pragma unroll
+  for (int v = 1; v < NV; ++v)
+    vis[v] = fx_to(own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p], (mag[FX_F + v] >> 20) + EJm - 2044 + 6 - fx.kc);
+  // advective part: bounds b of rho, velocity, Ja, H, p as powers of two
+  const int bR = (mag[FX_W] >> 20) - 1022, bJ = EJm - 1022, bH = (mag[FX_F] >> 20) - 1022;
+  const int bU = (max(mag[FX_W + 1], max(mag[FX_W + 2], mag[FX_W + 3])) >> 20) - 1022;
+  const int sh = min(max(0, (mag[FX_W + 4] >> 20) - 1022 - (bR + 2 * bU + 2)), 62);  // shift of m against p
+  const int bP = max(bR + 2 * bU + 2 + sh, (mag[FX_W + 4] >> 20) - 1022);
+  fx64 q[6];
+  q[0] = fx_from<60>(W[0], bR + 1022);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) q[1 + d] = fx_from<60>(W[1 + d], bU + 1022);
+  q[4] = fx_from<60>(W[4], bP + 1022);
+  q[5] = fx_from<60>(H, bH + 1022);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) own[c * n3p] = q[c];
+  {
+    FxSplit ji[9];
+    metric(ji, EJm);
+    if constexpr (!AFF) {
+#pragma unroll
+      for (int c = 0; c < 9; ++c) own[(6 + c) * n3p] = fx_shr(((fx64)ji[c].h << 32) + ji[c].l, 2);
+    } else {  // J^l_d is the pair's mean: its sum in the same units
+#pragma unroll
+      for (int c = 0; c < 9; ++c) own[(6 + c) * n3p] = fx_shr(((fx64)ji[c].h << 32) + ji[c].l, 1);
+    }
+  }
+  __syncthreads();
+  fx64 sum[NV] = {0, 0, 0, 0, 0};
+#pragma unroll 1
+  for (int l = 0; l < 3; ++l) {
+    const int il = l == 0 ? node % n : (l == 1 ? (node / n) % n : node / n2), stride = l == 0 ? 1 : (l == 1 ? P : P * n);
+    const fx64* jo = own + (6 + 3 * l) * n3p;
+    const fx64 J0 = jo[0], J1 = jo[n3p], J2 = jo[2 * n3p];
+    FxAcc s[NV];
+    int a = il;
+#pragma unroll 1
+    for (int k = 1; k < n; ++k) {
+      a = a + 1 == n ? 0 : a + 1;
+      const fx64* f = own + (a - il) * stride;
+      const FxSplit u = fx_split(q[1] + f[n3p]), v = fx_split(q[2] + f[2 * n3p]), w = fx_split(q[3] + f[3 * n3p]);
+      FxSplit j0, j1, j2;
+      if constexpr (AFF) {
+        j0 = fx_split(J0);
+        j1 = fx_split(J1);
+        j2 = fx_split(J2);
+      } else {
+        const fx64* jp = f + (6 + 3 * l) * n3p;
+        j0 = fx_split(J0 + jp[0]);
+        j1 = fx_split(J1 + jp[n3p]);
+        j2 = fx_split(J2 + jp[2 * n3p]);
+      }
+      FxAcc c;
+      c.add(u, j0);
+      c.add(v, j1);
+      c.add(w, j2);
+      const fx64 mi = fx_mul(fx_split(q[0] + f[0]), fx_split(c.get() << 2));  // 8 {rho}{u . Ja} in its units
+      const FxSplit m4 = fx_split(mi << 2), ms = fx_split((mi << 2) >> sh), p = fx_split(q[4] + f[4 * n3p]);
+      const int2 D = sD[a * n + il];
+      const FxSplit d{D.x, D.y};
+      s[0].add(fx_split(mi), d);
+      FxAcc x;
+      x.add(ms, u);
+      x.add(p, j0);
+      s[1].add(fx_split(x.get()), d);
+      x = FxAcc();
+      x.add(ms, v);
+      x.add(p, j1);
+      s[2].add(fx_split(x.get()), d);
+      x = FxAcc();
+      x.add(ms, w);
+      x.add(p, j2);
+      s[3].add(fx_split(x.get()), d);
+      s[4].add(fx_split(fx_mul(m4, fx_split(q[5] + f[5 * n3p]))), d);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sum[v] += s[v].get();
+  }
+  if (valid) {
+    const int t0 = bR + bU + bJ + 64 - fd.k;
+    double* out = Utv + (size_t)e * NV * n3 + node;
+    out[0] = fx_to(sum[0], t0 - 56);
+#pragma unroll
+    for (int v = 1; v < 4; ++v) out[(size_t)v * n3] = vis[v] + fx_to(sum[v], bP + bJ - 57 + 64 - fd.k);
+    out[(size_t)4 * n3] = vis[4] + fx_to(sum[4], t0 + bH - 55);
+  }
+  return true;
+}
+
+template <int n, bool LGL, bool KEP = false>
 __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol_fx(
     const double* __restrict__ U, const double* __restrict__ Ja, const double* __restrict__ sJ,
     const double* __restrict__ Wf, const double* __restrict__ fgeo, const int* __restrict__ elemSide,
     double* __restrict__ Gf, double* __restrict__ Utv, double* __restrict__ Gvol, int K, int S, int bigBase,
     const double* __restrict__ QB, const int* __restrict__ order, const __grid_constant__ Ops<double> ops,
-    const __grid_constant__ FxOps fx, const __grid_constant__ Phys<double> ph) {
+    const __grid_constant__ FxOps fx, const __grid_constant__ FxStrong fd, const __grid_constant__ Phys<double> ph) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   constexpr bool kWarp = NE == 1;
@@ -246,7 +445,8 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx64* sA = reinterpret_cast<fx64*>(smem_raw);  // [NE][15][n3p] line fields l*5 + v, contracted in place
   fx64* sW = sA + NE * 15 * n3p;                 // [NE][6][8][n2] face means of W (5) and outward n_d s_hat (3)
-  int* sES = reinterpret_cast<int*>(sW + NE * 48 * n2);
+  int2* sD = reinterpret_cast<int2*>(sW + NE * 48 * n2);  // [n2] strong-form derivative (KEP)
+  int* sES = reinterpret_cast<int*>(sD + n2);
   int* sSlot = sES + NE * 6;
   int* sMpq = sSlot + NE * 6;            // [NE][6][n2] master-frame node of each face node
   int* sMag = sMpq + NE * 6 * n2;        // [NE][FX_SLOTS] largest magnitude words
@@ -337,7 +537,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
       sExp[el2 * 32 + 16 + c] = min(1 + x - prod, 62);
     }
     if (__syncthreads_or(bad)) {
-      lift_vol_fp64<n, LGL>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph,
+      lift_vol_fp64<n, LGL, KEP>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph,
                             reinterpret_cast<double*>(sA), reinterpret_cast<double*>(sW), sES, sMpq, grp);
       return;
     }
@@ -434,13 +634,19 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
     __syncthreads();
   }
   if (Utv == nullptr) return;  // the adjoint's recompute needs the gradients only
-  if (!volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, [&](FxSplit (&ji)[9], int& EJm) {
-        EJm = max(mag[FX_J], max(mag[FX_J + 1], mag[FX_J + 2])) >> 20;
+  auto metric = [&](FxSplit (&ji)[9], int& EJm) {
+    EJm = max(mag[FX_J], max(mag[FX_J + 1], mag[FX_J + 2])) >> 20;
 #pragma unroll
-        for (int c = 0; c < 9; ++c)
-          ji[c] = fx_split(fx_from<62>(valid ? Ja[((size_t)e * 9 + c) * n3 + node] : 0.0, EJm));
-      }))
-    lift_vol_fp64<n, LGL>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph, reinterpret_cast<double*>(sA),
+    for (int c = 0; c < 9; ++c)
+      ji[c] = fx_split(fx_from<62>(valid ? Ja[((size_t)e * 9 + c) * n3 + node] : 0.0, EJm));
+  };
+  bool done;
+  if constexpr (KEP)
+    done = split_volume_fx<n, false>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
+  else
+    done = volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
+  if (!done)
+    lift_vol_fp64<n, LGL, KEP>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph, reinterpret_cast<double*>(sA),
                           reinterpret_cast<double*>(sW), sES, sMpq, grp);
 }
 
@@ -454,7 +660,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
 template <int n>
 constexpr size_t lift_affine_smem() {
   using C = Cfg<n>;
-  return 8 * C::NE * (15 * C::n3p + 30 * C::n2 + 18) + sizeof(int) * C::NE * (12 + 6 * C::n2 + FX_SLOTS + 4);
+  return 8 * C::NE * (15 * C::n3p + 30 * C::n2 + 18) + 8 * C::n2 + sizeof(int) * C::NE * (12 + 6 * C::n2 + FX_SLOTS + 4);
 }
 
 // the general kernel's FP64 schedule needs its shared memory: 48 n^2 face values per element
@@ -463,13 +669,13 @@ constexpr size_t lift_affine_smem_total() {
   return lift_affine_smem<n>() > lift_fx_smem<n>() ? lift_affine_smem<n>() : lift_fx_smem<n>();
 }
 
-template <int n, bool LGL>
+template <int n, bool LGL, bool KEP = false>
 __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol_fx_affine(
     const double* __restrict__ U, const double* __restrict__ aff, const double* __restrict__ Ja,
     const double* __restrict__ sJ, const double* __restrict__ Wf, const double* __restrict__ fgeo,
     const int* __restrict__ elemSide, double* __restrict__ Gf, double* __restrict__ Utv, double* __restrict__ Gvol, int K,
     int S, int bigBase, const int* __restrict__ order, const __grid_constant__ Ops<double> ops,
-    const __grid_constant__ FxOps fx, const __grid_constant__ Phys<double> ph) {
+    const __grid_constant__ FxOps fx, const __grid_constant__ FxStrong fd, const __grid_constant__ Phys<double> ph) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   constexpr bool kWarp = NE == 1;
@@ -477,7 +683,8 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx64* sA = reinterpret_cast<fx64*>(smem_raw);  // [NE][15][n3p] line fields l*5 + v, contracted in place
   fx64* sW = sA + NE * 15 * n3p;                 // [NE][6][5][n2] face means of W
-  int* sES = reinterpret_cast<int*>(smem_raw + lift_affine_smem_total<n>()) - NE * (12 + 6 * n2 + FX_SLOTS + 4);
+  int2* sD = reinterpret_cast<int2*>(smem_raw + lift_affine_smem_total<n>()) - n2;  // [n2] strong-form derivative (KEP)
+  int* sES = reinterpret_cast<int*>(sD) - NE * (12 + 6 * n2 + FX_SLOTS + 4);
   int* sSlot = sES + NE * 6;
   int* sMpq = sSlot + NE * 6;          // [NE][6][n2] master-frame node of each face node
   int* sMag = sMpq + NE * 6 * n2;      // [NE][FX_SLOTS] largest magnitude words; FX_J + d: of J^l_d / J; FX_S: of J^l_d
@@ -552,7 +759,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   fx_max<kWarp, NV>(mag + FX_W, wmask, [&](int s) { return mW[s]; });
   __syncthreads();
   auto fp64 = [&]() {
-    lift_vol_fp64<n, LGL>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, nullptr, ops, ph, reinterpret_cast<double*>(sA),
+    lift_vol_fp64<n, LGL, KEP>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, nullptr, ops, ph, reinterpret_cast<double*>(sA),
                           reinterpret_cast<double*>(sW), sES, sMpq, grp);
   };
   {
@@ -645,11 +852,17 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   }
   if (Utv == nullptr) return;
   __syncthreads();
-  if (!volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, [&](FxSplit (&ji)[9], int& EJm) {
-        EJm = mag[FX_S] >> 20;
+  auto metric = [&](FxSplit (&ji)[9], int& EJm) {
+    EJm = mag[FX_S] >> 20;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) ji[c] = fx_split(sM[el * 18 + 9 + c]);
-      }))
+    for (int c = 0; c < 9; ++c) ji[c] = fx_split(sM[el * 18 + 9 + c]);
+  };
+  bool done;
+  if constexpr (KEP)
+    done = split_volume_fx<n, true>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
+  else
+    done = volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
+  if (!done)
     fp64();
 }
 

@@ -60,6 +60,7 @@ struct DevMesh {
   const int* order = nullptr;      // [groups]
   int nAffine = 0;
   FxOps fx{};                  // fixed-point line operators (FP64 form)
+  FxStrong fxD{};              // strong-form derivative (split forms)
   FxOps fxT{};                 // and their transposes (adjoint)
   unsigned* status = nullptr;  // device status word (bit 0: non-physical face state)
 };
@@ -143,8 +144,8 @@ cudaError_t geom_jacobian(const double* const dX[3], double* sJ, double* wJ, con
                           unsigned* bad, cudaStream_t st);
 cudaError_t geom_faces(const double* Ja, const double* X, const int* sideMaster, const double* lm,
                        const double* lp, double* fgeo, double* xbc, int S, int nBC, int n, cudaStream_t st);
-// constant metric terms of affine elements (flag[e] != 0): Ja, 1/J and the quadrature weights
-cudaError_t geom_affine(const double* aff, const int* flag, double* Ja, double* sJ, double* wJ, const double* w, int K, int n,
+// constant metric terms of affine elements (aff[e][9] = 1/J != 0): Ja, 1/J and the quadrature weights
+cudaError_t geom_affine(const double* aff, double* Ja, double* sJ, double* wJ, const double* w, int K, int n,
                         cudaStream_t st);
 // sine and cosine of pi (x + y + z) at the solution nodes, [K][2][n^3]
 cudaError_t geom_phase(const double* X, void* phase, bool fp64, int K, int n3, cudaStream_t st);
