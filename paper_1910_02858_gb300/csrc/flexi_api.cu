@@ -512,6 +512,19 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   fill_ops<double>(c->ops64, Ds, ws, lmv, lpv, n);
   fill_ops<float>(c->ops32, Ds, ws, lmv, lpv, n);
   c->m.fx = make_fx_ops(c->ops64, n);
+  for (int a = 0; a < (n + 1) / 2; ++a) {
+    const int b = n - 1 - a;  // mirror node
+    const bool mid = a == b;
+    c->m.eo.pe[a] = (float)(mid ? lpv[a] : 0.5 * (lpv[a] + lmv[a]));
+    c->m.eo.po[a] = (float)(0.5 * (lpv[a] - lmv[a]));
+    c->m.eo.s[a] = (float)(0.5 * (c->ops64.lhp[a] + c->ops64.lhm[a]));
+    c->m.eo.t[a] = (float)(0.5 * (c->ops64.lhp[a] - c->ops64.lhm[a]));
+    for (int i = 0; i < (n + 1) / 2; ++i) {
+      const double x = c->ops64.DhatT[a * n + i], y = c->ops64.DhatT[b * n + i];
+      c->m.eo.e[i][a] = (float)(mid ? x : 0.5 * (x + y));
+      c->m.eo.o[i][a] = (float)(0.5 * (x - y));
+    }
+  }
   c->m.fxD = make_fx_strong(c->ops64, n);
   c->m.fxT = make_fx_ops_transposed(c->ops64, n);
   fill_mortar_ops<double>(c->mops64, xs, ws, n);
@@ -635,11 +648,12 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   CK(geom_jacobian(dX, c->sJ64, c->wJ, wdev, K, n, c->status, st));
   // affine elements: constant metric terms from the edge vectors (their differences from the
   // derivatives above are the coordinates' rounding), where the lifting kernel has a variant
-  // for such elements (launch_lift_vol: not BR2 or the entropy-conservative form) and the mesh is not one of the
-  // smallest, whose kernels read the metric terms per node
+  // for such elements (launch_lift_vol: not BR2, not the split forms without one) and the mesh is not one of the
+  // smallest FP64 ones, whose kernels read the metric terms per node
   int nsm = 1;
   CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
-  if (c->fp64 && p->lifting == FLEXI_LIFTING_BR1 && p->split_form != FLEXI_SPLIT_EC && !(n <= 4 && K < nsm)) {
+  if (p->lifting == FLEXI_LIFTING_BR1 &&
+      (c->fp64 ? p->split_form != FLEXI_SPLIT_EC && !(n <= 4 && K < nsm) : p->split_form == FLEXI_SPLIT_STANDARD)) {
     std::vector<double> aff((size_t)K * 10, 0.0);  // 1/J = 0: not affine
     std::vector<char> flag(K);
     bool any = false;
@@ -654,6 +668,12 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
       CK(geom_affine(daff, c->Ja64, c->sJ64, c->wJ, wdev, K, n, st));
       CK(cudaStreamSynchronize(st));
       c->m.affine = daff;
+      if (!c->fp64) {
+        float* faff;
+        AL(faff, aff.size());
+        CK(convert_f64_to_f32(daff, faff, aff.size(), st));
+        c->m.affine = faff;
+      }
       // groups of elements per CTA, affine ones first (a big side's lifting flux is not a face mean)
       for (int m2 = 0; m2 < M; ++m2) flag[mortars[15 * m2]] = 0;
       const int ne = n3 >= 64 ? 1 : (64 + n3 - 1) / n3, groups = (K + ne - 1) / ne;  // Cfg<n>::NE

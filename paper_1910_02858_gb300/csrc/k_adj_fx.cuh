@@ -342,7 +342,7 @@ static cudaError_t launch_adj_vol_fx(const DevMesh& m, const double* U, const do
 #define FLEXI_ADJ_FX(AFF, GRID, ORDER)                                                                                \
   do {                                                                                                                \
     if ((err = ensure_dynamic_smem(&k_adj_vol_fx<n, AFF>, smem, attr[AFF])) != cudaSuccess) return err;              \
-    k_adj_vol_fx<n, AFF><<<GRID, C::T, smem, st>>>(U, (const double*)m.Ja, m.affine, (const double*)m.sJ,           \
+    k_adj_vol_fx<n, AFF><<<GRID, C::T, smem, st>>>(U, (const double*)m.Ja, (const double*)m.affine, (const double*)m.sJ,           \
                                                    (const double*)m.Gvol, (const double*)m.fgeo, m.elemSide, lam,    \
                                                    LGf, LWs, LWf, muv, m.K, m.S, m.Sface, LQB, ORDER, ops, m.fxT, ph); \
     if ((err = cudaGetLastError()) != cudaSuccess) return err;                                                        \

@@ -404,7 +404,7 @@ __device__ __forceinline__ void lift_vol_body(
     const real* __restrict__ U, const real* __restrict__ Ja, const real* __restrict__ sJ,
     const real* __restrict__ Wf, const real* __restrict__ fgeo, const int* __restrict__ elemSide,
     real* __restrict__ Gf, real* __restrict__ Utv, real* __restrict__ Gvol, int K, int S, int bigBase,
-    const real* __restrict__ QB, const Ops<real>& ops, const Phys<real>& ph) {
+    const real* __restrict__ QB, const int* __restrict__ order, const Ops<real>& ops, const Phys<real>& ph) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -426,7 +426,7 @@ __device__ __forceinline__ void lift_vol_body(
 
   const int tid = threadIdx.x;
   const int el = tid / n3, node = tid - el * n3;
-  const int e0 = blockIdx.x * NE;
+  const int e0 = (order != nullptr ? order[blockIdx.x] : blockIdx.x) * NE;
   const int e = e0 + el;
   const bool valid = e < K;
   const int i = node % n, j = (node / n) % n, k = node / n2;
@@ -931,8 +931,8 @@ __device__ __forceinline__ void lift_vol_body(
   const real *__restrict__ U, const real *__restrict__ Ja, const real *__restrict__ sJ,                   \
       const real *__restrict__ Wf, const real *__restrict__ fgeo, const int *__restrict__ elemSide,        \
       real *__restrict__ Gf, real *__restrict__ Utv, real *__restrict__ Gvol, int K, int S, int bigBase, \
-      const real *__restrict__ QB, Ops<real> ops, Phys<real> ph
-#define FLEXI_LIFT_VOL_ARGS U, Ja, sJ, Wf, fgeo, elemSide, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph
+      const real *__restrict__ QB, const int *__restrict__ order, Ops<real> ops, Phys<real> ph
+#define FLEXI_LIFT_VOL_ARGS U, Ja, sJ, Wf, fgeo, elemSide, Gf, Utv, Gvol, K, S, bigBase, QB, order, ops, ph
 
 // the kernel at the compiler's default register allocation
 template <typename real, int n, int SW, bool LGL, int SPLIT = 0, bool BR2 = false>
@@ -949,6 +949,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_vol_min_blocks<real, n, SW, SP
 #undef FLEXI_LIFT_VOL_ARGS
 
 }  // namespace flexi
+#include "k_lift_f32_affine.cuh"
 #include "k_lift_fx.cuh"
 #include "k_surf_fx.cuh"
 namespace flexi {
@@ -2014,12 +2015,27 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
   static std::atomic<unsigned long long> attr{0};
   cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
   if (err != cudaSuccess) return err;
-  const int grid = (m.K + C::NE - 1) / C::NE;
+  const int groups = (m.K + C::NE - 1) / C::NE;
+  const int* order = nullptr;
+  int grid = groups;
+  if constexpr (sizeof(real) == 4 && SPLIT == 0 && !BR2) {  // affine elements by their own kernel
+    if (m.nAffine > 0) {
+      constexpr size_t smemA = lift_f32_affine_smem<n, SW>();
+      static std::atomic<unsigned long long> attrA{0};
+      if ((err = ensure_dynamic_smem(&k_lift_vol_f32_affine<n, SW, LGL>, smemA, attrA)) != cudaSuccess) return err;
+      k_lift_vol_f32_affine<n, SW, LGL><<<m.nAffine, C::T, smemA, st>>>(
+          U, (const float*)m.affine, (const float*)m.Wf, m.elemSide, (float*)m.Gf, (float*)m.Utv,
+          store_grad ? (float*)m.Gvol : nullptr, m.K, m.S, m.nAffine < groups ? m.order : nullptr, ops, m.eo, ph);
+      if ((err = cudaGetLastError()) != cudaSuccess || m.nAffine == groups) return err;
+      order = m.order + m.nAffine;
+      grid = groups - m.nAffine;
+    }
+  }
   kernel<<<grid, C::T, smem, st>>>(U, (const real*)m.Ja, (const real*)m.sJ,
                                                          (const real*)m.Wf, (const real*)m.fgeo, m.elemSide,
                                                          (real*)m.Gf, (real*)m.Utv,
                                                          store_grad ? (real*)m.Gvol : nullptr, m.K, m.S,
-                                                         m.Sface, (const real*)m.QB,
+                                                         m.Sface, (const real*)m.QB, order,
                                                          ops, ph);
   return cudaGetLastError();
 }
@@ -2039,7 +2055,7 @@ static cudaError_t lift_fx_n(const DevMesh& m, const double* U, const Ops<double
     static std::atomic<unsigned long long> attr{0};
     cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
     if (err != cudaSuccess) return err;
-    kernel<<<m.nAffine, C::T, smem, st>>>(U, m.affine, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
+    kernel<<<m.nAffine, C::T, smem, st>>>(U, (const double*)m.affine, (const double*)m.Ja, (const double*)m.sJ, (const double*)m.Wf,
                                           (const double*)m.fgeo, m.elemSide, (double*)m.Gf, Utv, Gvol, m.K, m.S, m.Sface,
                                           m.nAffine < groups ? m.order : nullptr, ops, m.fx, m.fxD, ph);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;

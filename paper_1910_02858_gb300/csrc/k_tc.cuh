@@ -63,17 +63,22 @@ __device__ __forceinline__ void split3_bf16(float x, float& x1, float& x2, float
   x3 = __bfloat162float(__float2bfloat16_rn(r1 - x2));
 }
 
-// B fragments of Dhat^T (B[a][i] = Dhat[i][a] = DhatT[a*n+i]) held per lane
+// B fragments of Dhat^T (B[a][i] = Dhat[i][a] = DhatT[a*n+i]) held per lane; AUG (n <= 6): rows n
+// and n + 1 are l_hat(-1) and l_hat(+1) (at n*n + 2n and n*n + 3n)
 template <int SW>
 struct BFrag {
   uint32_t r[6];
 };
 
-template <int n, int SW>
+template <int n, int SW, bool AUG = false>
 __device__ __forceinline__ BFrag<SW> make_bfrag(const float* sD, int lane) {
   const int gid = lane >> 2, tig = lane & 3;
   BFrag<SW> f;
-  auto B = [&](int a, int i) -> float { return (a < n && i < n) ? sD[a * n + i] : 0.f; };
+  auto B = [&](int a, int i) -> float {
+    if (i >= n) return 0.f;
+    if (AUG && (a == n || a == n + 1)) return sD[n * n + (a - n + 2) * n + i];
+    return a < n ? sD[a * n + i] : 0.f;
+  };
   if (SW == 1) {
     // r[2t], r[2t+1]: term t of the rows (tig, tig + 4) at column gid
     split3_tf32(B(tig, gid), f.r[0], f.r[2], f.r[4]);
@@ -89,6 +94,46 @@ __device__ __forceinline__ BFrag<SW> make_bfrag(const float* sD, int lane) {
     f.r[3] = f.r[4] = f.r[5] = 0u;
   }
   return f;
+}
+
+// c += A B of one 16-line tile: Aval(h, a) is entry a of row gid + 8 h
+template <int SW, typename Get>
+__device__ __forceinline__ void tc_product(Get Aval, const BFrag<SW>& bf, int tig, float c[4]) {
+  if (SW == 1) {
+    uint32_t a[3][4];  // a[term][reg]: regs (row gid, col tig), (gid+8, tig), (gid, tig+4), (gid+8, tig+4)
+    split3_tf32(Aval(0, tig), a[0][0], a[1][0], a[2][0]);
+    split3_tf32(Aval(1, tig), a[0][1], a[1][1], a[2][1]);
+    split3_tf32(Aval(0, tig + 4), a[0][2], a[1][2], a[2][2]);
+    split3_tf32(Aval(1, tig + 4), a[0][3], a[1][3], a[2][3]);
+    const uint32_t b1[2] = {bf.r[0], bf.r[1]}, b2[2] = {bf.r[2], bf.r[3]}, b3[2] = {bf.r[4], bf.r[5]};
+    mma_tf32(c, a[2], b1);  // A3 B1
+    mma_tf32(c, a[1], b2);  // A2 B2
+    mma_tf32(c, a[0], b3);  // A1 B3
+    mma_tf32(c, a[1], b1);  // A2 B1
+    mma_tf32(c, a[0], b2);  // A1 B2
+    mma_tf32(c, a[0], b1);  // A1 B1
+  } else {
+    float s00[3], s01[3], s10[3], s11[3];  // rows gid / gid+8, cols 2tig / 2tig+1
+    split3_bf16(Aval(0, 2 * tig), s00[0], s00[1], s00[2]);
+    split3_bf16(Aval(0, 2 * tig + 1), s01[0], s01[1], s01[2]);
+    split3_bf16(Aval(1, 2 * tig), s10[0], s10[1], s10[2]);
+    split3_bf16(Aval(1, 2 * tig + 1), s11[0], s11[1], s11[2]);
+    auto afrag = [&](int p, int q, uint32_t a[4]) {
+      a[0] = pack_bf16(s00[p], s01[p]);
+      a[1] = pack_bf16(s10[p], s11[p]);
+      a[2] = pack_bf16(s00[q], s01[q]);
+      a[3] = pack_bf16(s10[q], s11[q]);
+    };
+    uint32_t a[4];
+    const uint32_t b31[2] = {bf.r[2], bf.r[0]};
+    afrag(0, 2, a);
+    mma_bf16(c, a, b31);  // A1 B3 + A3 B1
+    const uint32_t b21[2] = {bf.r[1], bf.r[0]};
+    afrag(0, 1, a);
+    mma_bf16(c, a, b21);  // A1 B2 + A2 B1
+    const uint32_t b12[2] = {bf.r[0], bf.r[1]};
+    mma_bf16(c, a, b12);  // A1 B1 + A2 B2
+  }
 }
 
 // Accumulate sOut[el][v][node] (+)= sum over the 3 directions of the Dhat sweep of
@@ -125,41 +170,7 @@ __device__ __forceinline__ void tc_sweep3(const float* __restrict__ buf, float* 
           return (ok[h] && a < n) ? buf[fld[h] + base[h] + stride * a] : 0.f;
         };
         float c[4] = {0.f, 0.f, 0.f, 0.f};
-        if (SW == 1) {
-          uint32_t a[3][4];  // a[term][reg]: regs (row gid, col tig), (gid+8, tig), (gid, tig+4), (gid+8, tig+4)
-          split3_tf32(Aval(0, tig), a[0][0], a[1][0], a[2][0]);
-          split3_tf32(Aval(1, tig), a[0][1], a[1][1], a[2][1]);
-          split3_tf32(Aval(0, tig + 4), a[0][2], a[1][2], a[2][2]);
-          split3_tf32(Aval(1, tig + 4), a[0][3], a[1][3], a[2][3]);
-          const uint32_t b1[2] = {bf.r[0], bf.r[1]}, b2[2] = {bf.r[2], bf.r[3]}, b3[2] = {bf.r[4], bf.r[5]};
-          mma_tf32(c, a[2], b1);  // A3 B1
-          mma_tf32(c, a[1], b2);  // A2 B2
-          mma_tf32(c, a[0], b3);  // A1 B3
-          mma_tf32(c, a[1], b1);  // A2 B1
-          mma_tf32(c, a[0], b2);  // A1 B2
-          mma_tf32(c, a[0], b1);  // A1 B1
-        } else {
-          float s00[3], s01[3], s10[3], s11[3];  // rows gid / gid+8, cols 2tig / 2tig+1
-          split3_bf16(Aval(0, 2 * tig), s00[0], s00[1], s00[2]);
-          split3_bf16(Aval(0, 2 * tig + 1), s01[0], s01[1], s01[2]);
-          split3_bf16(Aval(1, 2 * tig), s10[0], s10[1], s10[2]);
-          split3_bf16(Aval(1, 2 * tig + 1), s11[0], s11[1], s11[2]);
-          auto afrag = [&](int p, int q, uint32_t a[4]) {
-            a[0] = pack_bf16(s00[p], s01[p]);
-            a[1] = pack_bf16(s10[p], s11[p]);
-            a[2] = pack_bf16(s00[q], s01[q]);
-            a[3] = pack_bf16(s10[q], s11[q]);
-          };
-          uint32_t a[4];
-          const uint32_t b31[2] = {bf.r[2], bf.r[0]};
-          afrag(0, 2, a);
-          mma_bf16(c, a, b31);  // A1 B3 + A3 B1
-          const uint32_t b21[2] = {bf.r[1], bf.r[0]};
-          afrag(0, 1, a);
-          mma_bf16(c, a, b21);  // A1 B2 + A2 B1
-          const uint32_t b12[2] = {bf.r[0], bf.r[1]};
-          mma_bf16(c, a, b12);  // A1 B1 + A2 B2
-        }
+        tc_product<SW>(Aval, bf, tig, c);
         // scatter C[row][i] to the node accumulator
 #pragma unroll
         for (int h = 0; h < 2; ++h) {

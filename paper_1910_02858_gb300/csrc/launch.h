@@ -26,6 +26,12 @@ cudaError_t ensure_dynamic_smem(Kernel* kernel, size_t smem, std::atomic<unsigne
   return err;
 }
 
+// FP32 one-dimensional operators split by the symmetry of the node sets (as FxOps in fx.cuh):
+// e, o, s, t for a line contraction with face terms, pe, po for the line's end values
+struct EvenOdd {
+  float e[MAXN / 2][MAXN / 2], o[MAXN / 2][MAXN / 2], s[MAXN / 2], t[MAXN / 2], pe[MAXN / 2], po[MAXN / 2];
+};
+
 // Device-resident mesh, geometry and scratch of one context (type-erased).
 struct DevMesh {
   int K = 0, S = 0, nBC = 0, N = 0, n = 0;
@@ -56,7 +62,8 @@ struct DevMesh {
   // Affine elements (parallelepipeds without a mortar big side): their constant metric terms
   // and 1/J, and the order in which the lifting kernels take the CTAs' element groups
   // (Cfg<n>::NE consecutive elements): nAffine groups of affine elements, then the others
-  const double* affine = nullptr;  // [K][10] Ja^l_d at l*3+d, 1/J
+  const void* affine = nullptr;    // [K][10] Ja^l_d at l*3+d, 1/J
+  EvenOdd eo{};                    // (FP32 forms)
   const int* order = nullptr;      // [groups]
   int nAffine = 0;
   FxOps fx{};                  // fixed-point line operators (FP64 form)
