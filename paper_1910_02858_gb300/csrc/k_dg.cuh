@@ -1535,8 +1535,9 @@ __global__ void __launch_bounds__(128) k_face3(const real* __restrict__ Wf, cons
 // TM > 1 (small meshes): TM times the threads, the first NE n^3 of them one per node, all
 // of them sharing the loops over face nodes (the gather of the face fluxes and the face
 // states of the new U), which otherwise take several dependent rounds of global-memory
-// latency per thread on a mesh that leaves most SMs idle.
-template <typename real, int n, int MODE, bool LGL, int TM = 1>
+// latency per thread on a mesh that leaves most SMs idle.  SRC = false: no source term (the
+// FP32 form runs at 32 registers, where the term's code costs 3 % without being run).
+template <typename real, int n, int MODE, bool LGL, int TM = 1, bool SRC = true>
 __global__ void __launch_bounds__(Cfg<n>::T * TM, TM > 1 ? 1 : ((sizeof(real) == 4 && Cfg<n>::T == 512) ? 4 : ((sizeof(real) == 4 && Cfg<n>::T == 216) ? 8 : 2))) k_surf(
     const real* __restrict__ Ff, const int* __restrict__ elemSide, const real* __restrict__ sJ,
     const real* __restrict__ Utv, real* __restrict__ U, real* __restrict__ dU, real* __restrict__ Ut,
@@ -1592,7 +1593,9 @@ __global__ void __launch_bounds__(Cfg<n>::T * TM, TM > 1 ? 1 : ((sizeof(real) ==
   if (valid) {
     const real* lhm = sOp + n2 + 2 * n;
     const real* lhp = sOp + n2 + 3 * n;
-    const real c0 = lhm[i], c1 = lhp[i], c2 = lhm[j], c3 = lhp[j], c4 = lhm[k], c5 = lhp[k];
+    // Gauss-Lobatto: nonzero at the end nodes only, so two registers hold the six factors
+    const real c0 = lhm[LGL ? 0 : i], c1 = lhp[LGL ? n - 1 : i];
+    const real c2 = LGL ? c0 : lhm[j], c3 = LGL ? c1 : lhp[j], c4 = LGL ? c0 : lhm[k], c5 = LGL ? c1 : lhp[k];
     const int pq0 = j + n * k, pq1 = i + n * k, pq2 = i + n * j;
     const real* Fe = sF + el * 6 * NV * n2;
     const real scale = MODE == 1 ? -(rk.dt * sj) : -sj;
@@ -1616,7 +1619,7 @@ __global__ void __launch_bounds__(Cfg<n>::T * TM, TM > 1 ? 1 : ((sizeof(real) ==
       }
       ut[v] = s * scale;
     }
-    if (src.on) {
+    if (SRC && src.on) {
       const real* p = phase + (size_t)e * 2 * n3 + node;
       const real sdt = MODE == 1 ? rk.dt : real(1);
       real Sv[NV];
@@ -2191,16 +2194,16 @@ static cudaError_t surf_n(const DevMesh& m, int mode, real* U, real* dU, real* U
                           const SourceParams& src, const Ops<real>& ops, const Phys<real>& ph, cudaStream_t st) {
   using C = Cfg<n>;
   const int grid = (m.K + C::NE - 1) / C::NE;
-#define FLEXI_SURF(MODEV, TMV)                                                                                    \
-  k_surf<real, n, MODEV, LGL, TMV><<<grid, C::T * TMV, 0, st>>>((const real*)m.Ff, m.elemSide, (const real*)m.sJ, \
+#define FLEXI_SURF(MODEV, TMV, SRCV)                                                                              \
+  k_surf<real, n, MODEV, LGL, TMV, SRCV><<<grid, C::T * TMV, 0, st>>>((const real*)m.Ff, m.elemSide, (const real*)m.sJ, \
                                                                  (const real*)m.Utv, U, dU, Ut, (real*)m.Wf, (const real*)m.phase, \
                                                                  rk, src, m.K, m.S, ops, ph, m.status)
   if constexpr (n <= 4) {
     if (grid < m.nsm) {  // fewer CTAs than SMs: six times the threads for the face loops
       if (mode == 0)
-        FLEXI_SURF(0, 6);
+        FLEXI_SURF(0, 6, true);
       else
-        FLEXI_SURF(1, 6);
+        FLEXI_SURF(1, 6, true);
       return cudaGetLastError();
     }
   }
@@ -2215,9 +2218,11 @@ static cudaError_t surf_n(const DevMesh& m, int mode, real* U, real* dU, real* U
                                                   ph, m.status);
   } else {
     if (mode == 0)
-      FLEXI_SURF(0, 1);
+      FLEXI_SURF(0, 1, true);
+    else if (src.on)
+      FLEXI_SURF(1, 1, true);
     else
-      FLEXI_SURF(1, 1);
+      FLEXI_SURF(1, 1, false);
   }
 #undef FLEXI_SURF
   return cudaGetLastError();
