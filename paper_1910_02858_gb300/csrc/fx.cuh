@@ -165,16 +165,17 @@ __device__ __forceinline__ fx64 fx_from(double x, int E) {
   return ((fx64)m ^ s) - s;
 }
 
-// r 2^t, rounded to nearest; 0 below the normal range
+// r 2^t, rounded to nearest; below the normal range a value under 2^-1021
 __device__ __forceinline__ double fx_to(fx64 r, int t) {
   const long long s = r >> 63;
   const unsigned long long a = (unsigned long long)((r ^ s) - s);
   const unsigned ahi = (unsigned)(a >> 32), alo = (unsigned)a;
   const int lz = __clz(ahi ? ahi : alo) + (ahi ? 0 : 32);  // >= 1; 64 for zero
   const unsigned long long m = ((a << (lz - 1)) + 0x200) >> 10;
-  const int e = 1086 + t - lz;
-  const unsigned long long b = ((unsigned long long)(unsigned)(e - 1) << 52) + m;
-  return __longlong_as_double((lz == 64 || e < 1) ? 0ll : (long long)(b | ((unsigned long long)s << 63)));
+  // the exponent field joins the high word only; the leading bit of m adds one to it
+  const int e = lz == 64 ? 0 : max(1085 + t - lz, 0);
+  const int hi = ((int)(m >> 32) + (e << 20)) | ((int)s & (int)0x80000000);
+  return __hiloint2double(hi, (int)(unsigned)m);
 }
 
 // a value as v = h 2^32 + l with the low half signed, |l| <= 2^31 (|v| < 2^62)

@@ -5,8 +5,8 @@
 // products of the surface integral and the l(+-1) products of the next face states; at 64
 // clocks per FP64 warp instruction that is 3.5 times the kernel's memory time.  Here they
 // take three integer multiply-adds each; the FP64 pipe keeps the RK update and the
-// primitive face states.  16^3 elements, N = 7: k_surf 297 -> 188 us (268 B per node:
-// 84 us at the measured copy rate), k_prolong 158 -> 87 us.  Elements with values outside the
+// primitive face states.  16^3 elements, N = 7: k_surf 297 -> 181 us (268 B per node:
+// 84 us at the measured copy rate), k_prolong 158 -> 83 us.  Elements with values outside the
 // fixed-point range use the FP64 expressions of k_surf.
 #pragma once
 #include "fx.cuh"
@@ -110,9 +110,11 @@ __global__ void __launch_bounds__(Cfg<n>::T, n >= 7 ? 2 : 4) k_prolong_fx(
   faces_from_volume_fx<n, LGL>(sU, sFace, sMag, ops, fx, sES, e0, K, S, Wf, ph, status, tid, wmask);
 }
 
-// surface integral, -1/J, RK stage update (MODE 1; MODE 0: U_t) and the face states of the new U
+// surface integral, -1/J, RK stage update (MODE 1; MODE 0: U_t) and the face states of the new U.
+// Registers are capped for 1024-1536 resident threads: 24^3 curved elements with a source,
+// N = 7, 3 CTAs against 2 (865 -> 835 us)
 template <int n, int MODE, bool LGL>
-__global__ void __launch_bounds__(Cfg<n>::T, n >= 7 ? 2 : 4) k_surf_fx(
+__global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 3 : (n == 7 ? 4 : (n == 6 ? 6 : 8))) k_surf_fx(
     const double* __restrict__ Ff, const int* __restrict__ elemSide, const double* __restrict__ sJ,
     const double* __restrict__ Utv, double* __restrict__ U, double* __restrict__ dU, double* __restrict__ Ut,
     double* __restrict__ Wf, const double* __restrict__ phase, const RkStage<double> rk, const SourceParams src, int K, int S,
