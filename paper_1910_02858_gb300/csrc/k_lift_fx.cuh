@@ -173,9 +173,10 @@ constexpr size_t lift_fx_smem() {
   return 8 * C::NE * (15 * C::n3p + 48 * C::n2) + 8 * C::n2 + sizeof(int) * C::NE * (12 + 6 * C::n2 + FX_SLOTS + 32);
 }
 
-// CTAs per SM asked of the register allocator (n = 8: two of 512 threads at 64 registers)
+// CTAs per SM asked of the register allocator (n = 8: two of 512 threads at 64 registers;
+// n = 7: three of 343 at 56 against two at 80, 16^3: 657 -> 601 us, affine 453 -> 398 us)
 template <int n>
-constexpr int lift_fx_min_blocks() { return n >= 7 ? 2 : (n == 6 ? 4 : (n == 5 ? 7 : (n == 4 ? 12 : 6))); }
+constexpr int lift_fx_min_blocks() { return n == 8 ? 2 : (n == 7 ? 3 : (n == 6 ? 4 : (n == 5 ? 7 : (n == 4 ? 12 : 6)))); }
 
 // free indices and stride of line `line` along l; offset of its first entry in a field
 template <int n>
