@@ -422,6 +422,7 @@ __device__ __forceinline__ void lift_vol_body(
   int* sSlot = sES + NE * 6;   // [NE][6] side slot (slave * S + side) of each face
   int* sMpq = sSlot + NE * 6;  // [NE][6][n2] master-frame node of each face node
   static_assert(!SPLIT || (LGL && SW == 0), "the split form is built on Gauss-Lobatto nodes with CUDA-core sweeps");
+  static_assert(sizeof(real) == 4 || SPLIT == 2 || BR2, "the other FP64 forms are k_lift_fx.cuh's");
   static_assert(!BR2 || (SW == 0 && !SPLIT), "BR2 face gradients are built for the standard form, CUDA-core sweeps");
 
   const int tid = threadIdx.x;
@@ -788,8 +789,8 @@ __device__ __forceinline__ void lift_vol_body(
         for (int ii = 0; ii < n; ++ii)
 #pragma unroll
           for (int c = 0; c < NV; ++c) o[c * n3p + ii * stride] = real(0);
-        // (the entropy-conservative pair flux is long: keep its loops rolled)
-#pragma unroll(SPLIT == 2 ? 1 : n)
+        // (entropy-conservative pairs, whose flux is long: loops kept rolled)
+#pragma unroll 1
         for (int ii = 0; ii < n; ++ii) {
           const real* fi = f + ii * stride;
           const real ri = fi[0], ui = fi[n3p], vi = fi[2 * n3p], wi = fi[3 * n3p], pi = fi[4 * n3p];
@@ -799,44 +800,22 @@ __device__ __forceinline__ void lift_vol_body(
           for (int c = 0; c < NV; ++c) ai[c] = real(0);
           if (ii == 0 || ii == n - 1) {  // 2 D_ii F#(i, i) = 2 D_ii Fcal^{c,l}(U_i)
             const real dd = real(2) * sD[ii * n + ii];
-            if constexpr (SPLIT == 2) {
-              const real u3[3] = {ui, vi, wi}, J3[3] = {ji0, ji1, ji2};
-              real F[NV];
-              ec_flux(ri, u3, pi, Hi, ri, u3, pi, Hi, J3, ph, F);
+            const real u3[3] = {ui, vi, wi}, J3[3] = {ji0, ji1, ji2};
+            real F[NV];
+            ec_flux(ri, u3, pi, Hi, ri, u3, pi, Hi, J3, ph, F);
 #pragma unroll
-              for (int c = 0; c < NV; ++c) ai[c] = dd * F[c];
-            } else {
-              const real uc = ui * ji0 + vi * ji1 + wi * ji2;
-              const real m = dd * ri * uc;
-              ai[0] = m;
-              ai[1] = m * ui + dd * pi * ji0;
-              ai[2] = m * vi + dd * pi * ji1;
-              ai[3] = m * wi + dd * pi * ji2;
-              ai[4] = m * Hi;
-            }
+            for (int c = 0; c < NV; ++c) ai[c] = dd * F[c];
           }
-#pragma unroll(SPLIT == 2 ? 1 : n)
+#pragma unroll 1
           for (int aa = ii + 1; aa < n; ++aa) {
             const real* fa = f + aa * stride;
             real F0, F1, F2, F3, F4;  // 2 F#(i, a)
-            if constexpr (SPLIT == 2) {
-              const real u3[3] = {ui, vi, wi}, ua3[3] = {fa[n3p], fa[2 * n3p], fa[3 * n3p]};
-              const real Jm[3] = {real(0.5) * (ji0 + fa[jo]), real(0.5) * (ji1 + fa[jo + n3p]),
-                                  real(0.5) * (ji2 + fa[jo + 2 * n3p])};
-              real F[NV];
-              ec_flux(ri, u3, pi, Hi, fa[0], ua3, fa[4 * n3p], fa[5 * n3p], Jm, ph, F);
-              F0 = real(2) * F[0]; F1 = real(2) * F[1]; F2 = real(2) * F[2]; F3 = real(2) * F[3]; F4 = real(2) * F[4];
-            } else {
-              // pair sums (twice the arithmetic means)
-              const real rs = ri + fa[0], us = ui + fa[n3p], vs = vi + fa[2 * n3p], ws = wi + fa[3 * n3p];
-              const real ps = pi + fa[4 * n3p], Hs = Hi + fa[5 * n3p];
-              const real j0 = ji0 + fa[jo], j1 = ji1 + fa[jo + n3p], j2 = ji2 + fa[jo + 2 * n3p];
-              const real m = real(0.125) * rs * (us * j0 + vs * j1 + ws * j2);  // {rho} {u . Ja^l}
-              const real hp = real(0.5) * ps;
-              // 2 F#: mass 2 m; momentum m u_s + (p_s / 2) Ja_s; energy m H_s
-              F0 = real(2) * m; F1 = m * us + hp * j0; F2 = m * vs + hp * j1; F3 = m * ws + hp * j2;
-              F4 = m * Hs;
-            }
+            const real u3[3] = {ui, vi, wi}, ua3[3] = {fa[n3p], fa[2 * n3p], fa[3 * n3p]};
+            const real Jm[3] = {real(0.5) * (ji0 + fa[jo]), real(0.5) * (ji1 + fa[jo + n3p]),
+                                real(0.5) * (ji2 + fa[jo + 2 * n3p])};
+            real F[NV];
+            ec_flux(ri, u3, pi, Hi, fa[0], ua3, fa[4 * n3p], fa[5 * n3p], Jm, ph, F);
+            F0 = real(2) * F[0]; F1 = real(2) * F[1]; F2 = real(2) * F[2]; F3 = real(2) * F[3]; F4 = real(2) * F[4];
             const real dia = sD[aa * n + ii], dai = sD[ii * n + aa];
             ai[0] += dia * F0; ai[1] += dia * F1; ai[2] += dia * F2; ai[3] += dia * F3; ai[4] += dia * F4;
             real* oa = o + aa * stride;
@@ -2134,17 +2113,19 @@ cudaError_t launch_lift_vol(const DevMesh& m, const real* U, const Ops<real>& op
     }
     FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, false, 0, true>(m, U, ops, ph, store_grad, st));
   }
-  if (m.lgl && m.split == 1) {
-    FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, true, 1>(m, U, ops, ph, store_grad, st));
-  }
   if (m.lgl && m.split == 2) {
     FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, true, 2>(m, U, ops, ph, store_grad, st));
   }
-  if (m.lgl) {
-    FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, true>(m, U, ops, ph, store_grad, st));
+  if constexpr (sizeof(real) == 4) {
+    if (m.lgl && m.split == 1) {
+      FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, true, 1>(m, U, ops, ph, store_grad, st));
+    }
+    if (m.lgl) {
+      FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0, true>(m, U, ops, ph, store_grad, st));
+    }
+    FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0>(m, U, ops, ph, store_grad, st));
   }
-  FLEXI_DISPATCH_N(m.n, return lift_vol_n<real, NN, 0>(m, U, ops, ph, store_grad, st));
-  return cudaSuccess;
+  return cudaErrorInvalidValue;  // no other form
 }
 
 template <typename real>
