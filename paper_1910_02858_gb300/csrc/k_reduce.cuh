@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(RED_T, 4) k_reduce(const real* __restrict__ U,
   if (threadIdx.x < RED_Q) partial[(size_t)(1 + blockIdx.x) * RED_Q + 1 + threadIdx.x] = red[threadIdx.x][0];
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) sLast = atomicAdd(arrived, 1u) == gridDim.x - 1;
+  // the count wraps, so it is 0 again after every launch's blocks, whatever runs beside them
+  if (threadIdx.x == 0) sLast = atomicInc(arrived, gridDim.x - 1) == gridDim.x - 1;
   __syncthreads();
   if (!sLast) return;
   __threadfence();
@@ -185,10 +186,7 @@ __global__ void __launch_bounds__(RED_T, 4) k_reduce(const real* __restrict__ U,
   __syncthreads();
   reduce_block(red);
   if (threadIdx.x < RED_Q) partial[threadIdx.x] = red[threadIdx.x][0];
-  if (threadIdx.x == 0) {
-    partial[RED_Q] = (double)*status;
-    *arrived = 0;
-  }
+  if (threadIdx.x == 0) partial[RED_Q] = (double)*status;
 }
 
 template <typename real>
