@@ -45,12 +45,12 @@ def peaks():
         return {}
 
 
-# DRAM bytes (read + write) per launch of the lifting/volume kernel (k_lift_vol_mb) from the ncu captures
+# DRAM bytes (read + write) per launch of the lifting/volume kernel (affine elements) from the ncu captures
 # summarised in profiles/, keyed by form and by a hash of the kernel sources at
 # capture time; reported only while the sources are unchanged (else null).
 KERNEL_SOURCES = ["paper_1910_02858_gb300/csrc/k_dg.cuh", "paper_1910_02858_gb300/csrc/dg_common.cuh",
                   "paper_1910_02858_gb300/csrc/k_tc.cuh", "paper_1910_02858_gb300/csrc/k_adj.cuh"]
-NCU_TRAFFIC = {("fp64", "41f95f6d2cdf1e15"): 574419200, ("fp32", "41f95f6d2cdf1e15"): 266935296}
+NCU_TRAFFIC = {("fp64", "00797a78b72715c4"): 380981248, ("fp32", "00797a78b72715c4"): 154781184}
 
 
 def kernel_source_hash(texts=None) -> str:
@@ -77,6 +77,14 @@ def kernel_source_hash(texts=None) -> str:
 FP64_PEAK_TFLOPS = 152 * 4 * 2.070e9 / 1e12
 # FP32 FMA peak from the same unit counts: 128 FP32 lanes x 2 flop/clk per SM
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
+
+
+def step_floor_ns(s, dof, fp64: bool, F) -> float:
+    """Nanoseconds per DOF and stage that the algorithmic bytes take at the measured HBM
+    bandwidth and, in the FP32 forms, the algorithmic flops at the FP32 peak.  The FP64 form
+    contracts in integers, so its flop count over the FP64 pipe's peak is no floor."""
+    t_mem = s.query(F.Q_BYTES_PER_STAGE) / dof / peaks().get("hbm_gbs", 6800.0)
+    return t_mem if fp64 else max(t_mem, s.query(F.Q_FLOPS_PER_STAGE) / dof / (FP32_PEAK_TFLOPS * 1e3))
 
 
 class ClockSampler:
@@ -412,8 +420,8 @@ def main():
     ms_step = ms_total / args.steps
     pid = whole_job_pid(ms_total * 1e-3, args.steps, dof, world)
 
-    # roofline of the dominant kernel (lifting + volume): FP64 form ALU-bound (FP64 pipe),
-    # FP32 forms HBM-bound
+    # roofline of the dominant kernel (lifting + volume) against HBM; instruction issue is what
+    # holds it (profiles/)
     n = N + 1
     word = 8 if args.form == "fp64" else 4
     bytes_stage, bytes_lv, flops_lv = algorithmic_per_dof(n, word)
@@ -421,32 +429,26 @@ def main():
     lv_avg_s = lv_ms / max(lv_cnt, 1) * 1e-3
     share = lv_ms / max(sum(v[0] for v in ktimes.values()), 1e-9)
     traffic = NCU_TRAFFIC.get((args.form, kernel_source_hash()))
-    if args.form == "fp64":
-        achieved_tflops = flops_lv * dof / lv_avg_s / 1e12
-        roofline = {"bound": "alu", "achieved": achieved_tflops, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                    "frac": achieved_tflops / FP64_PEAK_TFLOPS, "traffic": traffic, "kernel": "k_lift_vol_mb<double,8>",
-                    "peak_source": "derived: 152 SM x 4 FP64 flop/clk x 2070 MHz (nominal 1.25 TFLOP/s)",
-                    "kernel_share": share}
-    else:
-        hbm = peaks().get("hbm_gbs", 6800.0)
-        achieved = bytes_lv * dof / lv_avg_s / 1e9
-        roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                    "traffic": traffic,
-                    # k_lift_vol_mb: the instance with a minimum of resident CTAs per SM
-                    "kernel": "k_lift_vol_mb<float,8>" if args.form == "fp32" else f"k_lift_vol<float,8,{args.form}>",
-                    "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks() else "fallback 6.8 TB/s",
-                    "kernel_share": share}
+    hbm = peaks().get("hbm_gbs", 6800.0)
+    achieved = bytes_lv * dof / lv_avg_s / 1e9
+    roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
+                "traffic": traffic,
+                # the workload's elements are affine
+                "kernel": "k_lift_vol_fx_affine<8>" if args.form == "fp64" else f"k_lift_vol_f32_affine<8,{args.form}>",
+                "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks() else "fallback 6.8 TB/s",
+                "kernel_share": share}
+    if args.form == "fp64":  # above 1: the contractions are not on the FP64 pipe
+        roofline["flops_over_fp64_pipe_peak"] = flops_lv * dof / lv_avg_s / 1e12 / FP64_PEAK_TFLOPS
     step_bytes_gbs = bytes_stage * dof * NSTAGES / (ms_step * 1e-3) / 1e9
-    # whole-step roofline: the slower of the step's algorithmic bytes over the measured HBM
-    # bandwidth and its algorithmic flops at the form's FMA peak (the library's own counts)
+    # whole-step roofline (step_floor_ns; the library's own counts)
     bps = s.query(F.Q_BYTES_PER_STAGE) / dof
     fps = s.query(F.Q_FLOPS_PER_STAGE) / dof
-    fpk = FP64_PEAK_TFLOPS if args.form == "fp64" else FP32_PEAK_TFLOPS
-    t_mem, t_alu = bps / peaks().get("hbm_gbs", 6800.0), fps / (fpk * 1e3)  # ns per DOF and stage
-    step_roofline = {"bound": "alu" if t_alu > t_mem else "hbm", "floor_ns": max(t_mem, t_alu),
-                     "achieved_ns": pid * world, "frac": max(t_mem, t_alu) / (pid * world),
-                     "bytes_per_dof": bps, "flops_per_dof": fps, "alu_peak_tflops": fpk,
-                     "alu_peak_source": "derived from unit counts at 2070 MHz"}
+    floor = step_floor_ns(s, dof, args.form == "fp64", F)
+    step_roofline = {"bound": "hbm" if floor == bps / hbm else "alu", "floor_ns": floor,
+                     "achieved_ns": pid * world, "frac": floor / (pid * world),
+                     "bytes_per_dof": bps, "flops_per_dof": fps}
+    if args.form != "fp64":
+        step_roofline.update(alu_peak_tflops=FP32_PEAK_TFLOPS, alu_peak_source="derived from unit counts at 2070 MHz")
     kernels = {k: {"ms_per_launch": (v[0] / v[1]) if v[1] else 0.0, "launches": v[1]} for k, v in ktimes.items() if v[1]}
 
     # end to end through the public API with host buffers (H2D + step + D2H per step)
@@ -527,8 +529,7 @@ def extras(args, s64, U0, mesh, dt, dev, F, wl, Solver, SolverConfig, torch, np)
             bytes_stage = (46.0 + 117.0 * 3.0 / n) * 4 * dof
             lv = kt["lift_vol"][0] / max(kt["lift_vol"][1], 1)
             pid32 = ms * 1e6 / (nsteps * NSTAGES * dof)
-            floor = max(s.query(F.Q_BYTES_PER_STAGE) / dof / peaks().get("hbm_gbs", 6800.0),
-                        s.query(F.Q_FLOPS_PER_STAGE) / dof / (FP32_PEAK_TFLOPS * 1e3))
+            floor = step_floor_ns(s, dof, False, F)
             out[name] = {"pid": pid32, "step_roofline_frac": floor / pid32, "steps": nsteps,
                          "rel_l2_err_vs_fp64": rel_err_per_var(U, U64),
                          "step_algorithmic_hbm_gbs": bytes_stage * NSTAGES * nsteps / (ms * 1e-3) / 1e9,
@@ -622,20 +623,14 @@ def c4_curved_pid(dev, F, wl, Solver, SolverConfig, torch):
                 ms, kt = timed_steps(s, U, dU, dt, nsteps, F, torch, dev)
                 dof = s.query(F.Q_DOF)
                 pid = ms * 1e6 / (nsteps * NSTAGES * dof)
-                fpk = FP64_PEAK_TFLOPS if prec == F.FP64 else FP32_PEAK_TFLOPS
-                floor = max(s.query(F.Q_BYTES_PER_STAGE) / dof / peaks().get("hbm_gbs", 6800.0),
-                            s.query(F.Q_FLOPS_PER_STAGE) / dof / (fpk * 1e3))
+                floor = step_floor_ns(s, dof, prec == F.FP64, F)
                 tot = sum(v[0] for v in kt.values())
                 lv = kt["lift_vol"][0] / max(kt["lift_vol"][1], 1)
                 row = {"dof": dof, "dt": dt, "steps": nsteps, "pid": pid, "step_roofline_frac": floor / pid,
                        "floor_ns": floor, "lift_vol_ms_per_launch": lv,
                        "lift_vol_share": kt["lift_vol"][0] / tot if tot > 0 else None}
-                if prec == F.FP64:
-                    row["lift_vol_alu_frac"] = (algorithmic_per_dof(N + 1, 8)[2] * dof / (lv * 1e-3) / 1e12
-                                                / FP64_PEAK_TFLOPS)
-                else:
-                    row["lift_vol_hbm_frac"] = (algorithmic_per_dof(N + 1, 4)[1] * dof / (lv * 1e-3) / 1e9
-                                                / peaks().get("hbm_gbs", 6800.0))
+                row["lift_vol_hbm_frac"] = (algorithmic_per_dof(N + 1, 8 if prec == F.FP64 else 4)[1] * dof / (lv * 1e-3)
+                                            / 1e9 / peaks().get("hbm_gbs", 6800.0))
                 if case == "freestream":
                     # 2 * nsteps steps were taken from U0 (timed + profiled pass)
                     U0d = torch.tensor(U0, device=dev, dtype=s.dtype)
@@ -675,9 +670,7 @@ def c3_forms_pid(dev, F, wl, Solver, SolverConfig, torch):
             torch.cuda.synchronize(dev)
             dof = s.query(F.Q_DOF)
             pid = e0.elapsed_time(e1) * 1e6 / (nsteps * NSTAGES * dof)
-            fpk = FP64_PEAK_TFLOPS if prec == F.FP64 else FP32_PEAK_TFLOPS
-            floor = max(s.query(F.Q_BYTES_PER_STAGE) / dof / peaks().get("hbm_gbs", 6800.0),
-                        s.query(F.Q_FLOPS_PER_STAGE) / dof / (fpk * 1e3))
+            floor = step_floor_ns(s, dof, prec == F.FP64, F)
             res[name] = {"pid": pid, "step_roofline_frac": floor / pid, "steps": nsteps, "dt": dt}
             red = s.reduce(U, s.rhs(U))
             if ref is None:
