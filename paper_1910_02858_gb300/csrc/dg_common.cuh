@@ -542,24 +542,42 @@ __device__ __forceinline__ void exact_state(int kind, const double x[3], double 
 // differentiation in the tests).  s0, c0: sine and cosine of pi (x + y + z), which belong to
 // the mesh; sin and cos of the phase pi (x + y + z - 2t) follow by turning them by 2 pi t
 // (an FP64 sincos per node cost as much as the rest of the surface kernel: 24^3 curved
-// elements, N = 7, 1747 -> 924 us per stage with k_surf_fx).
+// elements, N = 7, 1746 -> 696 us per stage with k_surf_fx).
+// The constants are formed on the host in both widths: per thread their FP64 division and
+// conversions cost more than the term itself (surface kernel of that case 835 -> 696 us, FP32 162 us).
 struct SourceParams {
   int on = 0;
   double gamma = 1.4, mu = 0, Pr = 0.72;
-  double st = 0, ct = 1;  // sine and cosine of 2 pi t, set per launch
+  // gamma - 1, 3 lambda pi^2 A of the heat flux, sine and cosine of 2 pi t; set per launch
+  struct {
+    double f64[4] = {0, 0, 0, 1};
+    float f32[4] = {0, 0, 0, 1};
+  } k;
+  void at(double sine, double cosine) {
+    const double v[4] = {gamma - 1.0, 3.0 * (mu * gamma / Pr) * M_PI * M_PI * 0.1, sine, cosine};
+    for (int i = 0; i < 4; ++i) {
+      k.f64[i] = v[i];
+      k.f32[i] = (float)v[i];
+    }
+  }
 };
 
 template <typename real>
 __device__ __forceinline__ void manufactured_source(real s0, real c0, const SourceParams& q, real S[NV]) {
-  const real A = real(0.1), pi = real(M_PI), g1 = real(q.gamma - 1.0);
-  const real st = real(q.st), ct = real(q.ct);
+  const real A = real(0.1), pi = real(M_PI);
+  real g1, heat, st, ct;
+  if constexpr (sizeof(real) == 4) {
+    g1 = q.k.f32[0]; heat = q.k.f32[1]; st = q.k.f32[2]; ct = q.k.f32[3];
+  } else {
+    g1 = q.k.f64[0]; heat = q.k.f64[1]; st = q.k.f64[2]; ct = q.k.f64[3];
+  }
   const real s = s0 * ct - c0 * st, c = c0 * ct + s0 * st;
   const real rho = real(2) + A * s;
   const real dr = pi * A * c;  // d rho / dx (= dy = dz); d rho/dt = -2 dr
   const real dpx = g1 * (real(2) * rho - real(1.5)) * dr;
   S[0] = dr;
   S[1] = S[2] = S[3] = dr + dpx;
-  S[4] = real(2) * rho * dr + real(3) * dpx + real(3.0 * (q.mu * q.gamma / q.Pr) * M_PI * M_PI * 0.1) * s;
+  S[4] = real(2) * rho * dr + real(3) * dpx + heat * s;
 }
 
 }  // namespace flexi

@@ -165,8 +165,7 @@ const Phys<float>& ph_of<float>(const flexi_ctx* c) { return c->ph32; }
 SourceParams source_at(const flexi_ctx* c, double t) {
   SourceParams q = c->src;
   const double a = M_PI * std::fmod(2.0 * t, 2.0);
-  q.st = std::sin(a);
-  q.ct = std::cos(a);
+  q.at(std::sin(a), std::cos(a));
   return q;
 }
 

@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n >= 7 ? 2 : 4) k_prolong_fx(
 
 // surface integral, -1/J, RK stage update (MODE 1; MODE 0: U_t) and the face states of the new U.
 // Registers are capped for 1024-1536 resident threads: 24^3 curved elements with a source,
-// N = 7, 3 CTAs against 2 (865 -> 835 us)
+// N = 7, 3 CTAs against 2: 865 -> 835 us (696 with the source constants formed on the host)
 template <int n, int MODE, bool LGL>
 __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 3 : (n == 7 ? 4 : (n == 6 ? 6 : 8))) k_surf_fx(
     const double* __restrict__ Ff, const int* __restrict__ elemSide, const double* __restrict__ sJ,
