@@ -1,12 +1,14 @@
 // Lifting and volume integral of the FP64 form with the line contractions in block
-// fixed point (fx.cuh).  Standard volume integral, BR1.
+// fixed point (fx.cuh).  Standard and kinetic-energy-preserving volume integral, BR1.
 //
-// The FP64 body (lift_vol_body) is bound by the FP64 pipe: of its 850 FP64 instructions
+// With FP64 sweeps the kernel is bound by the FP64 pipe: of its 850 FP64 instructions
 // per node (n = 8, Gauss) 480 are D_hat multiply-adds, 90 lifting face terms, 90 gradient
 // prolongation and 90 metric products.  All of those are sums of products under one scale
 // and run here on the integer pipes; the FP64 pipe keeps the primitive variables, the
 // surface means and the pointwise fluxes.  Elements whose values leave the fixed-point
-// range (above 2^200, infinities, NaN) take the FP64 body.
+// range (above 2^200, infinities, NaN) take the FP64 schedule of lift_vol_fp64.  16^3 elements,
+// N = 7: 3061 -> 751 us (curved), 566 us (affine; 77 FP64 and 3,760 integer instructions per
+// node, bound by their issue); 638 MB are 95 us at the measured copy rate.
 #pragma once
 #include "fx.cuh"
 
@@ -656,7 +658,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
 // constants of the element, so the lifting contracts the 5 primitive variables along the 3
 // directions (15 line fields instead of 45) and combines the results with J^l_d / J, the face
 // terms of a line are the face means themselves (n_d s_hat = +-Ja^l_d on both ends), and no
-// metric term is read per node.  16^3 elements, N = 7: 757 -> 579 us.
+// metric term is read per node.  16^3 elements, N = 7: 751 -> 566 us.
 // ---------------------------------------------------------------------------
 template <int n>
 constexpr size_t lift_affine_smem() {
