@@ -15,9 +15,9 @@
 namespace flexi {
 
 // slots of an element's magnitude table: primitive variables (nodes and face means), metric
-// terms by physical direction (nodes and faces), 1/J, fluxes by variable, projected lifting
-// fluxes of mortar sides (v*3+d)
-enum { FX_W = 0, FX_J = 5, FX_S = 8, FX_F = 9, FX_Q = 16, FX_SLOTS = 32 };
+// terms by physical direction (nodes and faces; affine elements J^l_d / J), 1/J (affine
+// elements J^l_d by direction), fluxes at d*5+v, projected lifting fluxes of mortar sides (v*3+d)
+enum { FX_W = 0, FX_J = 5, FX_S = 8, FX_F = 11, FX_Q = 26, FX_SLOTS = 42 };
 // largest exponent fields that the fixed-point kernel takes: products of four such values
 // stay inside the FP64 range
 constexpr int FX_MAX_EXP = 1022 + 200, FX_MAX_FLUX = 1022 + 600;
@@ -189,10 +189,36 @@ __device__ __forceinline__ int fx_line_at(int l, int line, int& stride) {
   return l == 0 ? P * line : (l == 1 ? a0 + P * n * a1 : a0 + P * a1);
 }
 
+// Scale of the fluxes of variables v >= V0: their largest magnitude words at FX_F + d*5+v
+// become the exponents under which F_d,v is converted, x_v - E(Ja_d), where x_v is the largest
+// of E(F_d,v) + E(Ja_d).  False when a flux leaves the fixed-point range.  Block-wide; synced.
+template <int NE, int T, int V0>
+__device__ __forceinline__ bool flux_exponents(int* sMag, int JS) {
+  int bad = 0;
+  for (int t = threadIdx.x; t < NE * (NV - V0); t += T) {
+    int* m = sMag + (t / (NV - V0)) * FX_SLOTS;
+    int* f = m + FX_F + V0 + t % (NV - V0);
+    int x = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      bad |= (f[d * NV] >> 20) > FX_MAX_FLUX;
+      x = max(x, (f[d * NV] >> 20) + (m[JS + d] >> 20));
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) f[d * NV] = x - (m[JS + d] >> 20);
+  }
+  return !__syncthreads_or(bad);
+}
+
 // a6, a7: physical fluxes in FP64, contravariant fluxes and the volume integral in fixed
-// point.  metric(ji, EJm): the node's nine metric terms under one exponent.  False, with
-// nothing written, when a flux leaves the fixed-point range.  Block-wide.
-template <int n, bool LGL, typename Metric>
+// point.  metric(ji): the node's nine metric terms, direction d under the exponent of slot
+// JS + d.  A variable's three fluxes are scaled by direction: in a flat element the flux
+// through the large area may be far smaller than the others and still decide the sum, so
+// F_d is taken to the scale at which its product with the largest |Ja^l_d| meets the largest
+// such product of the three directions (one exponent for all three lost a digit of U_t per
+// factor ten of aspect ratio against FP64).  False, with nothing written, when a flux leaves
+// the fixed-point range.  Block-wide.
+template <int n, bool LGL, int JS, typename Metric>
 __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* __restrict__ Utv, const double (&W)[NV],
                                           const double (&G)[15], int K, int grp, unsigned wmask, fx64* sA, int* sMag,
                                           const FxOps& fx, const Phys<double>& ph, Metric metric) {
@@ -210,35 +236,26 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
 #pragma unroll
       for (int v = 0; v < NV; ++v) Uo[v] = U[((size_t)e * NV + v) * n3 + node];
     }
-    int mx[NV] = {0, 0, 0, 0, 0};
     const double ir = 1.0 / Uo[0];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       double F[NV];
       flux_total(Uo, W, ir, G, d, ph, F);
 #pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        own[(d * NV + v) * n3p] = __double_as_longlong(F[v]);
-        mx[v] = max(mx[v], fx_mag(F[v]));
-      }
+      for (int v = 0; v < NV; ++v) own[(d * NV + v) * n3p] = __double_as_longlong(F[v]);
+      fx_max<NE == 1, NV>(mag + FX_F + d * NV, wmask, [&](int s) { return fx_mag(F[s]); });
     }
-    fx_max<NE == 1, NV>(mag + FX_F, wmask, [&](int s) { return mx[s]; });
   }
   __syncthreads();
-  {
-    int bad = 0;
-    for (int t = tid; t < NE * NV; t += T) bad |= (sMag[(t / NV) * FX_SLOTS + FX_F + t % NV] >> 20) > FX_MAX_FLUX;
-    if (__syncthreads_or(bad)) return false;
-  }
-  int EJm;
+  if (!flux_exponents<NE, T, 0>(sMag, JS)) return false;
   {
     FxSplit ji[9];
-    metric(ji, EJm);
+    metric(ji);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       FxSplit F[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) F[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FX_F + v] >> 20));
+      for (int d = 0; d < 3; ++d) F[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FX_F + d * NV + v]));
 #pragma unroll
       for (int l = 0; l < 3; ++l) {
         FxAcc s;
@@ -261,7 +278,8 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const fx64* r = own + v * n3p;
-      Utv[((size_t)e * NV + v) * n3 + node] = fx_to(r[0] + r[NV * n3p] + r[2 * NV * n3p], (mag[FX_F + v] >> 20) + EJm - 2044 + 6 - fx.kc);
+      Utv[((size_t)e * NV + v) * n3 + node] =
+          fx_to(r[0] + r[NV * n3p] + r[2 * NV * n3p], mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx.kc);
     }
   }
   return true;
@@ -271,10 +289,12 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
 // advective part 2 sum_a D_ia F#(i, a) with one thread per node over its 3 (n - 1) pairs, in
 // fixed point: pair sums and their products replace 21 FP64 multiply-adds per pair.  The
 // diagonal terms 2 D_ii F(U_i) and the strong form's face terms -(+-1) l_hat(+-1) F(U_i) cancel
-// (2 w_i D_ii = +-1 at the ends, 0 inside), so neither is formed.  Scales: rho, (u, v, w),
-// H and Ja each under one power of two; p and the mass flux times velocity share one (sh).
+// (2 w_i D_ii = +-1 at the ends, 0 inside), so neither is formed.  Scales: rho, p, H and, by
+// direction, the velocity and Ja each under a power of two of their own.  Their products meet
+// at the largest of them: the mass flux at 2^bC, the largest of |u_d| |Ja_d|, momentum d at the
+// larger of mass flux times u_d and p Ja_d (shifts sc, sm, sp of the smaller operands).
 // 990 elements, N = 7: 1130 -> 232 us with the lifting.
-template <int n, bool AFF, typename Metric>
+template <int n, bool AFF, int JS, typename Metric>
 __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, double* __restrict__ Utv, const double (&W)[NV],
                                                 const double (&G)[15], int K, int grp, unsigned wmask, fx64* sA, int* sMag,
                                                 int2* sD, const FxOps& fx, const FxStrong& fd, const Phys<double>& ph,
@@ -293,38 +313,33 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
     if (valid) E = U[((size_t)e * NV + 4) * n3 + node];
     const double ir = 1.0 / W[0];
     H = (E + W[4]) * ir;
-    int mx[NV] = {0, 0, 0, 0, 0};  // slot 0: H, 1-4: viscous flux
-    mx[0] = fx_mag(H);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       double F[NV];
       flux_viscous(W, ir, G, d, ph, F);
+      F[0] = H;  // slots of the first variable: H
 #pragma unroll
-      for (int v = 1; v < NV; ++v) {
-        own[(d * NV + v) * n3p] = __double_as_longlong(-F[v]);
-        mx[v] = max(mx[v], fx_mag(F[v]));
-      }
+      for (int v = 1; v < NV; ++v) own[(d * NV + v) * n3p] = __double_as_longlong(-F[v]);
+      fx_max<NE == 1, NV>(mag + FX_F + d * NV, wmask, [&](int s) { return fx_mag(F[s]); });
     }
-    fx_max<NE == 1, NV>(mag + FX_F, wmask, [&](int s) { return mx[s]; });
   }
   for (int t = tid; t < n2; t += T) sD[t] = make_int2(fd.h[t], fd.l[t]);
   __syncthreads();
   {
     int bad = 0;
-    for (int t = tid; t < NE * NV; t += T)
-      bad |= (sMag[(t / NV) * FX_SLOTS + FX_F + t % NV] >> 20) > (t % NV == 0 ? FX_MAX_EXP + 200 : FX_MAX_FLUX);
+    for (int t = tid; t < NE; t += T) bad |= (sMag[t * FX_SLOTS + FX_F] >> 20) > FX_MAX_EXP + 200;
     if (__syncthreads_or(bad)) return false;
   }
-  int EJm;
+  if (!flux_exponents<NE, T, 1>(sMag, JS)) return false;
   double vis[NV];
   {
     FxSplit ji[9];
-    metric(ji, EJm);
+    metric(ji);
 #pragma unroll
     for (int v = 1; v < NV; ++v) {
       FxSplit F[3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d) F[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FX_F + v] >> 20));
+      for (int d = 0; d < 3; ++d) F[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FX_F + d * NV + v]));
 #pragma unroll
       for (int l = 0; l < 3; ++l) {
         FxAcc s;
@@ -347,23 +362,33 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
   vis[0] = 0.0;
 #pragma unroll
   for (int v = 1; v < NV; ++v)
-    vis[v] = fx_to(own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p], (mag[FX_F + v] >> 20) + EJm - 2044 + 6 - fx.kc);
-  // advective part: bounds b of rho, velocity, Ja, H, p as powers of two
-  const int bR = (mag[FX_W] >> 20) - 1022, bJ = EJm - 1022, bH = (mag[FX_F] >> 20) - 1022;
-  const int bU = (max(mag[FX_W + 1], max(mag[FX_W + 2], mag[FX_W + 3])) >> 20) - 1022;
-  const int sh = min(max(0, (mag[FX_W + 4] >> 20) - 1022 - (bR + 2 * bU + 2)), 62);  // shift of m against p
-  const int bP = max(bR + 2 * bU + 2 + sh, (mag[FX_W + 4] >> 20) - 1022);
+    vis[v] = fx_to(own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p],
+                   mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx.kc);
+  // advective part: bounds b of rho, H, p, mass flux and momentum flux as powers of two
+  const int bR = (mag[FX_W] >> 20) - 1022, bH = (mag[FX_F] >> 20) - 1022, bP = (mag[FX_W + 4] >> 20) - 1022;
+  int bC = -4096;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) bC = max(bC, (mag[FX_W + 1 + d] >> 20) + (mag[JS + d] >> 20) - 2044);
+  int sc[3], sm[3], sp[3], bM[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int bU = (mag[FX_W + 1 + d] >> 20) - 1022, bJ = (mag[JS + d] >> 20) - 1022;
+    bM[d] = max(bP + bJ, bR + bC + bU + 2);
+    sc[d] = min(bC - bU - bJ, 62);
+    sm[d] = min(bM[d] - (bR + bC + bU + 2), 62);
+    sp[d] = min(bM[d] - (bP + bJ), 62);
+  }
   fx64 q[6];
   q[0] = fx_from<60>(W[0], bR + 1022);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) q[1 + d] = fx_from<60>(W[1 + d], bU + 1022);
+  for (int d = 0; d < 3; ++d) q[1 + d] = fx_from<60>(W[1 + d], mag[FX_W + 1 + d] >> 20);
   q[4] = fx_from<60>(W[4], bP + 1022);
   q[5] = fx_from<60>(H, bH + 1022);
 #pragma unroll
   for (int c = 0; c < 6; ++c) own[c * n3p] = q[c];
   {
     FxSplit ji[9];
-    metric(ji, EJm);
+    metric(ji);
     if constexpr (!AFF) {
 #pragma unroll
       for (int c = 0; c < 9; ++c) own[(6 + c) * n3p] = fx_shr(((fx64)ji[c].h << 32) + ji[c].l, 2);
@@ -386,49 +411,46 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
       a = a + 1 == n ? 0 : a + 1;
       const fx64* f = own + (a - il) * stride;
       const FxSplit u = fx_split(q[1] + f[n3p]), v = fx_split(q[2] + f[2 * n3p]), w = fx_split(q[3] + f[3 * n3p]);
-      FxSplit j0, j1, j2;
-      if constexpr (AFF) {
-        j0 = fx_split(J0);
-        j1 = fx_split(J1);
-        j2 = fx_split(J2);
-      } else {
+      fx64 j0 = J0, j1 = J1, j2 = J2;
+      if constexpr (!AFF) {
         const fx64* jp = f + (6 + 3 * l) * n3p;
-        j0 = fx_split(J0 + jp[0]);
-        j1 = fx_split(J1 + jp[n3p]);
-        j2 = fx_split(J2 + jp[2 * n3p]);
+        j0 += jp[0];
+        j1 += jp[n3p];
+        j2 += jp[2 * n3p];
       }
       FxAcc c;
-      c.add(u, j0);
-      c.add(v, j1);
-      c.add(w, j2);
+      c.add(u, fx_split(j0 >> sc[0]));
+      c.add(v, fx_split(j1 >> sc[1]));
+      c.add(w, fx_split(j2 >> sc[2]));
       const fx64 mi = fx_mul(fx_split(q[0] + f[0]), fx_split(c.get() << 2));  // 8 {rho}{u . Ja} in its units
-      const FxSplit m4 = fx_split(mi << 2), ms = fx_split((mi << 2) >> sh), p = fx_split(q[4] + f[4 * n3p]);
+      const fx64 m4 = mi << 2;
+      const FxSplit p = fx_split(q[4] + f[4 * n3p]);
       const int2 D = sD[a * n + il];
       const FxSplit d{D.x, D.y};
       s[0].add(fx_split(mi), d);
       FxAcc x;
-      x.add(ms, u);
-      x.add(p, j0);
+      x.add(fx_split(m4 >> sm[0]), u);
+      x.add(p, fx_split(j0 >> sp[0]));
       s[1].add(fx_split(x.get()), d);
       x = FxAcc();
-      x.add(ms, v);
-      x.add(p, j1);
+      x.add(fx_split(m4 >> sm[1]), v);
+      x.add(p, fx_split(j1 >> sp[1]));
       s[2].add(fx_split(x.get()), d);
       x = FxAcc();
-      x.add(ms, w);
-      x.add(p, j2);
+      x.add(fx_split(m4 >> sm[2]), w);
+      x.add(p, fx_split(j2 >> sp[2]));
       s[3].add(fx_split(x.get()), d);
-      s[4].add(fx_split(fx_mul(m4, fx_split(q[5] + f[5 * n3p]))), d);
+      s[4].add(fx_split(fx_mul(fx_split(m4), fx_split(q[5] + f[5 * n3p]))), d);
     }
 #pragma unroll
     for (int v = 0; v < NV; ++v) sum[v] += s[v].get();
   }
   if (valid) {
-    const int t0 = bR + bU + bJ + 64 - fd.k;
+    const int t0 = bR + bC + 64 - fd.k;
     double* out = Utv + (size_t)e * NV * n3 + node;
     out[0] = fx_to(sum[0], t0 - 56);
 #pragma unroll
-    for (int v = 1; v < 4; ++v) out[(size_t)v * n3] = vis[v] + fx_to(sum[v], bP + bJ - 57 + 64 - fd.k);
+    for (int v = 1; v < 4; ++v) out[(size_t)v * n3] = vis[v] + fx_to(sum[v], bM[v - 1] - 57 + 64 - fd.k);
     out[(size_t)4 * n3] = vis[4] + fx_to(sum[4], t0 + bH - 55);
   }
   return true;
@@ -637,17 +659,16 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
     __syncthreads();
   }
   if (Utv == nullptr) return;  // the adjoint's recompute needs the gradients only
-  auto metric = [&](FxSplit (&ji)[9], int& EJm) {
-    EJm = max(mag[FX_J], max(mag[FX_J + 1], mag[FX_J + 2])) >> 20;
+  auto metric = [&](FxSplit (&ji)[9]) {
 #pragma unroll
     for (int c = 0; c < 9; ++c)
-      ji[c] = fx_split(fx_from<62>(valid ? Ja[((size_t)e * 9 + c) * n3 + node] : 0.0, EJm));
+      ji[c] = fx_split(fx_from<62>(valid ? Ja[((size_t)e * 9 + c) * n3 + node] : 0.0, mag[FX_J + c % 3] >> 20));
   };
   bool done;
   if constexpr (KEP)
-    done = split_volume_fx<n, false>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
+    done = split_volume_fx<n, false, FX_J>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
   else
-    done = volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
+    done = volume_fx<n, LGL, FX_J>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
   if (!done)
     lift_vol_fp64<n, LGL, KEP>(U, Ja, sJ, Wf, fgeo, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph, reinterpret_cast<double*>(sA),
                           reinterpret_cast<double*>(sW), sES, sMpq, grp);
@@ -690,8 +711,8 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   int* sES = reinterpret_cast<int*>(sD) - NE * (12 + 6 * n2 + FX_SLOTS + 4);
   int* sSlot = sES + NE * 6;
   int* sMpq = sSlot + NE * 6;          // [NE][6][n2] master-frame node of each face node
-  int* sMag = sMpq + NE * 6 * n2;      // [NE][FX_SLOTS] largest magnitude words; FX_J + d: of J^l_d / J; FX_S: of J^l_d
-  fx64* sM = sW + NE * 30 * n2;        // [NE][2][9] J^l_d / J (exponent by d) and J^l_d (one exponent)
+  int* sMag = sMpq + NE * 6 * n2;      // [NE][FX_SLOTS] largest magnitude words
+  fx64* sM = sW + NE * 30 * n2;        // [NE][2][9] J^l_d / J and J^l_d, exponents by d
   const int tid = threadIdx.x;
   const int el = tid / n3, node = tid - el * n3;
   const int e0 = grp * NE, e = e0 + el;
@@ -721,9 +742,8 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
     int big = 0, md = 0;
     double m[3];
 #pragma unroll
-    for (int c = 0; c < 9; ++c) big = max(big, fx_mag(a[c]));
-#pragma unroll
     for (int l = 0; l < 3; ++l) {
+      big = max(big, fx_mag(a[l * 3 + d]));
       m[l] = a[l * 3 + d] * a[9];
       md = max(md, fx_mag(m[l]));
     }
@@ -733,7 +753,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
       sM[el2 * 18 + 9 + l * 3 + d] = fx_from<62>(a[l * 3 + d], big >> 20);
     }
     sMag[el2 * FX_SLOTS + FX_J + d] = md;
-    if (d == 0) sMag[el2 * FX_SLOTS + FX_S] = big;
+    sMag[el2 * FX_SLOTS + FX_S + d] = big;
   }
   int mW[NV];
 #pragma unroll
@@ -855,16 +875,15 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   }
   if (Utv == nullptr) return;
   __syncthreads();
-  auto metric = [&](FxSplit (&ji)[9], int& EJm) {
-    EJm = mag[FX_S] >> 20;
+  auto metric = [&](FxSplit (&ji)[9]) {
 #pragma unroll
     for (int c = 0; c < 9; ++c) ji[c] = fx_split(sM[el * 18 + 9 + c]);
   };
   bool done;
   if constexpr (KEP)
-    done = split_volume_fx<n, true>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
+    done = split_volume_fx<n, true, FX_S>(U, Utv, W, G, K, grp, wmask, sA, sMag, sD, fx, fd, ph, metric);
   else
-    done = volume_fx<n, LGL>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
+    done = volume_fx<n, LGL, FX_S>(U, Utv, W, G, K, grp, wmask, sA, sMag, fx, ph, metric);
   if (!done)
     fp64();
 }
