@@ -176,9 +176,13 @@ constexpr size_t lift_fx_smem() {
 }
 
 // CTAs per SM asked of the register allocator (n = 8: two of 512 threads at 64 registers;
-// n = 7: three of 343 at 56 against two at 80, 16^3: 657 -> 601 us, affine 453 -> 398 us)
-template <int n>
-constexpr int lift_fx_min_blocks() { return n == 8 ? 2 : (n == 7 ? 3 : (n == 6 ? 4 : (n == 5 ? 7 : (n == 4 ? 12 : 6)))); }
+// n = 7: three of 343 at 56 against two at 80, 16^3: 657 -> 601 us, affine 453 -> 398 us; the
+// pairs of the split form want the registers: 14^3 curved, N = 6, 647 -> 627 us with two, 18^3
+// curved, N = 4, 367 -> 343 us with six of 125 threads instead of seven)
+template <int n, bool KEP>
+constexpr int lift_fx_min_blocks() {
+  return n == 8 ? 2 : (n == 7 ? (KEP ? 2 : 3) : (n == 6 ? 4 : (n == 5 ? (KEP ? 6 : 7) : (n == 4 ? 12 : 6))));
+}
 
 // free indices and stride of line `line` along l; offset of its first entry in a field
 template <int n>
@@ -378,12 +382,13 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
     sm[d] = min(bM[d] - (bR + bC + bU + 2), 62);
     sp[d] = min(bM[d] - (bP + bJ), 62);
   }
+  const bool shift_p = (sp[0] | sp[1] | sp[2]) != 0;
   fx64 q[6];
-  q[0] = fx_from<60>(W[0], bR + 1022);
+  q[0] = fx_from<61>(W[0], bR + 1022);
 #pragma unroll
   for (int d = 0; d < 3; ++d) q[1 + d] = fx_from<60>(W[1 + d], mag[FX_W + 1 + d] >> 20);
   q[4] = fx_from<60>(W[4], bP + 1022);
-  q[5] = fx_from<60>(H, bH + 1022);
+  q[5] = fx_from<61>(H, bH + 1022);
 #pragma unroll
   for (int c = 0; c < 6; ++c) own[c * n3p] = q[c];
   {
@@ -404,6 +409,7 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
     const int il = l == 0 ? node % n : (l == 1 ? (node / n) % n : node / n2), stride = l == 0 ? 1 : (l == 1 ? P : P * n);
     const fx64* jo = own + (6 + 3 * l) * n3p;
     const fx64 J0 = jo[0], J1 = jo[n3p], J2 = jo[2 * n3p];
+    const bool end = il == 0 || il == n - 1;
     FxAcc s[NV];
     int a = il;
 #pragma unroll 1
@@ -422,42 +428,48 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
       c.add(u, fx_split(j0 >> sc[0]));
       c.add(v, fx_split(j1 >> sc[1]));
       c.add(w, fx_split(j2 >> sc[2]));
-      const fx64 mi = fx_mul(fx_split(q[0] + f[0]), fx_split(c.get() << 2));  // 8 {rho}{u . Ja} in its units
-      const fx64 m4 = mi << 2;
+      // 8 {rho}{u . Ja}; the operands of D are shifted up, below 2^60.6 for the sums over a row
+      const fx64 m4 = fx_mul(fx_split(q[0] + f[0]), fx_split(c.get() << 2)) << 1;
+      const FxSplit ms = fx_split(m4);
+      if (shift_p) {  // a momentum flux beyond the pressure's
+        j0 >>= sp[0];
+        j1 >>= sp[1];
+        j2 >>= sp[2];
+      }
       const FxSplit p = fx_split(q[4] + f[4 * n3p]);
       const int2 D = sD[a * n + il];
       const FxSplit d{D.x, D.y};
-      s[0].add(fx_split(mi), d);
+      s[0].add(ms, d);
       FxAcc x;
       x.add(fx_split(m4 >> sm[0]), u);
-      x.add(p, fx_split(j0 >> sp[0]));
-      s[1].add(fx_split(x.get()), d);
+      x.add(p, fx_split(j0));
+      s[1].add(fx_split(x.get() << 1), d);
       x = FxAcc();
       x.add(fx_split(m4 >> sm[1]), v);
-      x.add(p, fx_split(j1 >> sp[1]));
-      s[2].add(fx_split(x.get()), d);
+      x.add(p, fx_split(j1));
+      s[2].add(fx_split(x.get() << 1), d);
       x = FxAcc();
       x.add(fx_split(m4 >> sm[2]), w);
-      x.add(p, fx_split(j2 >> sp[2]));
-      s[3].add(fx_split(x.get()), d);
-      s[4].add(fx_split(fx_mul(fx_split(m4), fx_split(q[5] + f[5 * n3p]))), d);
+      x.add(p, fx_split(j2));
+      s[3].add(fx_split(x.get() << 1), d);
+      s[4].add(fx_split(fx_mul(ms, fx_split(q[5] + f[5 * n3p])) << 2), d);
     }
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sum[v] += s[v].get();
+    for (int v = 0; v < NV; ++v) sum[v] += s[v].get() << (end ? 2 : 0);  // scale of the rows of D
   }
   if (valid) {
     const int t0 = bR + bC + 64 - fd.k;
     double* out = Utv + (size_t)e * NV * n3 + node;
-    out[0] = fx_to(sum[0], t0 - 56);
+    out[0] = fx_to(sum[0], t0 - 60);
 #pragma unroll
-    for (int v = 1; v < 4; ++v) out[(size_t)v * n3] = vis[v] + fx_to(sum[v], bM[v - 1] - 57 + 64 - fd.k);
-    out[(size_t)4 * n3] = vis[4] + fx_to(sum[4], t0 + bH - 55);
+    for (int v = 1; v < 4; ++v) out[(size_t)v * n3] = vis[v] + fx_to(sum[v], bM[v - 1] - 60 + 64 - fd.k);
+    out[(size_t)4 * n3] = vis[4] + fx_to(sum[4], t0 + bH - 60);
   }
   return true;
 }
 
 template <int n, bool LGL, bool KEP = false>
-__global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol_fx(
+__global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lift_vol_fx(
     const double* __restrict__ U, const double* __restrict__ Ja, const double* __restrict__ sJ,
     const double* __restrict__ Wf, const double* __restrict__ fgeo, const int* __restrict__ elemSide,
     double* __restrict__ Gf, double* __restrict__ Utv, double* __restrict__ Gvol, int K, int S, int bigBase,
@@ -509,6 +521,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
   for (int v = 0; v < NV; ++v) mW[v] = fx_mag(W[v]);
   // a2: face means of W and outward n_d s_hat (mortar big sides: their projected lifting flux
   // is read by the line tasks)
+  constexpr int half = 1 << 20;  // one exponent step of a magnitude word
   for (int it = tid; it < NE * 6 * n2; it += T) {
     const int el2 = it / (6 * n2);
     const int r = it - el2 * 6 * n2;
@@ -529,9 +542,9 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
         const double* w0 = Wf + ((size_t)side * NV) * n2 + mpq;
         const double* w1 = Wf + ((size_t)(S + side) * NV) * n2 + mpq;
         const double* g = fgeo + ((size_t)side * 4) * n2 + mpq;
-        const double sc = dg_neg_if(0.5 * g[3 * n2], es_slave(es));
+        const double sc = dg_neg_if(g[3 * n2], es_slave(es));
 #pragma unroll
-        for (int v = 0; v < NV; ++v) w[v] = w0[v * n2] + w1[v * n2];  // twice the mean: the half is in n_d s_hat
+        for (int v = 0; v < NV; ++v) w[v] = w0[v * n2] + w1[v * n2];  // twice the mean: halved by its exponent
 #pragma unroll
         for (int d = 0; d < 3; ++d) w[5 + d] = g[d * n2] * sc;
       }
@@ -540,12 +553,12 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
     for (int c = 0; c < 8; ++c) sW[((el2 * 6 + s) * 8 + c) * n2 + pq] = __double_as_longlong(w[c]);
     if constexpr (kWarp) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) mW[v] = max(mW[v], fx_mag(w[v]));
+      for (int v = 0; v < NV; ++v) mW[v] = max(mW[v], fx_mag(w[v]) - half);
 #pragma unroll
       for (int d = 0; d < 3; ++d) mJ[d] = max(mJ[d], fx_mag(w[5 + d]));
     } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) atomicMax(sMag + el2 * FX_SLOTS + FX_W + c, fx_mag(w[c]));
+      for (int c = 0; c < 8; ++c) atomicMax(sMag + el2 * FX_SLOTS + FX_W + c, fx_mag(w[c]) - (c < NV ? half : 0));
     }
   }
   fx_max<kWarp, 9>(mag, wmask, [&](int s) { return s < 5 ? mW[s < 5 ? s : 0] : (s < 8 ? mJ[s < 8 && s > 4 ? s - 5 : 0] : fx_mag(sj)); });
@@ -574,7 +587,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       fx64* x = sW + ((el2 * 6 + s) * 8 + c) * n2 + pq;
-      *x = fx_from<62>(__longlong_as_double(*x), sMag[el2 * FX_SLOTS + FX_W + c] >> 20);
+      *x = fx_from<62>(__longlong_as_double(*x), (sMag[el2 * FX_SLOTS + FX_W + c] >> 20) + (c < NV ? 1 : 0));
     }
   }
   const int ES = mag[FX_S] >> 20;
@@ -694,7 +707,7 @@ constexpr size_t lift_affine_smem_total() {
 }
 
 template <int n, bool LGL, bool KEP = false>
-__global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n>()) k_lift_vol_fx_affine(
+__global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lift_vol_fx_affine(
     const double* __restrict__ U, const double* __restrict__ aff, const double* __restrict__ Ja,
     const double* __restrict__ sJ, const double* __restrict__ Wf, const double* __restrict__ fgeo,
     const int* __restrict__ elemSide, double* __restrict__ Gf, double* __restrict__ Utv, double* __restrict__ Gvol, int K,
