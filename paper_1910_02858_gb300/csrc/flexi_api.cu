@@ -510,7 +510,7 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
   const std::vector<double> lmv = host::interp_matrix(xs, {-1.0}), lpv = host::interp_matrix(xs, {1.0});
   fill_ops<double>(c->ops64, Ds, ws, lmv, lpv, n);
   fill_ops<float>(c->ops32, Ds, ws, lmv, lpv, n);
-  c->m.fx = make_fx_ops(c->ops64, n);
+  c->m.fx = make_fx_ops(c->ops64, n, p->node_type == FLEXI_NODES_LOBATTO);
   for (int a = 0; a < (n + 1) / 2; ++a) {
     const int b = n - 1 - a;  // mirror node
     const bool mid = a == b;

@@ -29,6 +29,12 @@ constexpr int FXH = MAXN / 2;
 //   E_i = sum_a DE_ia e_a + t_i q_d,  O_i = sum_a DO_ia o_a + s_i q_s,
 // which halves the multiply-adds.  An entry c is stored as round(c 2^kc) = h 2^32 + l,
 // |l| <= 2^31, with kc the largest for which every row's sum of magnitudes stays below 2^62.
+// Gauss-Lobatto: the rows of the inner nodes are 5.3 to 9.8 times smaller than the first one, so
+// their scale is 2^(kc + fx_up), and fx_line<LGL> brings the ends' results to it.
+constexpr int fx_up(int n, bool lgl) {
+  return !lgl ? 0 : (n == 6 || n == 8 ? 3 : 2);  // the most for which the sums over three lines stay in range
+}
+
 struct FxOps {
   int eh[FXH][FXH], el[FXH][FXH];  // DE[i][a], i < n/2, a < (n+1)/2
   int oh[FXH][FXH], ol[FXH][FXH];  // DO[i][a], i < (n+1)/2, a < n/2
@@ -68,10 +74,10 @@ inline FxStrong make_fx_strong(const Ops<double>& o, int n) {
 
 // host construction from the FP64 operators (integer rounding of scaled doubles: the
 // same on every machine)
-inline FxOps make_fx_ops(const Ops<double>& o, int n) {
+inline FxOps make_fx_ops(const Ops<double>& o, int n, bool lgl) {
   FxOps f;
   std::memset(&f, 0, sizeof(f));
-  const int N = n - 1, h = n / 2, c = (n + 1) / 2;
+  const int N = n - 1, h = n / 2, c = (n + 1) / 2, up = fx_up(n, lgl);
   double row = 0, prow = 0, pe = 0, po = 0;
   for (int i = 0; i < n; ++i) {
     double e = 0.5 * std::fabs(o.lhp[i] - o.lhm[i]), d = 0.5 * std::fabs(o.lhp[i] + o.lhm[i]);
@@ -98,11 +104,12 @@ inline FxOps make_fx_ops(const Ops<double>& o, int n) {
   };
   // the operators' symmetric means: A = 2^(kc - 1) times twice the entry, halved below
   auto A = [&](int i, int a) {
-    return std::llrint(std::ldexp(o.DhatT[a * n + i], f.kc - 2)) -
-           std::llrint(std::ldexp(o.DhatT[(N - a) * n + N - i], f.kc - 2));
+    const int k = f.kc - 2 + (i > 0 && i < N ? up : 0);
+    return std::llrint(std::ldexp(o.DhatT[a * n + i], k)) - std::llrint(std::ldexp(o.DhatT[(N - a) * n + N - i], k));
   };
   auto Q = [&](int i) {
-    return std::llrint(std::ldexp(o.lhp[i], f.kc - 2)) + std::llrint(std::ldexp(o.lhm[N - i], f.kc - 2));
+    const int k = f.kc - 2 + (i > 0 && i < N ? up : 0);
+    return std::llrint(std::ldexp(o.lhp[i], k)) + std::llrint(std::ldexp(o.lhm[N - i], k));
   };
   auto L = [&](int a) {
     return std::llrint(std::ldexp(o.lp[a], f.kp - 2)) + std::llrint(std::ldexp(o.lm[N - a], f.kp - 2));
@@ -137,7 +144,7 @@ inline FxOps make_fx_ops_transposed(const Ops<double>& o, int n) {
     t.lhm[i] = o.lm[i];
     t.lhp[i] = o.lp[i];
   }
-  return make_fx_ops(t, n);
+  return make_fx_ops(t, n, false);
 }
 
 // ---------------------------------------------------------------------------
@@ -214,8 +221,8 @@ __device__ __forceinline__ fx64 fx_mul(FxSplit a, FxSplit b) {
 __device__ __forceinline__ fx64 fx_shr(fx64 v, int sh) { return (v + (1ll << (sh - 1))) >> sh; }
 
 // One line of a D_hat contraction in place: x[0], x[stride], ... (|x| < 2^59.6) become the
-// contraction (< 2^58.6); FACE: plus the face terms l_hat_i(-1) qm + l_hat_i(+1) qp
-// (Gauss-Lobatto: only at the line's ends)
+// contraction (< 2^58.6; LGL: 2^fx_up times that, see FxOps); FACE: plus the face terms
+// l_hat_i(-1) qm + l_hat_i(+1) qp (Gauss-Lobatto: only at the line's ends)
 template <int n, bool LGL, bool FACE>
 __device__ __forceinline__ void fx_line(fx64* __restrict__ p, int stride, fx64 qm, fx64 qp, const FxOps& o) {
   constexpr int h = n / 2, c = (n + 1) / 2, N = n - 1;
@@ -239,13 +246,13 @@ __device__ __forceinline__ void fx_line(fx64* __restrict__ p, int stride, fx64 q
 #pragma unroll
     for (int a = 0; a < h; ++a) so.add(d[a], o.oh[i][a], o.ol[i][a]);
     if (face) so.add(qs, o.sh[i], o.sl[i]);
-    const fx64 O = so.get();
+    const fx64 O = so.get() << (i == 0 ? fx_up(n, LGL) : 0);
     if (i < h) {
       FxAcc se;
 #pragma unroll
       for (int a = 0; a < c; ++a) se.add(e[a], o.eh[i][a], o.el[i][a]);
       if (face) se.add(qd, o.th[i], o.tl[i]);
-      const fx64 E = se.get();
+      const fx64 E = se.get() << (i == 0 ? fx_up(n, LGL) : 0);
       p[i * stride] = O + E;
       p[(N - i) * stride] = O - E;
     } else {

@@ -283,7 +283,7 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
     for (int v = 0; v < NV; ++v) {
       const fx64* r = own + v * n3p;
       Utv[((size_t)e * NV + v) * n3 + node] =
-          fx_to(r[0] + r[NV * n3p] + r[2 * NV * n3p], mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx.kc);
+          fx_to(r[0] + r[NV * n3p] + r[2 * NV * n3p], mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx_up(n, LGL) - fx.kc);
     }
   }
   return true;
@@ -367,7 +367,7 @@ __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, do
 #pragma unroll
   for (int v = 1; v < NV; ++v)
     vis[v] = fx_to(own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p],
-                   mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx.kc);
+                   mag[FX_F + v] + (mag[JS] >> 20) - 2044 + 6 - fx_up(n, true) - fx.kc);
   // advective part: bounds b of rho, H, p, mass flux and momentum flux as powers of two
   const int bR = (mag[FX_W] >> 20) - 1022, bH = (mag[FX_F] >> 20) - 1022, bP = (mag[FX_W + 4] >> 20) - 1022;
   int bC = -4096;
@@ -478,6 +478,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lif
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   constexpr bool kWarp = NE == 1;
+  constexpr int kUp = LGL ? fx_up(n, true) - 2 : 0;
   const int grp = order != nullptr ? order[blockIdx.x] : blockIdx.x;  // NE consecutive elements
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx64* sA = reinterpret_cast<fx64*>(smem_raw);  // [NE][15][n3p] line fields l*5 + v, contracted in place
@@ -638,8 +639,8 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lif
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         fx64* r = sA + (el * 15 + v) * n3p + pn;
-        const fx64 g = fx_mul(fx_split((r[0] + r[NV * n3p] + r[2 * NV * n3p]) << 2), si);
-        G[d * NV + v] = fx_to(g, sExp[el * 32 + v * 3 + d] + 5 - fx.kc + ES - 1022);
+        const fx64 g = fx_mul(fx_split((r[0] + r[NV * n3p] + r[2 * NV * n3p]) << (LGL ? 0 : 2)), si);  // scale 2^(kc + 2 + kUp)
+        G[d * NV + v] = fx_to(g, sExp[el * 32 + v * 3 + d] + 5 - kUp - fx.kc + ES - 1022);
         r[0] = LGL ? __double_as_longlong(G[d * NV + v]) : g;
         if (Gvol != nullptr && valid) Gvol[((size_t)e * 15 + d * NV + v) * n3 + node] = G[d * NV + v];
       }
@@ -716,6 +717,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lif
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   constexpr bool kWarp = NE == 1;
+  constexpr int kUp = LGL ? fx_up(n, true) - 2 : 0;
   const int grp = order != nullptr ? order[blockIdx.x] : blockIdx.x;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fx64* sA = reinterpret_cast<fx64*>(smem_raw);  // [NE][15][n3p] line fields l*5 + v, contracted in place
@@ -844,14 +846,14 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lif
     for (int v = 0; v < NV; ++v) {
       FxSplit t[3];
 #pragma unroll
-      for (int l = 0; l < 3; ++l) t[l] = fx_split(own[(l * NV + v) * n3p] << 2);
+      for (int l = 0; l < 3; ++l) t[l] = fx_split(own[(l * NV + v) * n3p] << (LGL ? 0 : 2));  // scale 2^(kc + 2 + kUp)
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         FxAcc s;
 #pragma unroll
         for (int l = 0; l < 3; ++l) s.add(m[l * 3 + d], t[l]);
         const fx64 g = s.get();
-        G[d * NV + v] = fx_to(g, (mag[FX_J + d] >> 20) + (mag[FX_W + v] >> 20) - 2044 + 5 - fx.kc);
+        G[d * NV + v] = fx_to(g, (mag[FX_J + d] >> 20) + (mag[FX_W + v] >> 20) - 2044 + 5 - kUp - fx.kc);
         own[(d * NV + v) * n3p] = LGL ? __double_as_longlong(G[d * NV + v]) : g;
         if (Gvol != nullptr && valid) Gvol[((size_t)e * 15 + d * NV + v) * n3 + node] = G[d * NV + v];
       }

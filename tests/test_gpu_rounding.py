@@ -47,3 +47,10 @@ def _noise(N, mapping, split):
 def test_split_form(N, mapping):
     fixed, fp64 = _noise(N, mapping, 1)
     assert (fixed <= 1.25 * fp64).all(), fixed / fp64
+
+
+@pytest.mark.parametrize("mapping", ["cartesian", "sine"])
+@pytest.mark.parametrize("N", [3, 4, 5, 6, 7])
+def test_standard_form(N, mapping):
+    fixed, fp64 = _noise(N, mapping, 0)
+    assert (fixed <= 1.25 * fp64).all(), fixed / fp64
