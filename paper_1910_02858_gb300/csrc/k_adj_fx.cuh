@@ -11,9 +11,10 @@
 
 namespace flexi {
 
-// slots: lam/J by variable, metric terms (nodes and faces), lam_lift by variable, face gradient
-// adjoints by component
-enum { FXA_L = 0, FXA_J = 5, FXA_X = 6, FXA_B = 16, FXA_SLOTS = 32 };
+// slots: lam/J by variable, metric terms by physical direction (nodes and faces), lam_lift and
+// face gradient adjoints at d*5+v.  As in volume_fx, a variable's three lam_lift components are
+// scaled by direction so that their products with Ja_d meet at the largest of them.
+enum { FXA_L = 0, FXA_J = 5, FXA_X = 8, FXA_B = 23, FXA_SLOTS = 38 };
 
 // the FP64 kernel as a function, for elements outside the fixed-point range
 template <int n>
@@ -77,14 +78,14 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
   // lam_vol = -lam / J, the metric terms' and the face data's magnitudes
   {
     double lv[NV];
-    int mJ = 0;
+    int mJ[3] = {0, 0, 0};
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       lv[v] = valid ? -lam[((size_t)e * NV + v) * n3 + node] * sj : 0.0;
       own[v * n3p] = __double_as_longlong(lv[v]);
     }
 #pragma unroll
-    for (int c = 0; c < 9; ++c) mJ = max(mJ, fx_mag(metric(c)));
+    for (int c = 0; c < 9; ++c) mJ[c % 3] = max(mJ[c % 3], fx_mag(metric(c)));
     for (int it = tid; it < NE * 6 * n2; it += T) {
       const int f = it / n2, pq = it - f * n2;
       if (e0 + f / 6 >= K) continue;
@@ -106,12 +107,12 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
         for (int d = 0; d < 3; ++d) {
           const double x = side < bigBase ? g[d * n2] * sc : 0.0;
           sN[(f * 3 + d) * n2 + pq] = __double_as_longlong(x);
-          mJ = kWarp ? max(mJ, fx_mag(x)) : mJ;
-          if constexpr (!kWarp) atomicMax(m + FXA_J, fx_mag(x));
+          mJ[d] = kWarp ? max(mJ[d], fx_mag(x)) : mJ[d];
+          if constexpr (!kWarp) atomicMax(m + FXA_J + d, fx_mag(x));
         }
       }
     }
-    fx_max<kWarp, 6>(mag, wmask, [&](int s) { return s < 5 ? fx_mag(lv[s < 5 ? s : 0]) : mJ; });
+    fx_max<kWarp, 8>(mag, wmask, [&](int s) { return s < 5 ? fx_mag(lv[s < 5 ? s : 0]) : mJ[s < 5 ? 0 : s - 5]; });
   }
   __syncthreads();
   {
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
       return;
     }
   }
-  const int EJ = mag[FXA_J] >> 20;
+  const int* EJ = mag + FXA_J;  // exponent of direction d: EJ[d] >> 20
   for (int it = tid; it < NE * 6 * n2; it += T) {  // the thread's own entries, as above
     const int f = it / n2, pq = it - f * n2;
     if (e0 + f / 6 >= K) continue;
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         fx64* x = sN + (f * 3 + d) * n2 + pq;
-        *x = fx_from<62>(__longlong_as_double(*x), m[FXA_J] >> 20);
+        *x = fx_from<62>(__longlong_as_double(*x), m[FXA_J + d] >> 20);
       }
     }
   }
@@ -158,7 +159,6 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
   __syncthreads();
   // reverse of a6: lam_d = sum_l Ja^l_d lamF^l, then the pointwise fluxes
   double lamU[NV] = {0, 0, 0, 0, 0}, lamW[NV] = {0, 0, 0, 0, 0}, W[NV];
-  int mx[NV] = {0, 0, 0, 0, 0};
   {
     double Uo[NV] = {1.0, 0.0, 0.0, 0.0, 1.0}, lvisc[3][NV];
     if (valid) {
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
     {
       FxSplit ji[9];
 #pragma unroll
-      for (int c = 0; c < 9; ++c) ji[c] = fx_split(fx_from<62>(metric(c), EJ));
+      for (int c = 0; c < 9; ++c) ji[c] = fx_split(fx_from<62>(metric(c), EJ[c % 3] >> 20));
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         FxSplit t[3];
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
           FxAcc s;
 #pragma unroll
           for (int l = 0; l < 3; ++l) s.add(ji[l * 3 + d], t[l]);
-          lvisc[d][v] = -fx_to(s.get(), EJ + (mag[FXA_L + v] >> 20) - 2044 + 5 - fx.kc);
+          lvisc[d][v] = -fx_to(s.get(), (EJ[d] >> 20) + (mag[FXA_L + v] >> 20) - 2044 + 5 - fx.kc);
         }
       }
     }
@@ -208,18 +208,34 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
       return a.get();
     };
 #pragma unroll
-    for (int c = 0; c < 15; ++c) {
-      const fx64 b = spread(0, pq0, i, c) + spread(1, pq1, j, c) + spread(2, pq2, k, c);
-      const double x = (lamG[c] + fx_to(b, (mag[FXA_B + c] >> 20) - 1022 + 3 - fx.kl)) * sj;
-      mx[c % NV] = max(mx[c % NV], fx_mag(x));
-      own[c * n3p] = __double_as_longlong(x);  // the thread's entries: field d*5 + v
+    for (int d = 0; d < 3; ++d) {
+      int mx[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const int c = d * NV + v;
+        const fx64 b = spread(0, pq0, i, c) + spread(1, pq1, j, c) + spread(2, pq2, k, c);
+        const double x = (lamG[c] + fx_to(b, (mag[FXA_B + c] >> 20) - 1022 + 3 - fx.kl)) * sj;
+        mx[v] = fx_mag(x);
+        own[c * n3p] = __double_as_longlong(x);  // the thread's entries: field d*5 + v
+      }
+      fx_max<kWarp, NV>(mag + FXA_X + d * NV, wmask, [&](int s) { return mx[s]; });
     }
   }
-  fx_max<kWarp, NV>(mag + FXA_X, wmask, [&](int s) { return mx[s]; });
   __syncthreads();
-  {
+  {  // magnitude words -> the exponents under which lam_lift_d,v is converted (flux_exponents, k_lift_fx.cuh)
     int bad = 0;
-    for (int t = tid; t < NE * NV; t += T) bad |= (sMag[(t / NV) * FXA_SLOTS + FXA_X + t % NV] >> 20) > 1022 + 600;
+    for (int t = tid; t < NE * NV; t += T) {
+      int* m = sMag + (t / NV) * FXA_SLOTS;
+      int* f = m + FXA_X + t % NV;
+      int x = 0;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        bad |= (f[d * NV] >> 20) > 1022 + 600;
+        x = max(x, (f[d * NV] >> 20) + (m[FXA_J + d] >> 20));
+      }
+#pragma unroll
+      for (int d = 0; d < 3; ++d) f[d * NV] = x - (m[FXA_J + d] >> 20);
+    }
     if (__syncthreads_or(bad)) {
       fp64();
       return;
@@ -231,12 +247,12 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
     {
       FxSplit ji[9];
 #pragma unroll
-      for (int c = 0; c < 9; ++c) ji[c] = fx_split(fx_from<62>(metric(c), EJ));
+      for (int c = 0; c < 9; ++c) ji[c] = fx_split(fx_from<62>(metric(c), EJ[c % 3] >> 20));
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         FxSplit x[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) x[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FXA_X + v] >> 20));
+        for (int d = 0; d < 3; ++d) x[d] = fx_split(fx_from<60>(__longlong_as_double(own[(d * NV + v) * n3p]), mag[FXA_X + d * NV + v]));
 #pragma unroll
         for (int l = 0; l < 3; ++l) {
           FxAcc s;
@@ -263,12 +279,12 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
 #pragma unroll
     for (int v = 0; v < NV; ++v)
       lamW[v] += fx_to(own[v * n3p] + own[(NV + v) * n3p] + own[(2 * NV + v) * n3p],
-                       EJ + (mag[FXA_X + v] >> 20) - 2044 + 6 - fx.kc);
+                       (EJ[0] >> 20) + mag[FXA_X + v] - 2044 + 6 - fx.kc);
   } else {
     fx64 acc[NV] = {0, 0, 0, 0, 0};
     fx64 x[15];
 #pragma unroll
-    for (int c = 0; c < 15; ++c) x[c] = fx_from<59>(__longlong_as_double(own[c * n3p]), mag[FXA_X + c % NV] >> 20);
+    for (int c = 0; c < 15; ++c) x[c] = fx_from<59>(__longlong_as_double(own[c * n3p]), mag[FXA_X + c]);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
 #pragma unroll
@@ -293,13 +309,13 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
           const int side = es_side(sES[fc]);
           if (side >= bigBase && e0 + el2 < K)  // adjoint of the projected lifting flux QB
             LQB[((size_t)(side - bigBase) * 15 + v * 3 + d) * n2 + sMpq[fc * n2 + line]] =
-                fx_to(y[m], (sMag[el2 * FXA_SLOTS + FXA_X + v] >> 20) - 1022 + 5 - fx.kp);
+                fx_to(y[m], sMag[el2 * FXA_SLOTS + FXA_X + d * NV + v] - 1022 + 5 - fx.kp);
         }
       }
       __syncthreads();
       FxSplit a[3];
 #pragma unroll
-      for (int l = 0; l < 3; ++l) a[l] = fx_split(fx_from<62>(metric(l * 3 + d), EJ));
+      for (int l = 0; l < 3; ++l) a[l] = fx_split(fx_from<62>(metric(l * 3 + d), EJ[d] >> 20));
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         FxAcc s;
@@ -310,7 +326,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
       // a thread stages only its own entries, read by line tasks before the barrier above
     }
 #pragma unroll
-    for (int v = 0; v < NV; ++v) lamW[v] += fx_to(acc[v], EJ + (mag[FXA_X + v] >> 20) - 2044 + 5 - fx.kc);
+    for (int v = 0; v < NV; ++v) lamW[v] += fx_to(acc[v], (EJ[0] >> 20) + mag[FXA_X + v] - 2044 + 5 - fx.kc);
   }
   // adjoints of the face means of W to the side arrays
   for (int it = tid; it < NE * 6 * n2; it += T) {
@@ -321,7 +337,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 
     double* dst = LWs + ((size_t)(es_slave(es) * S + side) * NV) * n2 + sMpq[it];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      const int t = (m[FXA_J] >> 20) + (m[FXA_X + v] >> 20) - 2044 + (AFF ? 6 : 5) - fx.kp;
+      const int t = (m[FXA_J] >> 20) + m[FXA_X + v] - 2044 + (AFF ? 6 : 5) - fx.kp;
       dst[v * n2] = side >= bigBase ? 0.0 : fx_to(sS[(f * NV + v) * n2 + pq], t);
     }
   }

@@ -85,3 +85,27 @@ def test_thin_elements(N, nodes, split, mapping):
     tol = 4 * 2 * 3 * (N + 3) * 2.0 ** -53 * T * (4 if split else 1)  # pairs: as in test_gpu_fixed_point.py
     for v in range(5):
         assert np.abs(a[:, v] - c[:, v]).max() <= tol[v], v
+
+
+@pytest.mark.parametrize("mapping", ["box", "columns"])
+@pytest.mark.parametrize("N", [4, 5, 6, 7])
+def test_adjoint_of_thin_elements(N, mapping):
+    """The reverse kernel: adjoints of the y momentum, constant in z (Gauss-Lobatto: no jumps there).  The x and y
+    momentum receive from direction d at most g_d |dF_d,v / d(rho u, rho v)| |lam|, with F_z,v = rho w v.  The FP64
+    body is reached by lam 2^220, in which every operation is linear."""
+    import torch
+
+    mesh = _mesh(mapping, N)
+    W = _state(mesh, N, 1)
+    _, g = _bound(W, N, 1)
+    x = mesh.node_coords(N, 1)
+    lam = np.zeros_like(W)
+    lam[:, 2] = np.sin(x[:, 0] + 0.3) * np.cos(2 * x[:, 1])
+    U = torch.tensor(wl.prim_to_cons_np(*np.moveaxis(W, 1, 0), 1.4), device="cuda:0")
+    s = _solver(mesh, N, 1, adjoint=True)
+    a, c = (s.rhs_adjoint(U, torch.tensor(lam * f, device="cuda:0"), 0.0).cpu().numpy() / f for f in (1.0, 2.0 ** 220))
+    s.close()
+    u, v, w = (np.abs(W[:, d]).max() for d in (1, 2, 3))
+    T = {1: g[0] * v + g[1] * 0.4 * u, 2: g[0] * u + g[1] * 1.6 * v + g[2] * w}
+    for k in T:
+        assert np.abs(a[:, k] - c[:, k]).max() <= 4 * 2 * 3 * (N + 3) * 2.0 ** -53 * T[k], k
