@@ -282,51 +282,61 @@ __device__ __forceinline__ void fx_ends(const fx64* __restrict__ p, int stride, 
   ym = E - D;
 }
 
-// Normal of a face in fixed point for fx_visc_normal: n_d (62 bits under 2) and -2/3 n_d
+// Normal of a face in fixed point for fx_visc_normal: n_d and -2/3 n_d (60 bits) under the
+// exponent e_d of n_d
 struct FxNormal {
   FxSplit n[3], m[3];
+  int e[3];
 };
 __device__ __forceinline__ FxNormal fx_normal(const double n[3]) {
   FxNormal q;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    q.n[d] = fx_split(fx_from<62>(n[d], 1023));
-    q.m[d] = fx_split(fx_from<62>(-(2.0 / 3.0) * n[d], 1023));
+    q.e[d] = fx_mag(n[d]) >> 20;
+    q.n[d] = fx_split(fx_from<60>(n[d], q.e[d]));
+    q.m[d] = fx_split(fx_from<60>(-(2.0 / 3.0) * n[d], q.e[d]));
   }
   return q;
 }
 
 // visc_normal with the stress sums tn_c = sum_d (G_dc + G_cd) n_d - 2/3 div n_c in fixed point
-// (26 of its 45 FP64 instructions; HLLC k_face at 16^3, N = 7: 275 -> 226 us); gradients outside
-// the range take the FP64 sums
+// (26 of its 45 FP64 instructions; HLLC k_face at 16^3, N = 7: 275 -> 226 us).  The diagonal, each
+// pair of off-diagonal gradients and each component of n have their own exponent and the products
+// of a sum meet at its largest: a shear layer's gradient, large against all others, leaves the sums
+// that it does not enter as accurate as in FP64.  Gradients outside the range take the FP64 sums.
 __device__ __forceinline__ void fx_visc_normal(const double W[NV], const double ir, const double G[15], const double n[3],
                                                const FxNormal& q, const Phys<double>& ph, double f[NV]) {
-  int big = 0;
+  int ed = 0, eo[3];  // diagonal; off-diagonal pair k: the two directions other than k
 #pragma unroll
-  for (int d = 0; d < 3; ++d)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) big = max(big, fx_mag(G[d * 5 + 1 + c]));
-  const int E = big >> 20;
-  if (E > 1900) {
+  for (int k = 0; k < 3; ++k) {
+    const int i = (k + 1) % 3, j = (k + 2) % 3;
+    ed = max(ed, fx_mag(G[k * 5 + 1 + k]) >> 20);
+    eo[k] = max(fx_mag(G[i * 5 + 1 + j]), fx_mag(G[j * 5 + 1 + i])) >> 20;
+  }
+  if (max(max(ed, eo[0]), max(eo[1], eo[2])) > 1900) {
     visc_normal(W, ir, G, n, ph, f);
     return;
   }
-  fx64 g[3][3];
+  fx64 g[3], a[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) g[d][c] = fx_from<60>(G[d * 5 + 1 + c], E);
-  const FxSplit div = fx_split(g[0][0] + g[1][1] + g[2][2]);
-  const FxSplit a[3] = {fx_split(g[1][2] + g[2][1]), fx_split(g[0][2] + g[2][0]), fx_split(g[0][1] + g[1][0])};
+  for (int k = 0; k < 3; ++k) {
+    const int i = (k + 1) % 3, j = (k + 2) % 3;
+    g[k] = fx_from<60>(G[k * 5 + 1 + k], ed);
+    a[k] = fx_from<60>(G[i * 5 + 1 + j], eo[k]) + fx_from<60>(G[j * 5 + 1 + i], eo[k]);
+  }
+  const fx64 div = g[0] + g[1] + g[2];
   double tn[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
+    const int i = (c + 1) % 3, j = (c + 2) % 3;  // a[i] meets n_j, a[j] meets n_i
+    const int xd = ed + q.e[c], xi = eo[i] + q.e[j], xj = eo[j] + q.e[i], x = max(xd, max(xi, xj));
+    const int sd = min(x - xd, 62);
     FxAcc s;
-    s.add(fx_split(2 * g[c][c]), q.n[c]);
-    s.add(a[(c + 1) % 3], q.n[(c + 2) % 3]);  // a[k]: the pair of directions other than k
-    s.add(a[(c + 2) % 3], q.n[(c + 1) % 3]);
-    s.add(div, q.m[c]);
-    tn[c] = ph.mu * fx_to(s.get(), E - 1022 + 64 - 60 - 61);
+    s.add(fx_split((2 * g[c]) >> sd), q.n[c]);
+    s.add(fx_split(div >> sd), q.m[c]);
+    s.add(fx_split(a[i] >> min(x - xi, 62)), q.n[j]);
+    s.add(fx_split(a[j] >> min(x - xj, 62)), q.n[i]);
+    tn[c] = ph.mu * fx_to(s.get(), x - 2044 + 64 - 120);
   }
   const double pir = W[4] * ir;
   double dTn = 0.0;
