@@ -338,11 +338,12 @@ void fill_mortar_ops(MortarOps<real>& o, const std::vector<double>& x, const std
 }
 
 // Metric terms Ja^l_d (l*3+d) and 1/J of an element whose mapping is affine to within the
-// rounding of its coordinates: x [ng^3][3] at the tensor product of the points xg
+// rounding of its coordinates, each of which has its own (a far offset or a long edge in one
+// direction says nothing about the others): x [ng^3][3] at the tensor product of the points xg
 bool affine_metrics(const double* x, const std::vector<double>& xg, int ng, double* out) {
   const int last = ng - 1;
   auto at = [&](int i, int j, int k, int d) { return x[((k * ng + j) * ng + i) * 3 + d]; };
-  double a[3][3], size = 0.0;  // a[l] = dx / dxi_l: mean of the four parallel edges over 2
+  double a[3][3], tol[3];  // a[l] = dx / dxi_l: mean of the four parallel edges over 2
   for (int d = 0; d < 3; ++d) {
     for (int l = 0; l < 3; ++l) a[l][d] = 0.0;
     for (int p = 0; p < 2; ++p)
@@ -355,15 +356,14 @@ bool affine_metrics(const double* x, const std::vector<double>& xg, int ng, doub
   for (int d = 0; d < 3; ++d) {
     double s = std::fabs(at(0, 0, 0, d));
     for (int l = 0; l < 3; ++l) s += 2.0 * std::fabs(a[l][d]);
-    size = std::max(size, s);
+    tol[d] = 16.0 * 2.220446049250313e-16 * s;  // a few units of the coordinate's rounding
   }
-  const double tol = 16.0 * 2.220446049250313e-16 * size;  // a few units of the coordinates' rounding
   for (int k = 0; k < ng; ++k)
     for (int j = 0; j < ng; ++j)
       for (int i = 0; i < ng; ++i)
         for (int d = 0; d < 3; ++d) {
           const double y = at(0, 0, 0, d) + (xg[i] + 1.0) * a[0][d] + (xg[j] + 1.0) * a[1][d] + (xg[k] + 1.0) * a[2][d];
-          if (!(std::fabs(at(i, j, k, d) - y) <= tol)) return false;
+          if (!(std::fabs(at(i, j, k, d) - y) <= tol[d])) return false;
         }
   for (int l = 0; l < 3; ++l) {
     const double *u = a[(l + 1) % 3], *v = a[(l + 2) % 3];
