@@ -686,6 +686,11 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
         }
         if (pass == 0) c->m.nAffine = (int)order.size();
       }
+      // A mixed mesh takes two launches, one after the other, of which the affine one saves a quarter
+      // to a half of its time and the other ends in a wave of its own: worth it from about four
+      // waves of affine CTAs (1024 threads per SM) on.  10^3 elements, N = 1, FP32, some of them
+      // affine: 23 us in two launches, 14 us in one.
+      if (c->m.nAffine < groups && (int64_t)c->m.nAffine * ne * n3 < (int64_t)4 * 1024 * nsm) c->m.nAffine = 0;
       if (c->m.nAffine > 0 && c->m.nAffine < groups) {
         int* dorder;
         AL(dorder, order.size());
