@@ -399,12 +399,13 @@ constexpr int lift_vol_min_blocks() {
 // SPLIT (Gauss-Lobatto, SW = 0 only): the split-form volume integral of Sec. 3.3 with the
 // kinetic-energy-preserving two-point flux (1) or the entropy-conservative one (2)
 // (Eq. semiDiscreteSplit).
-template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2>
+// ORD: the CTAs take their element groups from order (the rest of a mesh with affine elements)
+template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2, bool ORD>
 __device__ __forceinline__ void lift_vol_body(
     const real* __restrict__ U, const real* __restrict__ Ja, const real* __restrict__ sJ,
     const real* __restrict__ Wf, const real* __restrict__ fgeo, const int* __restrict__ elemSide,
     real* __restrict__ Gf, real* __restrict__ Utv, real* __restrict__ Gvol, int K, int S, int bigBase,
-    const real* __restrict__ QB, const int* __restrict__ order, const Ops<real>& ops, const Phys<real>& ph) {
+    const real* __restrict__ QB, const Ops<real>& ops, const Phys<real>& ph, const int* __restrict__ order) {
   using C = Cfg<n>;
   constexpr int n2 = C::n2, n3 = C::n3, NE = C::NE, T = C::T, n3p = C::n3p;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -427,7 +428,7 @@ __device__ __forceinline__ void lift_vol_body(
 
   const int tid = threadIdx.x;
   const int el = tid / n3, node = tid - el * n3;
-  const int e0 = (order != nullptr ? order[blockIdx.x] : blockIdx.x) * NE;
+  const int e0 = (ORD ? order[blockIdx.x] : blockIdx.x) * NE;
   const int e = e0 + el;
   const bool valid = e < K;
   const int i = node % n, j = (node / n) % n, k = node / n2;
@@ -910,19 +911,19 @@ __device__ __forceinline__ void lift_vol_body(
   const real *__restrict__ U, const real *__restrict__ Ja, const real *__restrict__ sJ,                   \
       const real *__restrict__ Wf, const real *__restrict__ fgeo, const int *__restrict__ elemSide,        \
       real *__restrict__ Gf, real *__restrict__ Utv, real *__restrict__ Gvol, int K, int S, int bigBase, \
-      const real *__restrict__ QB, const int *__restrict__ order, Ops<real> ops, Phys<real> ph
-#define FLEXI_LIFT_VOL_ARGS U, Ja, sJ, Wf, fgeo, elemSide, Gf, Utv, Gvol, K, S, bigBase, QB, order, ops, ph
+      const real *__restrict__ QB, Ops<real> ops, Phys<real> ph, const int *__restrict__ order
+#define FLEXI_LIFT_VOL_ARGS U, Ja, sJ, Wf, fgeo, elemSide, Gf, Utv, Gvol, K, S, bigBase, QB, ops, ph, order
 
 // the kernel at the compiler's default register allocation
-template <typename real, int n, int SW, bool LGL, int SPLIT = 0, bool BR2 = false>
+template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2, bool ORD>
 __global__ void __launch_bounds__(Cfg<n>::T) k_lift_vol(FLEXI_LIFT_VOL_PARAMS) {
-  lift_vol_body<real, n, SW, LGL, SPLIT, BR2>(FLEXI_LIFT_VOL_ARGS);
+  lift_vol_body<real, n, SW, LGL, SPLIT, BR2, ORD>(FLEXI_LIFT_VOL_ARGS);
 }
 
 // the same kernel with lift_vol_min_blocks() CTAs per SM (register cap)
-template <typename real, int n, int SW, bool LGL, int SPLIT = 0, bool BR2 = false>
+template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2, bool ORD>
 __global__ void __launch_bounds__(Cfg<n>::T, lift_vol_min_blocks<real, n, SW, SPLIT, BR2>()) k_lift_vol_mb(FLEXI_LIFT_VOL_PARAMS) {
-  lift_vol_body<real, n, SW, LGL, SPLIT, BR2>(FLEXI_LIFT_VOL_ARGS);
+  lift_vol_body<real, n, SW, LGL, SPLIT, BR2, ORD>(FLEXI_LIFT_VOL_ARGS);
 }
 #undef FLEXI_LIFT_VOL_PARAMS
 #undef FLEXI_LIFT_VOL_ARGS
@@ -1381,12 +1382,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(15 * n * n * n / 2) 
   cluster_wait();  // the other CTA has finished reading this one's shared memory
 }
 
-template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2>
+template <typename real, int n, int SW, bool LGL, int SPLIT, bool BR2, bool ORD>
 constexpr auto lift_vol_kernel() {
   if constexpr (lift_vol_min_blocks<real, n, SW, SPLIT, BR2>() > 0)
-    return &k_lift_vol_mb<real, n, SW, LGL, SPLIT, BR2>;
+    return &k_lift_vol_mb<real, n, SW, LGL, SPLIT, BR2, ORD>;
   else
-    return &k_lift_vol<real, n, SW, LGL, SPLIT, BR2>;
+    return &k_lift_vol<real, n, SW, LGL, SPLIT, BR2, ORD>;
 }
 
 template <typename real, int n, int SW, int SPLIT = 0, bool BR2 = false>
@@ -1993,13 +1994,16 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
                               int store_grad, cudaStream_t st) {
   using C = Cfg<n>;
   constexpr size_t smem = lift_vol_smem<real, n, SW, SPLIT, BR2>();
-  auto* kernel = lift_vol_kernel<real, n, SW, LGL, SPLIT, BR2>();
-  static std::atomic<unsigned long long> attr{0};
-  cudaError_t err = ensure_dynamic_smem(kernel, smem, attr);
-  if (err != cudaSuccess) return err;
   const int groups = (m.K + C::NE - 1) / C::NE;
-  const int* order = nullptr;
-  int grid = groups;
+  cudaError_t err;
+  // the element groups order[0], ... (ORD) or all of them
+  auto general = [&](auto* kernel, std::atomic<unsigned long long>& attr, int grid, const int* order) {
+    if ((err = ensure_dynamic_smem(kernel, smem, attr)) != cudaSuccess) return err;
+    kernel<<<grid, C::T, smem, st>>>(U, (const real*)m.Ja, (const real*)m.sJ, (const real*)m.Wf, (const real*)m.fgeo,
+                                     m.elemSide, (real*)m.Gf, (real*)m.Utv, store_grad ? (real*)m.Gvol : nullptr, m.K, m.S,
+                                     m.Sface, (const real*)m.QB, ops, ph, order);
+    return cudaGetLastError();
+  };
   if constexpr (sizeof(real) == 4 && SPLIT == 0 && !BR2) {  // affine elements by their own kernel
     if (m.nAffine > 0) {
       constexpr size_t smemA = lift_f32_affine_smem<n, SW>();
@@ -2009,17 +2013,15 @@ static cudaError_t lift_vol_n(const DevMesh& m, const real* U, const Ops<real>& 
           U, (const float*)m.affine, (const float*)m.Wf, m.elemSide, (float*)m.Gf, (float*)m.Utv,
           store_grad ? (float*)m.Gvol : nullptr, m.K, m.S, m.nAffine < groups ? m.order : nullptr, ops, m.eo, ph);
       if ((err = cudaGetLastError()) != cudaSuccess || m.nAffine == groups) return err;
-      order = m.order + m.nAffine;
-      grid = groups - m.nAffine;
+      // an instance of its own: with the order read, or its argument tested, in the instance of meshes
+      // without affine elements the CTA's addresses leave the uniform registers (TF32, N = 4, 16^3
+      // curved elements: 111 -> 117 us)
+      static std::atomic<unsigned long long> attrO{0};
+      return general(lift_vol_kernel<real, n, SW, LGL, SPLIT, BR2, true>(), attrO, groups - m.nAffine, m.order + m.nAffine);
     }
   }
-  kernel<<<grid, C::T, smem, st>>>(U, (const real*)m.Ja, (const real*)m.sJ,
-                                                         (const real*)m.Wf, (const real*)m.fgeo, m.elemSide,
-                                                         (real*)m.Gf, (real*)m.Utv,
-                                                         store_grad ? (real*)m.Gvol : nullptr, m.K, m.S,
-                                                         m.Sface, (const real*)m.QB, order,
-                                                         ops, ph);
-  return cudaGetLastError();
+  static std::atomic<unsigned long long> attr{0};
+  return general(lift_vol_kernel<real, n, SW, LGL, SPLIT, BR2, false>(), attr, groups, nullptr);
 }
 
 // fixed-point lifting + volume kernel (FP64, BR1; standard or kinetic-energy-preserving split
