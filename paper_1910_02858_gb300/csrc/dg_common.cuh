@@ -421,12 +421,20 @@ __device__ __forceinline__ double dg_log<double>(double x) { return log(x); }
 template <>
 __device__ __forceinline__ float dg_log<float>(float x) { return logf(x); }
 
+// INT: quotients by dg_div, else by the language's division
+template <bool INT, typename real>
+__device__ __forceinline__ real quotient(real a, real b) {
+  if constexpr (INT)
+    return dg_div(a, b);
+  else
+    return a / b;
+}
 // logarithmic mean (a - b)/(ln a - ln b) of positive a, b (Ismail & Roe form):
 // f = (a - b)/(a + b), u = f^2; mean = (a + b)/(2 F) with
 // F = atanh(f)/f = ln(a/b)/(2 f), or its series sum_k u^k/(2k + 1) to u^7 for u < 1e-2
-template <typename real>
+template <bool INT = true, typename real>
 __device__ __forceinline__ real log_mean(real a, real b) {
-  const real f = dg_div(a - b, a + b);
+  const real f = quotient<INT>(a - b, a + b);
   const real u = f * f;
   real F;
   if (u < real(1e-2)) {
@@ -439,26 +447,26 @@ __device__ __forceinline__ real log_mean(real a, real b) {
     F = F * u + real(1.0 / 3.0);
     F = F * u + real(1);
   } else {
-    F = dg_div(dg_log(dg_div(a, b)), real(2) * f);
+    F = quotient<INT>(dg_log(quotient<INT>(a, b)), real(2) * f);
   }
-  return dg_div(a + b, real(2) * F);
+  return quotient<INT>(a + b, real(2) * F);
 }
 
 // Chandrashekar's entropy-conservative two-point flux in the direction Jm (the
 // averaged metric row, or the face normal), from the two sides' rho, velocity,
 // beta = rho/(2p) and |u|^2:  f_rho = rho_ln {u}.Jm, f_m = f_rho {u} + ({rho}/(2{beta})) Jm,
 // f_E = f_rho (1/(2(gamma-1) beta_ln) - {|u|^2}/2) + {u}.f_m
-template <typename real>
+template <bool INT = true, typename real>
 __device__ __forceinline__ void ec_flux(real ra, const real ua[3], real ba, real qa, real rb, const real ub[3],
                                         real bb, real qb, const real Jm[3], const Phys<real>& ph, real f[NV]) {
   const real um[3] = {real(0.5) * (ua[0] + ub[0]), real(0.5) * (ua[1] + ub[1]), real(0.5) * (ua[2] + ub[2])};
-  const real frho = log_mean(ra, rb) * (um[0] * Jm[0] + um[1] * Jm[1] + um[2] * Jm[2]);
-  const real ptil = dg_div(real(0.5) * (ra + rb), ba + bb);
+  const real frho = log_mean<INT>(ra, rb) * (um[0] * Jm[0] + um[1] * Jm[1] + um[2] * Jm[2]);
+  const real ptil = quotient<INT>(real(0.5) * (ra + rb), ba + bb);
   f[0] = frho;
   f[1] = frho * um[0] + ptil * Jm[0];
   f[2] = frho * um[1] + ptil * Jm[1];
   f[3] = frho * um[2] + ptil * Jm[2];
-  f[4] = frho * (dg_div(real(0.5) * ph.inv_gm1, log_mean(ba, bb)) - real(0.25) * (qa + qb)) + um[0] * f[1] + um[1] * f[2] +
+  f[4] = frho * (quotient<INT>(real(0.5) * ph.inv_gm1, log_mean<INT>(ba, bb)) - real(0.25) * (qa + qb)) + um[0] * f[1] + um[1] * f[2] +
          um[2] * f[3];
 }
 

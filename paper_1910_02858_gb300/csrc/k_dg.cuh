@@ -426,6 +426,10 @@ __device__ __forceinline__ void lift_vol_body(
   static_assert(sizeof(real) == 4 || SPLIT == 2 || BR2, "the other FP64 forms are k_lift_fx.cuh's");
   static_assert(!BR2 || (SW == 0 && !SPLIT), "BR2 face gradients are built for the standard form, CUDA-core sweeps");
 
+  // divisions of the entropy-conservative pairs: in integers but for n = 3, whose CTAs of 81 threads
+  // leave the FP64 pipe room (10^3, 16^3, 24^3 elements, integers against FP64: 138, 335, 1060
+  // against 108, 326, 985 us; n = 2, 32^3: 609 against 629, n = 4, 10^3: 204 against 250)
+  constexpr bool kInt = n != 3;
   const int tid = threadIdx.x;
   const int el = tid / n3, node = tid - el * n3;
   const int e0 = (ORD ? order[blockIdx.x] : blockIdx.x) * NE;
@@ -748,7 +752,7 @@ __device__ __forceinline__ void lift_vol_body(
             const real Jm[3] = {real(0.5) * (J0 + f[(6 + 3 * l) * n3p]), real(0.5) * (J1 + f[(7 + 3 * l) * n3p]),
                                 real(0.5) * (J2 + f[(8 + 3 * l) * n3p])};
             real F[NV];
-            ec_flux(W[0], ua, dg_div(real(0.5) * W[0], W[4]), H, f[0], ub, f[4 * n3p], f[5 * n3p], Jm, ph, F);
+            ec_flux<kInt>(W[0], ua, dg_div(real(0.5) * W[0], W[4]), H, f[0], ub, f[4 * n3p], f[5 * n3p], Jm, ph, F);
 #pragma unroll
             for (int v = 0; v < NV; ++v) sm[v] += real(2) * d * F[v];
           } else {
@@ -803,7 +807,7 @@ __device__ __forceinline__ void lift_vol_body(
             const real dd = real(2) * sD[ii * n + ii];
             const real u3[3] = {ui, vi, wi}, J3[3] = {ji0, ji1, ji2};
             real F[NV];
-            ec_flux(ri, u3, pi, Hi, ri, u3, pi, Hi, J3, ph, F);
+            ec_flux<kInt>(ri, u3, pi, Hi, ri, u3, pi, Hi, J3, ph, F);
 #pragma unroll
             for (int c = 0; c < NV; ++c) ai[c] = dd * F[c];
           }
@@ -815,7 +819,7 @@ __device__ __forceinline__ void lift_vol_body(
             const real Jm[3] = {real(0.5) * (ji0 + fa[jo]), real(0.5) * (ji1 + fa[jo + n3p]),
                                 real(0.5) * (ji2 + fa[jo + 2 * n3p])};
             real F[NV];
-            ec_flux(ri, u3, pi, Hi, fa[0], ua3, fa[4 * n3p], fa[5 * n3p], Jm, ph, F);
+            ec_flux<kInt>(ri, u3, pi, Hi, fa[0], ua3, fa[4 * n3p], fa[5 * n3p], Jm, ph, F);
             F0 = real(2) * F[0]; F1 = real(2) * F[1]; F2 = real(2) * F[2]; F3 = real(2) * F[3]; F4 = real(2) * F[4];
             const real dia = sD[aa * n + ii], dai = sD[ii * n + aa];
             ai[0] += dia * F0; ai[1] += dia * F1; ai[2] += dia * F2; ai[3] += dia * F3; ai[4] += dia * F4;
