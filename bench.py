@@ -48,9 +48,10 @@ def peaks():
 # DRAM bytes (read + write) per launch of the lifting/volume kernel (affine elements) from the ncu captures
 # summarised in profiles/, keyed by form and by a hash of the kernel sources at
 # capture time; reported only while the sources are unchanged (else null).
-KERNEL_SOURCES = ["paper_1910_02858_gb300/csrc/k_dg.cuh", "paper_1910_02858_gb300/csrc/dg_common.cuh",
-                  "paper_1910_02858_gb300/csrc/k_tc.cuh", "paper_1910_02858_gb300/csrc/k_adj.cuh"]
-NCU_TRAFFIC = {("fp64", "6ae1340b23330a2c"): 386398208, ("fp32", "6ae1340b23330a2c"): 154639104}
+KERNEL_SOURCES = ["paper_1910_02858_gb300/csrc/" + f for f in (
+    "k_dg.cuh", "dg_common.cuh", "k_tc.cuh", "k_adj.cuh", "fx.cuh", "fp64_math.cuh", "k_lift_fx.cuh", "k_lift_f32_affine.cuh",
+    "k_surf_fx.cuh", "k_adj_fx.cuh", "k_mortar.cuh", "k_reduce.cuh", "launch.h")]
+NCU_TRAFFIC = {("fp64", "5ad4761ee8a5f95e"): 386398208, ("fp32", "5ad4761ee8a5f95e"): 154639104}
 
 
 def kernel_source_hash(texts=None) -> str:
@@ -75,6 +76,8 @@ def kernel_source_hash(texts=None) -> str:
 # GB300 FP64 FMA peak derived from unit counts and clocks: 152 SMs x 2 DFMA/clk
 # (4 FP64 flop/clk/SM, consistent with the nominal 1.25 TFLOP/s) x 2070 MHz.
 FP64_PEAK_TFLOPS = 152 * 4 * 2.070e9 / 1e12
+# metric words per DOF that the lifting kernels of affine elements do not read (Ja, 1/J)
+AFFINE_WORDS = 10
 # FP32 FMA peak from the same unit counts: 128 FP32 lanes x 2 flop/clk per SM
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 
@@ -167,7 +170,8 @@ def dist_env():
 
 def algorithmic_per_dof(n: int, word: int):
     """Per DOF and RK stage: minimum-traffic bytes of the three-kernel schedule and
-    the flops of the dominant kernel (lifting + volume integral), FMA = 2 flops."""
+    the flops of the dominant kernel (lifting + volume integral), FMA = 2 flops.
+    Curved elements; affine ones read AFFINE_WORDS fewer words in the lifting."""
     f = 3.0 / n
     bytes_stage = (46.0 + 117.0 * f) * word
     bytes_liftvol = (20.0 + 48.0 * f) * word
@@ -420,11 +424,12 @@ def main():
     ms_step = ms_total / args.steps
     pid = whole_job_pid(ms_total * 1e-3, args.steps, dof, world)
 
-    # roofline of the dominant kernel (lifting + volume) against HBM; instruction issue is what
-    # holds it (profiles/)
+    # roofline of the dominant kernel (lifting + volume) against HBM, which is not what holds it
+    # (profiles/)
     n = N + 1
     word = 8 if args.form == "fp64" else 4
     bytes_stage, bytes_lv, flops_lv = algorithmic_per_dof(n, word)
+    bytes_stage, bytes_lv = bytes_stage - AFFINE_WORDS * word, bytes_lv - AFFINE_WORDS * word  # all elements are affine
     lv_ms, lv_cnt = ktimes["lift_vol"]
     lv_avg_s = lv_ms / max(lv_cnt, 1) * 1e-3
     share = lv_ms / max(sum(v[0] for v in ktimes.values()), 1e-9)
@@ -433,7 +438,6 @@ def main():
     achieved = bytes_lv * dof / lv_avg_s / 1e9
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                 "traffic": traffic,
-                # the workload's elements are affine
                 "kernel": "k_lift_vol_fx_affine<8>" if args.form == "fp64" else f"k_lift_vol_f32_affine<8,{args.form}>",
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)" if peaks() else "fallback 6.8 TB/s",
                 "kernel_share": share}
@@ -526,7 +530,7 @@ def extras(args, s64, U0, mesh, dt, dev, F, wl, Solver, SolverConfig, torch, np)
             s.run(U, nsteps, dt)
             dof = s.query(F.Q_DOF)
             n = 8
-            bytes_stage = (46.0 + 117.0 * 3.0 / n) * 4 * dof
+            bytes_stage = (46.0 - AFFINE_WORDS + 117.0 * 3.0 / n) * 4 * dof
             lv = kt["lift_vol"][0] / max(kt["lift_vol"][1], 1)
             pid32 = ms * 1e6 / (nsteps * NSTAGES * dof)
             floor = step_floor_ns(s, dof, False, F)
@@ -534,7 +538,7 @@ def extras(args, s64, U0, mesh, dt, dev, F, wl, Solver, SolverConfig, torch, np)
                          "rel_l2_err_vs_fp64": rel_err_per_var(U, U64),
                          "step_algorithmic_hbm_gbs": bytes_stage * NSTAGES * nsteps / (ms * 1e-3) / 1e9,
                          "lift_vol_ms_per_launch": lv,
-                         "lift_vol_hbm_gbs": (20.0 + 48.0 * 3.0 / n) * 4 * dof / (lv * 1e-3) / 1e9}
+                         "lift_vol_hbm_gbs": (20.0 - AFFINE_WORDS + 48.0 * 3.0 / n) * 4 * dof / (lv * 1e-3) / 1e9}
         except Exception as exc:
             out[name] = {"error": str(exc)}
         finally:

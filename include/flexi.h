@@ -120,6 +120,12 @@ typedef struct {
  *           exact state by default).
  * Computes on the device: x at the solution nodes, curl-form metrics Ja, 1/J,
  * face normals and surface elements; allocates every buffer later calls use.
+ * Elements that are parallelepipeds to within the rounding of their coordinates
+ * take constant Ja and 1/J from their edge vectors where the lifting kernels have
+ * a form for them (BR1; not the EC split form, the KEP form in FP32, nor FP64
+ * meshes of fewer elements than the GPU has multiprocessors at N <= 3).  Contexts
+ * of one mesh with different options may therefore differ in the last bits of the
+ * metric terms and of the quadrature weights (the totals of flexi_reduce).
  * Returns FLEXI_EMESH for asymmetric connectivity or J <= 0, FLEXI_EINVAL for
  * bad sizes or parameters, FLEXI_EUNSUPPORTED for the split form with Gauss
  * nodes or a tensor-core form.  On success *out owns everything; free it with
@@ -239,7 +245,8 @@ flexi_status flexi_reduce_noalloc(flexi_ctx *ctx, const void *U, const void *Ut,
 
 enum {
   FLEXI_Q_K = 0, FLEXI_Q_N = 1, FLEXI_Q_NSIDES = 2, FLEXI_Q_NBCSIDES = 3, FLEXI_Q_DOF = 4,
-  FLEXI_Q_BYTES_PER_STAGE = 5, /* algorithmic HBM bytes of one RK stage (minimum-traffic schedule) */
+  FLEXI_Q_BYTES_PER_STAGE = 5, /* algorithmic HBM bytes of one RK stage (minimum-traffic schedule; elements
+                                  that go through the affine kernels: without metric terms per node) */
   FLEXI_Q_FLOPS_PER_STAGE = 6, /* algorithmic floating-point operations of one RK stage */
   FLEXI_Q_STATUS = 7,          /* synchronises and returns (then clears) the device status word */
   FLEXI_Q_DEVICE_BYTES = 8,    /* device memory held by the context */

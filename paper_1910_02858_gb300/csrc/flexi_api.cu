@@ -1115,8 +1115,11 @@ flexi_status flexi_query(flexi_ctx* c, int what, int64_t* val) {
     case FLEXI_Q_NBCSIDES: *val = c->nBC; return FLEXI_OK;
     case FLEXI_Q_DOF: *val = (int64_t)dof; return FLEXI_OK;
     case FLEXI_Q_BYTES_PER_STAGE: {
-      // minimum-traffic three-kernel schedule, words per DOF: 46 + 117 f
-      *val = (int64_t)((46.0 + 117.0 * f) * dof * c->rs);
+      // minimum-traffic three-kernel schedule, words per DOF: 46 + 117 f; the affine kernels read 10
+      // metric words per element, not per node
+      const double ne = c->n3 >= 64 ? 1 : (64 + c->n3 - 1) / c->n3;
+      const double affine = std::min((double)c->K, c->m.nAffine * ne);
+      *val = (int64_t)(((46.0 + 117.0 * f) * dof - 10.0 * affine * (c->n3 - 1)) * c->rs);
       return FLEXI_OK;
     }
     case FLEXI_Q_FLOPS_PER_STAGE: {

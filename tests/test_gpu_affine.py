@@ -49,3 +49,23 @@ def test_parallelepipeds_far_away_still_count():
     s.close()
     # sums of n + 2 terms up to rowsum(|Dhat| + |lhat|) 2 / h = 60 times the flux (3 at most), each rounded to 2^-53
     assert Ut.abs().max().item() <= 3 * 10 * 2.0 ** -53 * 3 * 60
+
+
+@pytest.mark.parametrize("N", [1, 4])
+def test_algorithmic_bytes_count_what_affine_elements_read(N):
+    """46 + 117 (3 / n) words per DOF and stage; affine elements read ten metric words per element, not per node."""
+    from paper_1910_02858_gb300 import Solver, SolverConfig
+    from paper_1910_02858_gb300 import flexi as F
+
+    n, shape = N + 1, (11, 12, 10)
+    words = {}
+    for mapping in ("cartesian", "bent"):
+        mesh = wl.box_mesh(shape, lo=(0.0,) * 3, hi=(6.0, 6.0, 6.0), Ngeo=1)
+        if mapping == "bent":
+            mesh.coords[:, 0, 0, 0] += 1e-3  # no element keeps its parallel edges
+        s = Solver(SolverConfig(N=N, mu=0.01), mesh.coords, mesh.conn)
+        words[mapping] = s.query(F.Q_BYTES_PER_STAGE) / 8
+        s.close()
+    K = np.prod(shape)
+    assert words["cartesian"] == (46 + 351 / n) * K * n ** 3 - 10 * K * (n ** 3 - 1)
+    assert words["bent"] == (46 + 351 / n) * K * n ** 3
