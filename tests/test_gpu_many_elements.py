@@ -111,3 +111,31 @@ def test_step_is_its_stages(N, nodes):
     scale = U.abs().amax(dim=(0, 2, 3, 4))
     bound = 5 * (4 * 2.0 ** -53 * 2 * scale.cpu().numpy() + dt * tol)
     assert ((V - U).abs().amax(dim=(0, 2, 3, 4)).cpu().numpy() <= bound).all()
+
+
+@pytest.mark.parametrize("mapping", ["cartesian", "sine"])
+@pytest.mark.parametrize("N", [2, 3, 4, 5, 6, 7])
+def test_surface_kernel_matches_its_fp64_branch(N, mapping):
+    """The surface kernel takes its FP64 expressions from 2^900 on, which finite data reach with a gas at rest (no
+    product of two such values): dm/dt = -grad p scales with p exactly.  Gauss-Lobatto nodes: no jumps, so no
+    dissipation.  Bound: that of the volume sums, twice, for the surface's products under the same row sums."""
+    import torch
+
+    from paper_1910_02858_gb300 import Solver, SolverConfig
+    from paper_1910_02858_gb300 import flexi as F
+
+    mesh, _, tol = _case(N, 1, mapping, SHAPE.get(N, (6, 6, 5)))
+    x = mesh.node_coords(N, 1)
+    U = np.zeros((x.shape[0], 5) + x.shape[2:])
+    U[:, 0] = 1.0
+    U[:, 4] = (1.0 + 0.1 * np.sin(x[:, 0]) * np.cos(x[:, 1] + x[:, 2])) / 0.4
+    out = []
+    for f in (1.0, 2.0 ** 910):
+        s = Solver(SolverConfig(N=N, Ngeo=mesh.Ngeo, node_type=1, riemann=F.RIEMANN_RUSANOV, mu=0.0), mesh.coords, mesh.conn)
+        V = U.copy()
+        V[:, 4] *= f
+        out.append(s.rhs(torch.tensor(V, device="cuda:0"), 0.0).cpu().numpy() / f)
+        s.close()
+    for v in (1, 2, 3):
+        assert np.abs(out[0][:, v]).max() > 1e-3
+        assert np.abs(out[0][:, v] - out[1][:, v]).max() <= 2 * tol[v], v
