@@ -686,11 +686,11 @@ flexi_status mesh_init_impl(flexi_ctx* c, const flexi_params* p, int K, const do
         }
         if (pass == 0) c->m.nAffine = (int)order.size();
       }
-      // A mixed mesh takes two launches, one after the other, of which the affine one saves a quarter
-      // to a half of its time and the other ends in a wave of its own: worth it from about four
-      // waves of affine CTAs (1024 threads per SM) on.  10^3 elements, N = 1, FP32, some of them
-      // affine: 23 us in two launches, 14 us in one.
-      if (c->m.nAffine < groups && (int64_t)c->m.nAffine * ne * n3 < (int64_t)4 * 1024 * nsm) c->m.nAffine = 0;
+      // A mixed mesh takes two launches, one after the other, each with a tail of its own: worth it from
+      // one and a half waves of affine CTAs (1024 threads per SM) on.  Steps in one launch against two,
+      // a tenth of the elements bent: FP64, N = 7: 0.71 of the time at 0.45 waves, 0.90 at 1.35, 1.10 at
+      // 1.8; N = 4: 0.93, 1.06, 1.09; FP32, N = 5: 0.86, 1.05, 1.05; N = 1, 10^3: 14 us against 23.
+      if (c->m.nAffine < groups && (int64_t)c->m.nAffine * ne * n3 < (int64_t)1536 * nsm) c->m.nAffine = 0;
       if (c->m.nAffine > 0 && c->m.nAffine < groups) {
         int* dorder;
         AL(dorder, order.size());
