@@ -5,7 +5,7 @@
 // prolongation's and the metric terms' transposes; at 64 clocks each they set its time.  Those sums
 // run on the integer pipes here, the pointwise flux derivatives stay in FP64.  Affine
 // elements fold the metric constants in before the lifting's transpose (15 line contractions
-// instead of 45).  8^3 elements, N = 5: 215 -> 80 us; curved 7 x 9 x 8, N = 6: 349 -> 181 us.
+// instead of 45).  8^3 elements, N = 5: 215 -> 80 us; curved 7 x 9 x 8, N = 6: 349 -> 144 us.
 #pragma once
 #include "fx.cuh"
 
@@ -36,7 +36,7 @@ constexpr size_t adj_fx_smem() {
 
 // affine: the metric terms are aff[e][10]; else Ja, fgeo.  n = 7: two CTAs of 343 threads at 80
 // registers (160 B spilled) against one at 168: reverse of one right-hand side, 16^3 curved
-// elements, 2539 -> 2209 us
+// elements, 2539 -> 2209 us (2200 with scales by direction)
 template <int n, bool AFF>
 __global__ void __launch_bounds__(Cfg<n>::T, n == 8 ? 1 : (n == 7 ? 2 : (n == 6 ? 3 : 4))) k_adj_vol_fx(
     const double* __restrict__ U, const double* __restrict__ Ja, const double* __restrict__ aff,

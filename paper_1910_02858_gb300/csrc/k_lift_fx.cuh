@@ -7,8 +7,10 @@
 // and run here on the integer pipes; the FP64 pipe keeps the primitive variables, the
 // surface means and the pointwise fluxes.  Elements whose values leave the fixed-point
 // range (above 2^200, infinities, NaN) take the FP64 schedule of lift_vol_fp64.  16^3 elements,
-// N = 7: 3061 -> 751 us (curved), 566 us (affine; 77 FP64 and 3,760 integer instructions per
-// node, bound by their issue); 638 MB are 95 us at the measured copy rate.
+// N = 7: 3061 -> 750 us (curved), 559 us (affine; 77 FP64 and 3,775 integer instructions per
+// node); 638 MB (470 affine) are 95 (70) us at the measured copy rate.  No pipe is the bound on its
+// own: FP64, ALU and FMA-heavy pipe and the issue slots are each busy 43 to 47 % of the time, as
+// the phases that use the one or the others follow each other with barriers between.
 #pragma once
 #include "fx.cuh"
 
@@ -176,7 +178,7 @@ constexpr size_t lift_fx_smem() {
 }
 
 // CTAs per SM asked of the register allocator (n = 8: two of 512 threads at 64 registers;
-// n = 7: three of 343 at 56 against two at 80, 16^3: 657 -> 601 us, affine 453 -> 398 us; the
+// n = 7: three of 343 at 56 against two at 80, 16^3: 657 -> 601 us, affine 453 -> 398 (now 608, 388); the
 // pairs of the split form want the registers: 14^3 curved, N = 6, 647 -> 627 us with two, 18^3
 // curved, N = 4, 367 -> 343 us with six of 125 threads instead of seven)
 template <int n, bool KEP>
@@ -297,7 +299,8 @@ __device__ __forceinline__ bool volume_fx(const double* __restrict__ U, double* 
 // direction, the velocity and Ja each under a power of two of their own.  Their products meet
 // at the largest of them: the mass flux at 2^bC, the largest of |u_d| |Ja_d|, momentum d at the
 // larger of mass flux times u_d and p Ja_d (shifts sc, sm, sp of the smaller operands).
-// 990 elements, N = 7: 1130 -> 232 us with the lifting.
+// 990 elements, N = 7: 1130 -> 240 us with the lifting (232 with one scale for all directions and
+// for all rows of D, at up to 190 times the rounding noise of FP64 sums).
 template <int n, bool AFF, int JS, typename Metric>
 __device__ __forceinline__ bool split_volume_fx(const double* __restrict__ U, double* __restrict__ Utv, const double (&W)[NV],
                                                 const double (&G)[15], int K, int grp, unsigned wmask, fx64* sA, int* sMag,
@@ -693,7 +696,7 @@ __global__ void __launch_bounds__(Cfg<n>::T, lift_fx_min_blocks<n, KEP>()) k_lif
 // constants of the element, so the lifting contracts the 5 primitive variables along the 3
 // directions (15 line fields instead of 45) and combines the results with J^l_d / J, the face
 // terms of a line are the face means themselves (n_d s_hat = +-Ja^l_d on both ends), and no
-// metric term is read per node.  16^3 elements, N = 7: 751 -> 566 us.
+// metric term is read per node.  16^3 elements, N = 7: 750 -> 559 us.
 // ---------------------------------------------------------------------------
 template <int n>
 constexpr size_t lift_affine_smem() {
